@@ -87,10 +87,11 @@ typedef struct {
 } vie_grid_desc;
 
 /* How the inner block solves of the preconditioner run (vie_grid_desc.flags).
- * AUTO: a persistent kernel in which each CTA solves whole blocks on its own,
- * for every group whose padded (x, y) plane fits in shared memory, when those
- * groups hold at least 32 blocks together; batched multi-CTA launches per
- * BiCGSTAB step otherwise. The two
+ * AUTO: a persistent kernel in which a thread-block cluster solves whole blocks
+ * on its own, for every group whose boxes are at most 16 voxels per axis
+ * (parity-split MVM, on chip) and for every group whose padded (x, y) plane fits
+ * in shared memory when the persistent groups hold at least 32 blocks together;
+ * batched multi-CTA launches per BiCGSTAB step otherwise. The two
  * paths compute the same iterations; the flags force one of them. */
 enum vie_grid_flags {
     VIE_GRID_INNER_AUTO = 0,
@@ -103,11 +104,12 @@ typedef struct {
     int32_t ngroups;         /* batches of blocks sharing one padded FFT shape     */
     int32_t Mx, My, Mz;      /* padded FFT shape of the full-grid operator         */
     int64_t device_bytes;    /* device memory held by the grid handle              */
-    int32_t inner_cluster[2];/* CTAs per block chosen by the block solver's tuner for
-                                complex128 [0] and complex64 [1]: 1, 2 or 4 for
-                                every block, -1 for the split launch of the
-                                register MVM (the slowest blocks on 4 CTAs and the
-                                rest on 2); 0 = not yet tuned                      */
+    int32_t inner_cluster[2];/* CTAs per block of the persistent block solver for
+                                complex128 [0] and complex64 [1]: 4 for boxes of at
+                                most 16 voxels per axis; for larger ones chosen by the
+                                tuner: 2 or 4 for every block, -1 for the split launch
+                                (the slowest blocks on 4 CTAs and the rest on 2);
+                                0 = not yet used or tuned                           */
 } vie_grid_info;
 
 /* Creates the grid on the current CUDA device: uploads chi = eps_r - 1,
@@ -262,14 +264,14 @@ int vie_solve_host(vie_grid* grid, const vie_spectrum* spectrum, const void* ein
  * application; their blocks then run in ONE persistent launch (one per
  * precision, inner tolerance and inner limit), the longest-running blocks
  * first. Merged are the blocks that the persistent block solver takes for
- * their grid alone (VIE_GRID_AUTO: grids with 32 or more fitting blocks) and
- * the complex64 blocks of its on-chip slab MVM (every padded axis in [8, 32]);
- * the other blocks run in their grid's batched launches meanwhile. A solve joins at its first application
+ * their grid alone when that grid has 32 or more fitting blocks, and the complex64
+ * blocks of at most 16 voxels per axis; the other blocks run in their grid's own
+ * launches meanwhile. A solve joins at its first application
  * and leaves when it stops applying the preconditioner, so requests that arrive
  * while others run share launches from then on (continuous batching). Each
  * solve runs exactly the iteration of vie_solve; its result equals the
- * vie_solve result up to rounding (the merged launches use clusters of 2 CTAs
- * per block, while vie_solve tunes the cluster size per grid). */
+ * vie_solve result up to rounding (the order of sums in a launch follows its shape,
+ * which depends on the number of blocks in it). */
 typedef struct vie_merge_session vie_merge_session;
 
 typedef struct {

@@ -439,6 +439,18 @@ extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
         }
         gr.bs.nb = (int)mem.size();
         set_shape(gr.bs, mx, my, mz);
+        if (par_path_ok(gr.bs)) {
+            // classes of equal transform lengths of the blocks' own extents
+            std::map<std::tuple<int, int, int>, ParClass> cls;
+            for (int j = 0; j < gr.bs.nb; ++j) {
+                const int* ext = &sext[3 * mem[j]];
+                ParClass& c = cls[std::make_tuple(par_len(ext[2]), par_len(ext[1]), par_len(ext[0]))];
+                c.hx = par_len(ext[0]); c.hy = par_len(ext[1]); c.hz = par_len(ext[2]);
+                c.ex = std::max(c.ex, ext[0]); c.ey = std::max(c.ey, ext[1]); c.ez = std::max(c.ez, ext[2]);
+                c.boxes.push_back(j);
+            }
+            for (auto& c : cls) gr.par.push_back(c.second);
+        }
         gr.bs.block_ids = mem;
         const int64_t box = gr.bs.box_elems();
         std::vector<double2> gchi(gr.bs.nb * box, make_double2(0, 0));
@@ -489,19 +501,26 @@ extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
             if (inner_persistent_ok(gr.bs, es, true)) fit_blocks += gr.bs.nb;
         const bool force = d->flags == VIE_GRID_INNER_PERSISTENT || fit_blocks >= kInnerMinBlocks;
         for (auto& gr : g->groups) {
-            // merged launches across grids take the blocks the persistent solver would take here, and
-            // complex64 blocks of the on-chip slab MVM (a few such blocks of one grid iterate faster in
-            // the batched launches, which spread each block over the whole GPU, but many of them, from
-            // several grids, fill the GPU in one launch; larger boxes stay batched)
+            // merged launches across grids take the blocks of grids with kInnerMinBlocks fitting blocks or
+            // more, and complex64 blocks of the parity-split MVM (larger boxes stay batched)
             gr.fit[prec] = d->flags != VIE_GRID_INNER_BATCHED && inner_persistent_ok(gr.bs, es, true) &&
-                           (force || (prec == 1 && slab_path_ok(gr.bs, es) && !slab_disabled()));
+                           (force || (prec == 1 && !gr.par.empty()));
             gr.last_iters[prec].assign(gr.bs.nb, 0.f);
             bool ok = d->flags != VIE_GRID_INNER_BATCHED && inner_persistent_ok(gr.bs, es, force);
             (prec == 0 ? gr.persistent128 : gr.persistent64) = ok;
             if (!ok) continue;
-            for (int b = 0; b < gr.bs.nb; ++b) items.push_back({gr.bs.spec_elems(), make_int2(job, b)});
-            g->job_group[prec].push_back((int)(&gr - g->groups.data()));
-            ++job;
+            // one job per class of the parity-split MVM, else one for the group
+            const int gidx = (int)(&gr - g->groups.data());
+            for (const ParClass& c : gr.par) {
+                for (int b : c.boxes) items.push_back({(int64_t)c.hx * c.hy * c.hz * 8, make_int2(job, b)});
+                g->job_group[prec].push_back(gidx);
+                ++job;
+            }
+            if (gr.par.empty()) {
+                for (int b = 0; b < gr.bs.nb; ++b) items.push_back({gr.bs.spec_elems(), make_int2(job, b)});
+                g->job_group[prec].push_back(gidx);
+                ++job;
+            }
         }
         std::stable_sort(items.begin(), items.end(),
                          [](const std::pair<int64_t, int2>& a, const std::pair<int64_t, int2>& b) { return a.first > b.first; });
@@ -518,7 +537,8 @@ extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
     }
     if (!g->groups.empty()) {
         char* descs = nullptr;
-        if ((rc = dalloc(g, &descs, (int64_t)(g->groups.size() * inner_group_desc_bytes())))) return bail(rc);
+        const size_t njobs = std::max<size_t>(1, std::max(g->job_group[0].size(), g->job_group[1].size()));
+        if ((rc = dalloc(g, &descs, (int64_t)(njobs * inner_group_desc_bytes())))) return bail(rc);
         g->inner_groups = descs;
         if ((rc = dalloc(g, &g->inner_next, 2))) return bail(rc);
     }
@@ -592,6 +612,35 @@ extern "C" int vie_green_spectrum_near(vie_grid* g, double k0, int mask, int32_t
     return green_spectrum(g, k0, mask, near, (cudaStream_t)stream, out);
 }
 
+static void free_par(vie_spectrum* sp) {
+    for (auto& v : sp->par)
+        for (ParSpec& p : v) {
+            dfree(p.g128);
+            dfree(p.g64);
+        }
+}
+
+// Spectra of the parity-split MVM for one group: the lengths of its box (they hold every block, so the
+// spectrum serves any grid of the same shape signature), then those of its smaller classes.
+static int par_spectra(const Group& gr, const double2* K, int mask, std::vector<ParSpec>& out, cudaStream_t s) {
+    if (gr.par.empty()) return VIE_OK;
+    auto add = [&](int hx, int hy, int hz) -> int {
+        for (const ParSpec& p : out)
+            if (p.hx == hx && p.hy == hy && p.hz == hz) return VIE_OK;
+        ParSpec p;
+        p.hx = hx; p.hy = hy; p.hz = hz;
+        out.push_back(p);
+        const int64_t n = par_spectrum_elems(hx, hy, hz);
+        ParSpec& q = out.back();
+        if (mask & VIE_C128) VIE_TRY(dmalloc((void**)&q.g128, n * sizeof(double2), "vie_green_spectrum"));
+        if (mask & VIE_C64) VIE_TRY(dmalloc((void**)&q.g64, n * sizeof(float2), "vie_green_spectrum"));
+        return par_spectrum(gr.bs, K, hx, hy, hz, q.g128, q.g64, s);
+    };
+    VIE_TRY(add(par_len(gr.bs.bx), par_len(gr.bs.by), par_len(gr.bs.bz)));
+    for (const ParClass& c : gr.par) VIE_TRY(add(c.hx, c.hy, c.hz));
+    return VIE_OK;
+}
+
 static int green_spectrum(vie_grid* g, double k0, int mask, const NearRule& near, cudaStream_t stream,
                           vie_spectrum** out) {
     if (!g || !out) return fail(VIE_EINVAL, "vie_green_spectrum: null argument");
@@ -609,7 +658,7 @@ static int green_spectrum(vie_grid* g, double k0, int mask, const NearRule& near
         cudaStreamSynchronize(s);         // kernels already queued may still use the spectra
         for (auto p : sp->g128) dfree(p);
         for (auto p : sp->g64) dfree(p);
-        for (auto p : sp->go64) dfree(p);
+        free_par(sp);
         delete sp;
         return rc;
     };
@@ -630,7 +679,6 @@ static int green_spectrum(vie_grid* g, double k0, int mask, const NearRule& near
         }
         sp->g128.push_back(G);
         sp->g64.push_back(G64);
-        sp->go64.push_back(nullptr);
         int rc = spectrum_build(g->full, k0, g->h, G, G64, nullptr, s, &near);
         if (rc) return bail(rc);
     }
@@ -642,6 +690,8 @@ static int green_spectrum(vie_grid* g, double k0, int mask, const NearRule& near
         if (arc) return bail(arc);
         sp->g128.push_back(G);
         int rc = green_sample(*bs, k0, g->h, G, s, &near);
+        sp->par.emplace_back();
+        if (!rc) rc = par_spectra(g->groups[sp->par.size() - 1], G, mask, sp->par.back(), s);
         if (!rc) rc = spectrum_fft<double2>(*bs, G, s);
         if (rc) return bail(rc);
         float2* G64 = nullptr;
@@ -653,16 +703,6 @@ static int green_spectrum(vie_grid* g, double k0, int mask, const NearRule& near
             }
         }
         sp->g64.push_back(G64);
-        // the slab MVM of the block solver reads an octant of the spectrum in natural order
-        float2* Go = nullptr;
-        if ((mask & VIE_C64) && slab_path_ok(*bs, sizeof(float2))) {
-            if ((arc = dmalloc((void**)&Go, 6 * bs->oct_elems() * sizeof(float2), "vie_green_spectrum")))
-                return bail(arc);
-            sp->go64.push_back(Go);
-            if ((rc = slab_spectrum(*bs, G, Go, s))) return bail(rc);
-        } else {
-            sp->go64.push_back(nullptr);
-        }
     }
     if (!(mask & VIE_C128)) {
         // the FP64 spectrum was only the source of the complex64 copy
@@ -681,7 +721,7 @@ extern "C" int vie_spectrum_release(vie_spectrum* sp) {
     cudaDeviceSynchronize();
     for (auto p : sp->g128) dfree(p);
     for (auto p : sp->g64) dfree(p);
-    for (auto p : sp->go64) dfree(p);
+    free_par(sp);
     delete sp;
     return VIE_OK;
 }
@@ -877,6 +917,41 @@ void merge_leave(MergeMember* mm) {
     if (!mc->pending.empty() && (int)mc->pending.size() >= mc->live) merge_flush(mc);
 }
 
+template <class C> static const C* par_of(const ParSpec& p);
+template <> const double2* par_of<double2>(const ParSpec& p) { return p.g128; }
+template <> const float2* par_of<float2>(const ParSpec& p) { return p.g64; }
+
+// The persistent solver's jobs of one group: one per class of the parity-split MVM (with the class's
+// lengths when the spectrum has them, else those of the group's box), or one for the whole group.
+template <class C>
+static void group_jobs(vie_grid* g, const vie_spectrum* sp, int i, std::vector<InnerJob<C>>& jobs) {
+    Group& gr = g->groups[i];
+    InnerJob<C> j;
+    j.bs = &gr.bs;
+    j.v = group_vecs<C>(gr);
+    j.chi = chi_of<C>(gr.bs);
+    j.G = spec_of<C>(sp, 1 + i);
+    j.st = gr.st;
+    if (gr.par.empty()) jobs.push_back(j);
+    for (const ParClass& c : gr.par) {
+        const ParSpec* p = &sp->par[i][0];
+        for (const ParSpec& q : sp->par[i])
+            if (q.hx == c.hx && q.hy == c.hy && q.hz == c.hz) p = &q;
+        j.hx = p->hx; j.hy = p->hy; j.hz = p->hz;
+        // with lengths larger than the class's own, the extents widen to the least those lengths serve
+        j.ex = std::max(c.ex, par_least(j.hx)); j.ey = std::max(c.ey, par_least(j.hy)); j.ez = std::max(c.ez, par_least(j.hz));
+        j.Gq = par_of<C>(*p);
+        jobs.push_back(j);
+    }
+}
+
+// Padded points of a block's MVM, the weight of its iterations in the work order.
+static double block_weight(const Group& gr, int box) {
+    for (const ParClass& c : gr.par)
+        if (std::binary_search(c.boxes.begin(), c.boxes.end(), box)) return 8.0 * c.hx * c.hy * c.hz;
+    return (double)gr.bs.spec_elems();
+}
+
 // The grid's jobs and work items for a merged launch: every group that fits, each block costed by
 // its iterations in its last application x its padded box.
 template <class C>
@@ -888,17 +963,17 @@ static void grid_merge_jobs(vie_grid* g, const vie_spectrum* sp, MergeReq* r) {
     for (size_t i = 0; i < g->groups.size(); ++i) {
         Group& gr = g->groups[i];
         if (!gr.fit[pi]) continue;
-        InnerJob<C> j;
-        j.bs = &gr.bs;
-        j.v = group_vecs<C>(gr);
-        j.chi = chi_of<C>(gr.bs);
-        j.G = spec_of<C>(sp, 1 + (int)i);
-        j.st = gr.st;
-        if (pi == 1 && !slab_disabled()) j.Go = reinterpret_cast<const C*>(sp->go64[1 + i]);
-        const int job = (int)jobs.size();
-        jobs.push_back(j);
-        for (int b = 0; b < gr.bs.nb; ++b)
-            r->items.push_back({(gr.last_iters[pi][b] + 1.0) * (double)gr.bs.spec_elems(), make_int2(job, b)});
+        int job = (int)jobs.size();
+        group_jobs<C>(g, sp, (int)i, jobs);
+        auto add = [&](int b) {
+            r->items.push_back({(gr.last_iters[pi][b] + 1.0) * block_weight(gr, b), make_int2(job, b)});
+        };
+        for (const ParClass& c : gr.par) {
+            for (int b : c.boxes) add(b);
+            ++job;
+        }
+        if (gr.par.empty())
+            for (int b = 0; b < gr.bs.nb; ++b) add(b);
     }
 }
 
@@ -921,22 +996,10 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
         Group& gr = g->groups[i];
         KrylovVecs<C>& v = group_vecs<C>(gr);
         VIE_TRY(precond_gather<C>(g, gr, b, v.b, s));
-        if (merged) {
-            // blocks that fit the persistent solver go to the merged launch, the rest run here
-            if (gr.fit[c128 ? 0 : 1]) any_fit = true;
-            else batched.push_back(i);
-        } else if (c128 ? gr.persistent128 : gr.persistent64) {
-            InnerJob<C> j;
-            j.bs = &gr.bs;
-            j.v = v;
-            j.chi = chi_of<C>(gr.bs);
-            j.G = spec_of<C>(sp, 1 + i);
-            j.st = gr.st;
-            if (!c128 && !slab_disabled()) j.Go = reinterpret_cast<const C*>(sp->go64[1 + i]);
-            jobs.push_back(j);
-        } else {
-            batched.push_back(i);
-        }
+        // in a session, blocks that fit go to the merged launch; the rest run as they would alone
+        if (merged && gr.fit[c128 ? 0 : 1]) any_fit = true;
+        else if (c128 ? gr.persistent128 : gr.persistent64) group_jobs<C>(g, sp, i, jobs);
+        else batched.push_back(i);
     }
     // after arriving, the request is waited for on every path out of this function
     if (merged && !any_fit) merge_leave(mm);   // nothing of this grid fits: do not hold the others
@@ -960,39 +1023,26 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
         merge_arrive(mm, &req);
         guard.armed = true;
     }
-    bool slab = false;
-    for (const InnerJob<C>& j : jobs) slab = slab || j.Go != nullptr;
-    // launch shape and MVM variant, tuned on the first applies, then the best. Register-FFT MVM: 2 and
-    // 4 CTAs per block, then the split launch (the slowest blocks of the previous apply on 4 CTAs, the
-    // rest on 2). Blocks the slab MVM takes (whole MVM on chip, the cluster splits the kz planes): 2, 1
-    // and 4 CTAs with 4 planes per round where they fit, 2 CTAs with 2 planes per round (a split cannot
-    // shorten the slowest block's solve, which bounds the apply once every block fits on the device at
-    // once), and the register-FFT MVM with 2 CTAs instead of the slab MVM.
-    // candidates (CTAs per block, kz planes per round of the slab MVM's plane stage with 0 = as many as
-    // fit, slab MVM or register MVM)
-    struct Cand {
-        int cluster, npl;
-        bool slab;
-    };
-    static const Cand kCand[3] = {{2, 0, false}, {4, 0, false}, {-1, 0, false}};
-    static const Cand kCandSlab[5] = {{2, 4, true}, {1, 4, true}, {4, 4, true}, {2, 2, true}, {2, 0, false}};
-    const int ncand = slab ? 5 : 3;
+    // Launch shape: the parity-split MVM runs on clusters of 4 CTAs. Without such jobs it is tuned on the
+    // first applies: 2 and 4 CTAs per block, then the split launch (the slowest blocks of the previous
+    // apply on 4 CTAs, the rest on 2), then the best.
+    bool par = false;
+    for (const InnerJob<C>& j : jobs) par = par || j.hx > 0;
+    static const int kCand[3] = {2, 4, -1};
+    const int ncand = 3;
     const int pi = c128 ? 0 : 1;
+    if (par) g->tune_best[pi] = 4;
     // the first apply only warms up (first launches of the kernel pay one-time costs that would bias
     // the candidate tried first); the candidates follow, one per apply
     const int tried = g->tune_count[pi] - 1;
-    const bool tuning = !jobs.empty() && tried < ncand && !inner_cluster_forced();
-    const Cand cand = tuning ? (slab ? kCandSlab : kCand)[std::max(tried, 0)]
-                             : Cand{g->tune_best[pi] ? g->tune_best[pi] : 2, g->tune_npl[pi], !g->tune_noslab[pi]};
-    const int choice = cand.cluster;
-    if (slab && !cand.slab)
-        for (InnerJob<C>& j : jobs) j.Go = nullptr;   // the register-FFT MVM for these blocks
+    const bool tuning = !jobs.empty() && !par && tried < ncand && !inner_cluster_forced();
+    const int choice = tuning ? kCand[std::max(tried, 0)] : (g->tune_best[pi] ? g->tune_best[pi] : 2);
     // with batched groups as well, the persistent launch runs on the grid's second stream beside
     // the batched steps (no split launch then)
     const bool beside = !jobs.empty() && !batched.empty();
     InnerSplit split;
     split.nheavy = choice == -1 && !beside ? g->nheavy[pi] : 0;
-    split.cluster = slab ? 2 : 4;
+    split.cluster = 4;
     split.s2 = g->s2;
     split.fork = g->fork_ev;
     split.join = g->join_ev;
@@ -1005,7 +1055,7 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
     if (tuning) VIE_CK(cudaEventRecord(g->tev[0], sp_stream));
     VIE_TRY(inner_persistent<C>(jobs, c128 ? g->work128 : g->work64, c128 ? g->nwork128 : g->nwork64,
                                 g->inner_groups, g->inner_next, tol, maxit, sp_stream,
-                                choice == -1 ? (slab ? 1 : 2) : choice, &split, cand.npl));
+                                choice == -1 ? 2 : choice, &split));
     if (tuning) VIE_CK(cudaEventRecord(g->tev[1], sp_stream));
     std::vector<Bicg<C>> bk(ng);
     for (int i : batched) {
@@ -1089,7 +1139,7 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
             items.reserve(wh.size());
             for (const int2& w : wh) {
                 const Group& gr = g->groups[jg[w.x]];
-                items.push_back({(hs[jg[w.x]][w.y].iters + 1.0) * (double)gr.bs.spec_elems(), w});
+                items.push_back({(hs[jg[w.x]][w.y].iters + 1.0) * block_weight(gr, w.y), w});
             }
             std::stable_sort(items.begin(), items.end(), [](const std::pair<double, int2>& a,
                                                             const std::pair<double, int2>& b) { return a.first > b.first; });
@@ -1126,9 +1176,7 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
             int best = 0;
             for (int k = 1; k < ncand; ++k)
                 if (g->tune_score[pi][k] < g->tune_score[pi][best]) best = k;
-            g->tune_best[pi] = (slab ? kCandSlab : kCand)[best].cluster;
-            g->tune_npl[pi] = (slab ? kCandSlab : kCand)[best].npl;
-            g->tune_noslab[pi] = slab && !kCandSlab[best].slab;
+            g->tune_best[pi] = kCand[best];
         }
     }
     return VIE_OK;

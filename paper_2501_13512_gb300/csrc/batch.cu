@@ -279,7 +279,9 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
     // complex128: octant layout (batched MVMs); complex64: full layout when the persistent
     // block solver reads it, else octant layout
     const int64_t so = 6 * bs.oct_elems();
-    const int64_t s64 = b->persistent ? 6 * bs.spec_elems() : so;
+    const int hx = par_len(bs.bx), hy = par_len(bs.by), hz = par_len(bs.bz);
+    const bool par = b->persistent && par_path_ok(bs);       // parity-split MVM: its own spectrum layout
+    const int64_t s64 = par ? par_spectrum_elems(hx, hy, hz) : b->persistent ? 6 * bs.spec_elems() : so;
     for (int i = 0; i < nb; ++i) {
         auto it = b->spectra.find(k0s[i]);
         if (it == b->spectra.end()) {
@@ -294,7 +296,7 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
             BoxSet one = bs;
             one.nb = 1;
             int rc = spectrum_build(one, k0s[i], b->h, G, b->persistent ? nullptr : G64,
-                                    b->persistent ? G64 : nullptr, s);
+                                    b->persistent && !par ? G64 : nullptr, s, nullptr, par ? G64 : nullptr);
             if (rc) {
                 cudaStreamSynchronize(s);
                 dfree(G);
@@ -384,6 +386,10 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
             jobs[0].v = b->k64;
             jobs[0].chi = bs.chi64;
             jobs[0].G = gb64[0];
+            if (par) {
+                jobs[0].hx = hx; jobs[0].hy = hy; jobs[0].hz = hz;
+                jobs[0].ex = bs.bx; jobs[0].ey = bs.by; jobs[0].ez = bs.bz;
+            }
             jobs[0].st = b->st;
             jobs[0].Gb = b->d_gb64;
             jobs[0].tols = b->d_tols;

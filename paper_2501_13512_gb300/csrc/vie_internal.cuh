@@ -171,7 +171,22 @@ struct ReduceScratch {
 };
 constexpr int kMaxCtaPerSeg = 256;
 
+// Blocks of a group whose own extents take the same transform lengths of the parity-split MVM
+// (inner_parity.cuh): one job of the persistent solver.
+struct ParClass {
+    int hx = 0, hy = 0, hz = 0;        // transform lengths (par_len of the extents)
+    int ex = 0, ey = 0, ez = 0;        // largest extents of its blocks
+    std::vector<int> boxes;            // indices within the group
+};
+// Spectrum of one set of transform lengths (par_spectrum).
+struct ParSpec {
+    int hx = 0, hy = 0, hz = 0;
+    double2* g128 = nullptr;
+    float2* g64 = nullptr;
+};
+
 struct Group {
+    std::vector<ParClass> par;         // empty: the boxes are too large for the parity-split MVM
     bool persistent128 = false;        // solved by the persistent block solver
     bool persistent64 = false;
     bool fit[2] = {false, false};      // may join a merged persistent launch (0: complex128, 1: complex64)
@@ -197,8 +212,9 @@ struct vie_spectrum {
     // frequency positions per axis), scaled by 1/(Mx My Mz).
     std::vector<double2*> g128;
     std::vector<float2*> g64;
-    // index 1 + g: complex64 octant spectrum of group g in natural order for the slab MVM, or null
-    std::vector<float2*> go64;
+    // index g: spectra of group g for the parity-split MVM: the lengths of the group's box first (they
+    // serve every block of the group), then those of its smaller classes
+    std::vector<std::vector<vie::ParSpec>> par;
 };
 
 struct vie_grid {
@@ -241,9 +257,7 @@ struct vie_grid {
     // applies 0 and 1 try the candidates, later applies use the best
     int tune_count[2] = {0, 0};
     int tune_best[2] = {0, 0};
-    int tune_npl[2] = {0, 0};             // slab MVM: kz planes per round of the best candidate (0: auto)
-    bool tune_noslab[2] = {false, false}; // the best candidate ran the register-FFT MVM instead of the slab MVM
-    double tune_score[2][5] = {{0, 0, 0, 0, 0}, {0, 0, 0, 0, 0}};
+    double tune_score[2][3] = {{0, 0, 0}, {0, 0, 0}};
     int nheavy[2] = {0, 0};               // blocks of the split launch's heavy part (from the last apply)
     cudaEvent_t tev[2] = {nullptr, nullptr};
     int64_t device_bytes = 0;
@@ -292,8 +306,9 @@ struct NearRule {
     double t[kNearMaxOrder], w[kNearMaxOrder];   // nodes and weights on [-1, 1]
 };
 int near_rule(int radius, int q, NearRule* out);   // VIE_EINVAL outside radius [0, 8], q [1, 16]
+// or par64 (parity-split layout of the lengths holding the box, par_spectrum).
 int spectrum_build(const BoxSet& bs, double k0, double h, double2* oct128, float2* oct64, float2* full64,
-                   cudaStream_t s, const NearRule* near = nullptr);
+                   cudaStream_t s, const NearRule* near = nullptr, float2* par64 = nullptr);
 
 // ---------------------------------------------------------------- green.cu
 int green_sample(const BoxSet& bs, double k0, double h, double2* G, cudaStream_t s, const NearRule* near = nullptr);
@@ -343,18 +358,23 @@ template <class C> struct InnerJob {
     SegState* st;
     const C* const* Gb = nullptr;   // optional device array: one spectrum per box
     const double* tols = nullptr;   // optional device array: one relative tolerance per box
-    const C* Go = nullptr;          // optional octant spectrum in natural order (slab MVM, complex64)
+    // parity-split MVM (hx > 0): transform lengths, extents and the spectrum (null with Gb)
+    int hx = 0, hy = 0, hz = 0, ex = 0, ey = 0, ez = 0;
+    const C* Gq = nullptr;
 };
 bool inner_persistent_ok(const BoxSet& bs, size_t es, bool force);
-bool slab_path_ok(const BoxSet& bs, size_t es);
-// Octant spectrum of the slab MVM from a full FP64 spectrum [6][Mz][My][Mx] (bit-reversed positions):
-// Go[kz][c][ky][kx] = G[c][brev(kz)][brev(ky)][brev(kx)] for k in [0, M/2] per axis, as complex64.
-int slab_spectrum(const BoxSet& bs, const double2* G, float2* Go, cudaStream_t s);
+// Parity-split MVM (inner_parity.cuh): smallest transform length holding b voxels (0: none), whether a
+// box set takes it, and its spectra from the lattice samples K of green_sample.
+int par_len(int b);
+int par_least(int h);                   // smallest extent that takes length h
+bool par_path_ok(const BoxSet& bs);
+int64_t par_spectrum_elems(int hx, int hy, int hz);
+int par_spectrum(const BoxSet& bs, const double2* K, int hx, int hy, int hz, double2* g128, float2* g64, cudaStream_t s);
 size_t inner_group_desc_bytes();
-// cluster: CTAs per block (1, 2, 4, 8; 0 = 2), unless VIE_INNER_CLUSTER forces one. npl: kz planes
-// per round of the slab MVM's plane stage (2 or 4; 0: 4 where it fits), unless VIE_SLAB_NPL forces one.
-// Split launch (split != null, 0 < split->nheavy < nwork): the first nheavy work items run
-// with split->cluster CTAs per block on s while the rest run with `cluster` CTAs per block on
+// cluster: CTAs per block (1, 2, 4, 8; 0 = 2) of launches without parity-split jobs (those take 4),
+// unless VIE_INNER_CLUSTER forces one.
+// Split launch (split != null, 0 < split->nheavy < nwork, no parity-split jobs): the first nheavy work
+// items run with split->cluster CTAs per block on s while the rest run with `cluster` CTAs per block on
 // split->s2, concurrently; d_next must hold two counters; s waits for both.
 struct InnerSplit {
     int nheavy = 0;
@@ -365,7 +385,7 @@ struct InnerSplit {
 template <class C>
 int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, int nwork, void* d_groups,
                      int* d_next, double tol, int maxit, cudaStream_t s, int cluster = 0,
-                     const InnerSplit* split = nullptr, int npl = 0);
+                     const InnerSplit* split = nullptr);
 int inner_cluster_forced();
 
 // ---------------------------------------------------------------- merge sessions (api.cu)
@@ -425,9 +445,6 @@ void merge_join(MergeMember* mm);
 void merge_arrive(MergeMember* mm, MergeReq* r);
 int merge_wait(MergeMember* mm, MergeReq* r, cudaStream_t s);
 void merge_leave(MergeMember* mm);
-// True when the environment variable VIE_INNER_SLAB is 0: complex64 blocks keep the register-FFT MVM
-// instead of the slab MVM (read once).
-bool slab_disabled();
 template <class C> inline const C* tw_of(const Twiddles& t);
 template <> inline const double2* tw_of<double2>(const Twiddles& t) { return t.d128; }
 template <> inline const float2* tw_of<float2>(const Twiddles& t) { return t.d64; }
