@@ -337,8 +337,8 @@ int vie_batch_destroy(vie_batch* batch);
  * the batch). Mixed precision only (opts->mode = VIE_MODE_MIXED): FP64 true
  * residuals of all instances from one batched complex128 MVM, then one
  * complex64 correction solve for every instance still above outer_tol, all in
- * one persistent launch (one CTA cluster per instance) when the padded plane
- * fits in shared memory, else batched launches per BiCGSTAB step; E += d.
+ * one persistent launch (one CTA cluster per instance) for grids of at most 16
+ * voxels per axis, else batched launches per BiCGSTAB step; E += d.
  * outer_maxit bounds each correction; inner_tol, inner_maxit and use_precond
  * are ignored (no blocks). An instance whose correction does not lower its
  * FP64 residual gets that correction undone and stops (VIE_ENOTCONV). einc_dev, e_dev: DEVICE complex128
@@ -430,7 +430,9 @@ int vie_far_field_rcs(const vie_grid* grid, double k0, const void* e_dev,
                       vie_stream_t stream);
 
 /* Device bytes held by the batch (with its cached spectra), and whether its
- * corrections run in the persistent kernel (1) or in batched launches (0). */
+ * instances fit the persistent kernel (1) or not (0). Those that fit run in it in
+ * merged launches (vie_batch_solve_many); alone, those of at most 16 voxels per
+ * axis do and larger ones use batched launches, as the instances that do not fit. */
 int vie_batch_get_info(const vie_batch* batch, int64_t* device_bytes, int32_t* persistent);
 
 /* Kernel-level profile, aggregated per kernel kind and precision. */

@@ -35,6 +35,7 @@ struct vie_batch {
     double* d_tols = nullptr;             // [count] correction tolerances (0: instance done)
     double2** d_gb128 = nullptr;          // [count] spectrum per instance
     float2** d_gb64 = nullptr;
+    float2** d_gb64full = nullptr;        // boxes over 16 voxels: full layout for the persistent solver
     int2* work = nullptr;                 // persistent work list (0, b)
     void* inner_groups = nullptr;
     int* inner_next = nullptr;
@@ -42,7 +43,12 @@ struct vie_batch {
     double* h_scal = nullptr;             // pinned [2 count]
     cudaEvent_t ev = nullptr;
     cudaEvent_t ev_ready = nullptr;       // gathers queued before a merged launch
-    std::map<double, std::pair<double2*, float2*>> spectra;   // cached per wavenumber
+    struct Spec {
+        double2* g128 = nullptr;          // octant
+        float2* g64 = nullptr;            // parity-split layout (boxes up to 16 voxels) or octant
+        float2* full64 = nullptr;         // full layout, boxes over 16 voxels that fit the persistent solver
+    };
+    std::map<double, Spec> spectra;       // cached per wavenumber
     std::vector<void*> allocations;
     int64_t device_bytes = 0;
 };
@@ -62,8 +68,9 @@ int balloc(vie_batch* b, T** p, int64_t count) {
 
 void release(vie_batch* b) {
     for (auto& kv : b->spectra) {
-        dfree(kv.second.first);
-        dfree(kv.second.second);
+        dfree(kv.second.g128);
+        dfree(kv.second.g64);
+        dfree(kv.second.full64);
     }
     for (void* p : b->allocations) dfree(p);
     if (b->h_scal) cudaFreeHost(b->h_scal);
@@ -197,7 +204,7 @@ extern "C" int vie_batch_create(const vie_batch_desc* d, vie_batch** out) {
         (rc = balloc(b, &b->tmp128, nv)) || (rc = balloc(b, &b->xprev, nv)) || (rc = balloc(b, &b->st, d->count)) ||
         (rc = balloc(b, &b->d_bn2, d->count)) || (rc = balloc(b, &b->d_rn2, d->count)) ||
         (rc = balloc(b, &b->d_tols, d->count)) || (rc = balloc(b, &b->d_gb128, d->count)) ||
-        (rc = balloc(b, &b->d_gb64, d->count)))
+        (rc = balloc(b, &b->d_gb64, d->count)) || (rc = balloc(b, &b->d_gb64full, d->count)))
         return bail(rc);
     k.y = k.p;
     k.z = k.s;
@@ -275,40 +282,42 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
     BoxSet& bs = b->bs;
     // spectra per distinct wavenumber (cached), one pointer per instance
     std::vector<double2*> gb128(nb);
-    std::vector<float2*> gb64(nb);
-    // complex128: octant layout (batched MVMs); complex64: full layout when the persistent
-    // block solver reads it, else octant layout
+    std::vector<float2*> gb64(nb), gb64full(nb);
+    // complex128: octant layout (batched MVMs); complex64: the layout of the parity-split MVM for boxes it
+    // takes, else octant for the batched launches and full for the persistent solver
     const int64_t so = 6 * bs.oct_elems();
     const int hx = par_len(bs.bx), hy = par_len(bs.by), hz = par_len(bs.bz);
-    const bool par = b->persistent && par_path_ok(bs);       // parity-split MVM: its own spectrum layout
-    const int64_t s64 = par ? par_spectrum_elems(hx, hy, hz) : b->persistent ? 6 * bs.spec_elems() : so;
+    const bool par = b->persistent && par_path_ok(bs);
     for (int i = 0; i < nb; ++i) {
         auto it = b->spectra.find(k0s[i]);
         if (it == b->spectra.end()) {
-            double2* G = nullptr;
-            float2* G64 = nullptr;
-            int arc = dmalloc((void**)&G, so * sizeof(double2), "vie_batch_solve");
-            if (!arc) arc = dmalloc((void**)&G64, s64 * sizeof(float2), "vie_batch_solve");
+            vie_batch::Spec g;
+            const int64_t n64 = par ? par_spectrum_elems(hx, hy, hz) : so;
+            int arc = dmalloc((void**)&g.g128, so * sizeof(double2), "vie_batch_solve");
+            if (!arc) arc = dmalloc((void**)&g.g64, n64 * sizeof(float2), "vie_batch_solve");
+            if (!arc && b->persistent && !par)
+                arc = dmalloc((void**)&g.full64, 6 * bs.spec_elems() * sizeof(float2), "vie_batch_solve");
+            if (!arc) {
+                BoxSet one = bs;
+                one.nb = 1;
+                arc = spectrum_build(one, k0s[i], b->h, g.g128, par ? nullptr : g.g64, g.full64, s, nullptr,
+                                     par ? g.g64 : nullptr);
+                if (arc) cudaStreamSynchronize(s);
+            }
             if (arc) {
-                dfree(G);
+                dfree(g.g128);
+                dfree(g.g64);
+                dfree(g.full64);
                 return arc;
             }
-            BoxSet one = bs;
-            one.nb = 1;
-            int rc = spectrum_build(one, k0s[i], b->h, G, b->persistent ? nullptr : G64,
-                                    b->persistent && !par ? G64 : nullptr, s, nullptr, par ? G64 : nullptr);
-            if (rc) {
-                cudaStreamSynchronize(s);
-                dfree(G);
-                dfree(G64);
-                return rc;
-            }
-            it = b->spectra.emplace(k0s[i], std::make_pair(G, G64)).first;
+            it = b->spectra.emplace(k0s[i], g).first;
         }
-        gb128[i] = it->second.first;
-        gb64[i] = it->second.second;
+        gb128[i] = it->second.g128;
+        gb64[i] = it->second.g64;
+        gb64full[i] = it->second.full64;
     }
     VIE_CK(cudaMemcpyAsync(b->d_gb128, gb128.data(), nb * sizeof(double2*), cudaMemcpyHostToDevice, s));
+    VIE_CK(cudaMemcpyAsync(b->d_gb64full, gb64full.data(), nb * sizeof(float2*), cudaMemcpyHostToDevice, s));
     VIE_CK(cudaMemcpyAsync(b->d_gb64, gb64.data(), nb * sizeof(float2*), cudaMemcpyHostToDevice, s));
     const double2* einc = (const double2*)einc_dev;
     double2* x = (double2*)e_dev;
@@ -380,20 +389,24 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
         VIE_CK(cudaMemcpyAsync(b->d_tols, tols.data(), nb * sizeof(double), cudaMemcpyHostToDevice, s));
         k_seg_scale<<<grid1(nv), 256, 0, s>>>(b->r128, b->d_rn2, b->d_tols, b->k64.b, b->n3, nb);
         VIE_CK(cudaGetLastError());
-        if (b->persistent) {
+        const bool merging = mm != nullptr && mm->live;
+        // Instances of more than 16 voxels per axis take the persistent solver in merged launches only: alone,
+        // the batched launches spread a step over the whole GPU (24^3: 354 us a step for 8 instances and
+        // 1490 us for 63, against 2300 and 3650 us with one cluster of two CTAs per instance).
+        if (b->persistent && (par || merging)) {
             std::vector<InnerJob<float2>> jobs(1);
             jobs[0].bs = &bs;
             jobs[0].v = b->k64;
             jobs[0].chi = bs.chi64;
-            jobs[0].G = gb64[0];
+            jobs[0].G = par ? gb64[0] : gb64full[0];
             if (par) {
                 jobs[0].hx = hx; jobs[0].hy = hy; jobs[0].hz = hz;
                 jobs[0].ex = bs.bx; jobs[0].ey = bs.by; jobs[0].ez = bs.bz;
             }
             jobs[0].st = b->st;
-            jobs[0].Gb = b->d_gb64;
+            jobs[0].Gb = par ? b->d_gb64 : b->d_gb64full;
             jobs[0].tols = b->d_tols;
-            if (mm != nullptr && mm->live) {
+            if (merging) {
                 // the corrections of every batch of the session that reached this step, in one launch
                 MergeReq req;
                 req.prec = 1;
