@@ -15,7 +15,7 @@ ROOT = os.path.dirname(HERE)
 SOURCES = ["fft.cu", "krylov.cu", "fields.cu", "api.cu", "profile.cu", "inner.cu", "noalloc.cu", "batch.cu",
            "farfield.cu", "rooftop.cu"]
 HEADERS = [os.path.join(CSRC, "vie_internal.cuh"), os.path.join(CSRC, "fft_core.cuh"), os.path.join(CSRC, "fft_reg.cuh"),
-           os.path.join(CSRC, "dft_small.cuh"), os.path.join(CSRC, "inner_parity.cuh"),
+           os.path.join(CSRC, "dft_small.cuh"), os.path.join(CSRC, "fft_plane.cuh"), os.path.join(CSRC, "inner_parity.cuh"),
            os.path.join(ROOT, "include", "vie.h")]
 LIB = os.path.join(HERE, "libvie.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -1,4 +1,4 @@
-// Register-resident DFTs of the lengths 2, 4, 6, 8, 10, 12 and 16, natural order in and out, fully
+// Register-resident DFTs of the lengths 1, 2, 4, 6, 8, 10, 12 and 16, natural order in and out, fully
 // unrolled. 6, 10 and 12 split into coprime factors by the prime-factor map (Good 1958, Thomas 1963:
 // no twiddles between the factors); 8 and 16 by one Cooley-Tukey step. Operation counts per complex
 // transform: 6: 36 additions + 8 products, 8: 52 + 4, 10: 88 + 24, 12: 96 + 16, 16: 144 + 24.
@@ -10,8 +10,6 @@ namespace vie {
 
 #define VIE_HD __host__ __device__ __forceinline__
 
-// Real addition and subtraction of the transforms. FP64 sums go through the fused multiply-add with an
-// exact factor of one when the caller passes one that the compiler cannot see through (ADD_ONE).
 template <class C> VIE_HD C cscale(C a, typename real_of<C>::type s) { return mk(a.x * s, a.y * s); }
 // a * (-i) forward, a * i inverse
 template <bool FWD, class C> VIE_HD C rot(C a) { return FWD ? mul_mi(a) : mul_i(a); }
@@ -58,7 +56,8 @@ template <bool FWD, class C> VIE_HD void dft5(C& a, C& b, C& c, C& d, C& e) {
 
 template <int H, bool FWD, class C> VIE_HD void dft(C (&a)[H]) {
     typedef typename real_of<C>::type R;
-    if constexpr (H == 2) {
+    if constexpr (H == 1) {
+    } else if constexpr (H == 2) {
         dft2<FWD>(a[0], a[1]);
     } else if constexpr (H == 4) {
         dft4<FWD>(a[0], a[1], a[2], a[3]);
@@ -124,6 +123,36 @@ template <int H, bool FWD, class C> VIE_HD void dft(C (&a)[H]) {
                 a[4 * k2 + k1] = t;
             }
     }
+}
+
+// s += a b, s -= a b, as four fused multiply-adds (the product's own sum first would take six operations)
+template <class C> VIE_HD void cmac(C& s, C a, C b) {
+    s.x = fma(-a.y, b.y, fma(a.x, b.x, s.x));
+    s.y = fma(a.y, b.x, fma(a.x, b.y, s.y));
+}
+template <class C> VIE_HD void cmacn(C& s, C a, C b) {
+    s.x = fma(a.y, b.y, fma(-a.x, b.x, s.x));
+    s.y = fma(-a.y, b.x, fma(-a.x, b.y, s.y));
+}
+
+// The symmetric 3x3 Green multiply of one frequency with the entries v (xx, xy, xz, yy, yz, zz), the
+// frequency being in the upper half of the axis AXIS (0: x, 2: z; the two off-diagonal components odd along
+// that axis change sign) when FLIP is set.
+template <int AXIS, bool FLIP, class C> VIE_HD void green3(C& X, C& Y, C& Z, const C (&v)[6]) {
+    C ox = cmul(v[0], X), oy = cmul(v[3], Y), oz = cmul(v[5], Z);
+    auto mac = [](bool neg, C& s, C a, C b) {
+        if (neg) cmacn(s, a, b);
+        else cmac(s, a, b);
+    };
+    mac(FLIP && AXIS == 0, ox, v[1], Y);
+    mac(FLIP && AXIS == 0, oy, v[1], X);
+    mac(FLIP, ox, v[2], Z);
+    mac(FLIP, oz, v[2], X);
+    mac(FLIP && AXIS == 2, oy, v[4], Z);
+    mac(FLIP && AXIS == 2, oz, v[4], Y);
+    X = ox;
+    Y = oy;
+    Z = oz;
 }
 
 }  // namespace vie

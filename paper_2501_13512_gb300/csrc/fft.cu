@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "dft_small.cuh"
 #include "fft_core.cuh"
 #include "fft_reg.cuh"
 #include "vie_internal.cuh"
@@ -217,9 +218,11 @@ __global__ void __launch_bounds__(kThreads) k_zgreen(ZArgs<C> a) {
         if (uy != uz) gyz = mk(-gyz.x, -gyz.y);
         C* p = buf + i * pitch + c;
         C X = p[0], Y = p[TC], Z = p[2 * TC];
-        p[0] = cmul(gxx, X) + cmul(gxy, Y) + cmul(gxz, Z);
-        p[TC] = cmul(gxy, X) + cmul(gyy, Y) + cmul(gyz, Z);
-        p[2 * TC] = cmul(gxz, X) + cmul(gyz, Y) + cmul(gzz, Z);
+        const C e[6] = {gxx, gxy, gxz, gyy, gyz, gzz};
+        green3<2, false>(X, Y, Z, e);
+        p[0] = X;
+        p[TC] = Y;
+        p[2 * TC] = Z;
     }
     __syncthreads();
     smem_fft<C, false, 3>(buf, a.lL, pitch, a.ltc, a.tw, a.twshift);
@@ -290,29 +293,37 @@ __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
         const int im = LGZ ? (int)(__brev((unsigned)fm) >> (32 - LGZ)) : 0;
         if (im < i) continue;
         const int col = c0 + c;
-        bool ux, uy, uz;
-        const int qx = octant_slot(col & ((1 << a.lx) - 1), a.lx, ux);
-        const int qy = octant_slot(col >> a.lx, a.ly, uy);
-        const int qz = octant_slot(i, LGZ, uz);
-        const F* gp = G + ((int64_t)qz * hy + qy) * hx + qx;
+        bool ux = false, uy = false, uz = false;
+        const F* gp;
+        if (a.oct) {
+            const int qx = octant_slot(col & ((1 << a.lx) - 1), a.lx, ux);
+            const int qy = octant_slot(col >> a.lx, a.ly, uy);
+            const int qz = octant_slot(i, LGZ, uz);
+            gp = G + ((int64_t)qz * hy + qy) * hx + qx;
+        } else {
+            gp = G + (int64_t)i * P + col;
+        }
         const F gxx = gp[0], gyy = gp[3 * a.gcomp], gzz = gp[5 * a.gcomp];
         F gxy = gp[a.gcomp], gxz = gp[2 * a.gcomp], gyz = gp[4 * a.gcomp];
         if (ux != uy) gxy = mk(-gxy.x, -gxy.y);
         if (ux != uz) gxz = mk(-gxz.x, -gxz.y);
         if (uy != uz) gyz = mk(-gyz.x, -gyz.y);
+        const F e[6] = {gxx, gxy, gxz, gyy, gyz, gzz};
         {
             F* q = sm + i * NC + c;
-            const F X = q[0], Y = q[cst], Z = q[2 * cst];
-            q[0] = cmul(gxx, X) + cmul(gxy, Y) + cmul(gxz, Z);
-            q[cst] = cmul(gxy, X) + cmul(gyy, Y) + cmul(gyz, Z);
-            q[2 * cst] = cmul(gxz, X) + cmul(gyz, Y) + cmul(gzz, Z);
+            F X = q[0], Y = q[cst], Z = q[2 * cst];
+            green3<2, false>(X, Y, Z, e);
+            q[0] = X;
+            q[cst] = Y;
+            q[2 * cst] = Z;
         }
         if (im != i) {   // frequency -f: xz and yz change sign
             F* q = sm + im * NC + c;
-            const F X = q[0], Y = q[cst], Z = q[2 * cst];
-            q[0] = cmul(gxx, X) + cmul(gxy, Y) - cmul(gxz, Z);
-            q[cst] = cmul(gxy, X) + cmul(gyy, Y) - cmul(gyz, Z);
-            q[2 * cst] = cmul(gzz, Z) - cmul(gxz, X) - cmul(gyz, Y);
+            F X = q[0], Y = q[cst], Z = q[2 * cst];
+            green3<2, true>(X, Y, Z, e);
+            q[0] = X;
+            q[cst] = Y;
+            q[2 * cst] = Z;
         }
     }
     __syncthreads();
@@ -338,6 +349,239 @@ __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
         }
     }
 }
+
+// Where a column's spectrum entries lie: octant (OCT) or full layout (bit-reversed positions). entry(f) is
+// the offset of component xx at the z frequency f in [0, M/2]; the six components are gcomp apart. sxy, sx,
+// sy: whether xy, xz and yz change sign with the column's x and y frequencies (octant).
+template <class C, bool OCT> struct ZColumn {
+    const C* g;
+    int64_t row;
+    bool sxy, sx, sy;
+    __device__ __forceinline__ ZColumn(const ZArgs<C>& a, int b, int col) {
+        g = a.Gb ? a.Gb[b] : a.G;
+        sxy = sx = sy = false;
+        if (OCT) {
+            const int hx = (1 << a.lx) / 2 + 1, hy = (1 << a.ly) / 2 + 1;
+            bool ux, uy;
+            const int qx = octant_slot(col & ((1 << a.lx) - 1), a.lx, ux), qy = octant_slot(col >> a.lx, a.ly, uy);
+            g += (int64_t)qy * hx + qx;
+            row = (int64_t)hy * hx;
+            sx = ux;
+            sy = uy;
+            sxy = ux != uy;
+        } else {
+            g += col;
+            row = a.axis;
+        }
+    }
+    // the six components at slot q of the z axis (octant_slot / bit-reversed position of the frequency)
+    __device__ __forceinline__ void load(C (&v)[6], int q, int64_t gcomp) const {
+        const C* p = g + q * row;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) v[c] = __ldg(p + c * gcomp);
+        if (OCT) {
+            v[1] = cneg_if(v[1], sxy);
+            v[2] = cneg_if(v[2], sx);
+            v[4] = cneg_if(v[4], sy);
+        }
+    }
+};
+
+// exp(-2 pi i m / 1024) at a compile-time m, times or conjugated times v.
+template <bool FWD> __device__ __forceinline__ float2 ztw(float2 v, int m, const float2*) { return twc<FWD>(v, m); }
+template <bool FWD> __device__ __forceinline__ double2 ztw(double2 v, int m, const double2* tw) { return twmul<FWD>(v, m, tw); }
+
+// Slot of the z frequency f in [0, M/2], M = 1 << l, of a compile-time f.
+template <bool OCT> __device__ __forceinline__ int zslot(int f, int l) {
+    const int H = (1 << l) >> 1;
+    if (!OCT) return (int)bit_reverse((unsigned)f, l);
+    return f == H ? H : (l >= 2 ? (int)bit_reverse((unsigned)f, l - 1) : 0);
+}
+
+// Pass Z of complex128 MVMs with Mz = 2H <= 32. The zero-padded 2H-point transform of a column of at most H planes is two H-point
+// transforms, of the column (even frequencies) and of the column times W_2H^j (odd ones). One thread takes one
+// parity of one column, all three components in registers: transform, Green multiply (one load of the six
+// entries serves the frequencies k and -k), inverse transform; the odd parity's thread hands its result over
+// through shared memory. Two parities per column, kZPairCols columns per CTA.
+// (Bound by the FP64 units: no operation is spent on the padding; 256x256x16 2320 -> 1730 us. In complex64 the pencils of k_zgreen_reg
+// are faster, 81 against 109 us at 256x256x16: three columns of 16 values do not fit the registers of a
+// thread at a useful occupancy.)
+constexpr int kZPairCols = 64;
+
+template <class C, int H, bool OCT, int PAR>
+__device__ __forceinline__ void z_parity(const ZArgs<C>& a, const ZColumn<C, OCT>& zc, const C* W, C (&v)[3][H]) {
+    constexpr int LG = ILog2<2 * H>::v, TS = kLmax / (2 * H);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int j = 0; j < H; ++j) v[c][j] = j < a.nzb ? W[c * a.comp_stride + j * a.axis] : czero<C>();
+        if (PAR) {
+#pragma unroll
+            for (int j = 1; j < H; ++j) v[c][j] = ztw<true>(v[c][j], j * TS, a.tw);
+        }
+        dft<H, true>(v[c]);
+    }
+    // frequencies k = 2m + PAR and their mirrors
+#pragma unroll
+    for (int m = 0; m < (PAR ? H / 2 : H / 2 + 1); ++m) {
+        C e[6];
+        zc.load(e, zslot<OCT>(2 * m + PAR, LG), a.gcomp);
+        const int mm = (H - m - PAR) % H;
+        green3<2, false>(v[0][m], v[1][m], v[2][m], e);
+        if (mm != m) green3<2, true>(v[0][mm], v[1][mm], v[2][mm], e);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        dft<H, false>(v[c]);
+        if (PAR) {
+#pragma unroll
+            for (int j = 1; j < H; ++j) v[c][j] = ztw<false>(v[c][j], j * TS, a.tw);
+        }
+    }
+}
+
+template <class C, int H, bool OCT>
+__global__ void __launch_bounds__(2 * kZPairCols, 2) k_z_pair(ZArgs<C> a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* sm = reinterpret_cast<C*>(smem_raw);      // [3 H][kZPairCols]: the odd parity's results
+    const int b = blockIdx.y;
+    if (!box_active(a.st, b)) return;
+    if (a.units != nullptr && threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(a.units, 1);
+    const int c = threadIdx.x % kZPairCols, odd = threadIdx.x / kZPairCols;   // whole warps per parity
+    const int col = blockIdx.x * kZPairCols + c;
+    const bool live = col < a.ncols;
+    C* W = a.w + (int64_t)b * a.box_stride + col;
+    const ZColumn<C, OCT> zc(a, b, live ? col : 0);
+    C v[3][H];
+    if (odd && live) {
+        z_parity<C, H, OCT, 1>(a, zc, W, v);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < H; ++j) sm[(i * H + j) * kZPairCols + c] = v[i][j];
+    } else if (live) {
+        z_parity<C, H, OCT, 0>(a, zc, W, v);
+    }
+    __syncthreads();
+    if (odd || !live) return;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < H; ++j)
+            if (j < a.nzb) W[i * a.comp_stride + j * a.axis] = v[i][j] + sm[(i * H + j) * kZPairCols + c];
+}
+
+// Pass Z with Mz = L = A B, 64 to 512 points: n = B n1 + n2, k = k1 + A k2.
+//   step A   one thread per (component, column, n2): the A-point transform over n1, whose upper half is
+//            padding: two A/2-point transforms as above;                         to shared memory
+//   step B   one thread per (column, k1), all components: twiddles W_L^{n2 k1}, B-point transform over n2,
+//            Green multiply of its B frequencies, inverse transform, twiddles;   to shared memory
+//   step A'  the inverse of step A, planes z < bz kept.
+// Four shared-memory accesses per value and no stage over padding, against 2 log4(L) + 4 of the radix-4 form:
+// complex64, 128^3 voxels (256 points) 525 -> 231 us, 64^3 (128 points) 62 -> 29 us, 100x37x60 113 -> 57 us;
+// complex128, bound by the FP64 units, 128^3 5970 -> 5220 us with sums as multiply-adds (radd).
+template <class C, int A, int B> struct ZFour {
+    static constexpr int L = A * B;
+    static constexpr int NC = 98304 / (3 * L * (int)sizeof(C)) >= 32 ? 32 : 98304 / (3 * L * (int)sizeof(C));   // columns per CTA
+    static constexpr size_t smem = (size_t)3 * L * NC * sizeof(C);
+    static constexpr int threads = sizeof(C) == 8 ? 256 : 128;
+    static constexpr int ctas = sizeof(C) == 16 || B < 16 ? 2 : 1;
+};
+
+template <class C, int A, int B, bool OCT>
+__global__ void __launch_bounds__((ZFour<C, A, B>::threads), (ZFour<C, A, B>::ctas)) k_z_four(ZArgs<C> a) {
+    constexpr int L = A * B, HA = A / 2, NC = ZFour<C, A, B>::NC, TS = kLmax / A, LG = ILog2<L>::v;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* sm = reinterpret_cast<C*>(smem_raw);      // [3][k1 B + n2][NC]
+    const int b = blockIdx.y;
+    if (!box_active(a.st, b)) return;
+    if (a.units != nullptr && threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(a.units, 1);
+    const int col0 = blockIdx.x * NC, nc = min(NC, a.ncols - col0);
+    C* W = a.w + (int64_t)b * a.box_stride + col0;
+    for (int task = threadIdx.x; task < 3 * B * NC; task += blockDim.x) {
+        const int c = task % NC, n2 = (task / NC) % B, comp = task / (NC * B);
+        if (c >= nc) continue;
+        const C* src = W + comp * a.comp_stride + c;
+        C* S = sm + (comp * L + n2) * NC + c;
+        C x[HA], y[HA];
+#pragma unroll
+        for (int j = 0; j < HA; ++j) {
+            const int n = j * B + n2;
+            x[j] = n < a.nzb ? src[n * a.axis] : czero<C>();
+            y[j] = j ? ztw<true>(x[j], j * TS, a.tw) : x[j];
+        }
+        dft<HA, true>(x);
+        dft<HA, true>(y);
+#pragma unroll
+        for (int m = 0; m < HA; ++m) {
+            S[(2 * m) * B * NC] = x[m];
+            S[(2 * m + 1) * B * NC] = y[m];
+        }
+    }
+    __syncthreads();
+    for (int task = threadIdx.x; task < A * NC; task += blockDim.x) {
+        const int c = task % NC, k1 = task / NC;
+        if (c >= nc) continue;
+        const ZColumn<C, OCT> zc(a, b, col0 + c);
+        C w[B], v[3][B];
+#pragma unroll
+        for (int n2 = 1; n2 < B; ++n2) w[n2] = __ldg(a.tw + ((n2 * k1) << (kLogLmax - LG)));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const C* S = sm + (i * L + k1 * B) * NC + c;
+#pragma unroll
+            for (int n2 = 0; n2 < B; ++n2) v[i][n2] = n2 ? cmul(S[n2 * NC], w[n2]) : S[0];
+            dft<B, true>(v[i]);
+        }
+#pragma unroll
+        for (int k2 = 0; k2 < B; ++k2) {
+            const int k = k1 + A * k2;
+            const bool up = k > L / 2;
+            const int f = up ? L - k : k;
+            int q;
+            if (OCT) q = f == L / 2 ? L / 2 : (int)(__brev((unsigned)f) >> (33 - LG));
+            else q = (int)(__brev((unsigned)f) >> (32 - LG));
+            C e[6];
+            zc.load(e, q, a.gcomp);
+            e[2] = cneg_if(e[2], up);
+            e[4] = cneg_if(e[4], up);
+            green3<2, false>(v[0][k2], v[1][k2], v[2][k2], e);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            C* S = sm + (i * L + k1 * B) * NC + c;
+            dft<B, false>(v[i]);
+#pragma unroll
+            for (int n2 = 0; n2 < B; ++n2) S[n2 * NC] = n2 ? cmulc(v[i][n2], w[n2]) : v[i][0];
+        }
+    }
+    __syncthreads();
+    for (int task = threadIdx.x; task < 3 * B * NC; task += blockDim.x) {
+        const int c = task % NC, n2 = (task / NC) % B, comp = task / (NC * B);
+        if (c >= nc) continue;
+        C* dst = W + comp * a.comp_stride + c;
+        const C* S = sm + (comp * L + n2) * NC + c;
+        C x[HA], y[HA];
+#pragma unroll
+        for (int m = 0; m < HA; ++m) {
+            x[m] = S[(2 * m) * B * NC];
+            y[m] = S[(2 * m + 1) * B * NC];
+        }
+        dft<HA, false>(x);
+        dft<HA, false>(y);
+#pragma unroll
+        for (int j = 0; j < HA; ++j) {
+            const int n = j * B + n2;
+            if (n < a.nzb) dst[n * a.axis] = x[j] + (j ? ztw<false>(y[j], j * TS, a.tw) : y[j]);
+        }
+    }
+}
+
+}  // namespace vie
+
+#include "fft_plane.cuh"
+
+namespace vie {
 
 // ---------------------------------------------------------------- four-step register passes (complex64)
 // An L = 32 A point transform (A = 2 .. 32) of a line as two register passes
@@ -623,6 +867,33 @@ static int launch_rows4_any(RowArgs<float2> a, Prof pf, cudaStream_t s) {
     }
 }
 
+template <class C, int A, int B, bool FWD>
+static int launch_line_rows(RowArgs<C> a, Prof pf, cudaStream_t s) {
+    constexpr int L = A * B, NR = LineRows<L>::n;
+    const size_t smem = (size_t)NR * (L + L / 8 + 8) * sizeof(C);
+    VIE_TRY(prep_smem(k_line_rows<C, A, B, FWD>, smem));
+    const int64_t grid = (a.nrows + NR - 1) / NR;
+    if (grid <= 0) return VIE_OK;
+    a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
+    k_line_rows<C, A, B, FWD><<<(unsigned)grid, kLineThreadsRow, smem, s>>>(a);
+    prof_end(s);
+    VIE_CK(cudaGetLastError());
+    return VIE_OK;
+}
+
+template <class C, int A, int B, bool FWD>
+static int launch_line_cols(ColArgs<C> a, int nb1, int nb2, Prof pf, cudaStream_t s) {
+    constexpr int NC = LineCols<C>::n;
+    const size_t smem = (size_t)A * B * NC * sizeof(C);
+    VIE_TRY(prep_smem(k_line_cols<C, A, B, FWD>, smem));
+    dim3 grid((a.ncols + NC - 1) / NC, nb1, nb2);
+    a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
+    k_line_cols<C, A, B, FWD><<<grid, line_threads_col<C>(), smem, s>>>(a);
+    prof_end(s);
+    VIE_CK(cudaGetLastError());
+    return VIE_OK;
+}
+
 template <class C, int MODE>
 static int launch_rows(RowArgs<C> a, Prof pf, cudaStream_t s) {
     if constexpr (std::is_same<C, float2>::value) {
@@ -632,6 +903,16 @@ static int launch_rows(RowArgs<C> a, Prof pf, cudaStream_t s) {
             if (MODE == ROW_FWD_CHI && 2 * a.n_in <= L && a.n_out == L) return launch_rows4_any<true>(a, pf, s);
             if (MODE == ROW_INV_UPDATE && 2 * a.n_out <= L && a.n_in == L) return launch_rows4_any<false>(a, pf, s);
         }
+    }
+    // complex128 rows of 256 and 512 points, given two waves of CTAs (below that the radix-4 form spreads a row
+    // over more threads: 28 against 42 us for 540 rows); complex64 rows are faster in the radix-2 form above
+    // (32 and 50 us forward and inverse against 37 and 62 at 256x256x16)
+    if (sizeof(C) == 16 && (a.lL == 8 || a.lL == 9) && a.nrows * (1 << a.lL) >= 2 * 152 * 4096) {
+        const int L = 1 << a.lL;
+        if (MODE == ROW_FWD_CHI && 2 * a.n_in <= L && a.n_out == L)
+            VIE_LONG_LINE_SWITCH(a.lL, return (launch_line_rows<C, AA, BB, true>(a, pf, s)));
+        if (MODE == ROW_INV_UPDATE && 2 * a.n_out <= L && a.n_in == L)
+            VIE_LONG_LINE_SWITCH(a.lL, return (launch_line_rows<C, AA, BB, false>(a, pf, s)));
     }
     a.ltr = pick_ltile(a.lL, sizeof(C), 1, 1);
     const int TR = 1 << a.ltr;
@@ -661,19 +942,17 @@ static int launch_cols4(ColArgs<float2> a, int nb1, int nb2, Prof pf, cudaStream
 template <class C, bool FWD>
 static int launch_cols(ColArgs<C> a, int nb1, int nb2, Prof pf, cudaStream_t s) {
     if constexpr (std::is_same<C, float2>::value) {
-        // four-step register path: complex64 columns of 64 .. 1024, pruned to half the length
+        // four-step register path: complex64 columns of 1024, pruned to half the length
         const int L = 1 << a.lL;
-        if (a.lL >= 6 && a.lL <= kLogLmax && (FWD ? (2 * a.n_in <= L && a.n_out == L)
+        if (a.lL == kLogLmax && (FWD ? (2 * a.n_in <= L && a.n_out == L)
                                                    : (2 * a.n_out <= L && a.n_in == L))) {
-            switch (a.lL) {
-                case 6: return launch_cols4<2, FWD>(a, nb1, nb2, pf, s);
-                case 7: return launch_cols4<4, FWD>(a, nb1, nb2, pf, s);
-                case 8: return launch_cols4<8, FWD>(a, nb1, nb2, pf, s);
-                case 9: return launch_cols4<16, FWD>(a, nb1, nb2, pf, s);
-                default: return launch_cols4<32, FWD>(a, nb1, nb2, pf, s);
-            }
+            return launch_cols4<32, FWD>(a, nb1, nb2, pf, s);
         }
     }
+    // two-step register transforms: columns of 64 to 512 points, pruned to half the length
+    if (a.lL >= 6 && a.lL <= 9 &&
+        (FWD ? (2 * a.n_in <= (1 << a.lL) && a.n_out == (1 << a.lL)) : (2 * a.n_out <= (1 << a.lL) && a.n_in == (1 << a.lL))))
+        VIE_LONG_LINE_SWITCH(a.lL, return (launch_line_cols<C, AA, BB, FWD>(a, nb1, nb2, pf, s)));
     a.ltc = pick_ltile(a.lL, sizeof(C), 1, 0);
     if ((1 << a.ltc) > a.ncols) a.ltc = ilog2(a.ncols) - ((1 << ilog2(a.ncols)) > a.ncols ? 1 : 0);
     if (a.ltc < 0) a.ltc = 0;
@@ -700,20 +979,66 @@ static int launch_zgreen_reg(ZArgs<float2> a, int nb, Prof pf, cudaStream_t s) {
     return VIE_OK;
 }
 
-template <class C>
-static int launch_zgreen(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
-    if constexpr (std::is_same<C, float2>::value) {
-        if (a.oct && a.lL <= 5) {   // register path: complex64, octant spectrum, Mz <= 32
-            switch (a.lL) {
-                case 0: return launch_zgreen_reg<1>(a, nb, pf, s);
-                case 1: return launch_zgreen_reg<2>(a, nb, pf, s);
-                case 2: return launch_zgreen_reg<4>(a, nb, pf, s);
-                case 3: return launch_zgreen_reg<8>(a, nb, pf, s);
-                case 4: return launch_zgreen_reg<16>(a, nb, pf, s);
-                default: return launch_zgreen_reg<32>(a, nb, pf, s);
-            }
+template <class C, int H, bool OCT>
+static int launch_z_pair(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
+    const size_t smem = (size_t)3 * H * kZPairCols * sizeof(C);
+    VIE_TRY(prep_smem(k_z_pair<C, H, OCT>, smem));
+    dim3 grid((a.ncols + kZPairCols - 1) / kZPairCols, nb);
+    a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
+    k_z_pair<C, H, OCT><<<grid, 2 * kZPairCols, smem, s>>>(a);
+    prof_end(s);
+    VIE_CK(cudaGetLastError());
+    return VIE_OK;
+}
+
+template <class C, int A, int B, bool OCT>
+static int launch_z_four(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
+    typedef ZFour<C, A, B> Z;
+    VIE_TRY(prep_smem(k_z_four<C, A, B, OCT>, Z::smem));
+    dim3 grid((a.ncols + Z::NC - 1) / Z::NC, nb);
+    a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
+    k_z_four<C, A, B, OCT><<<grid, Z::threads, Z::smem, s>>>(a);
+    prof_end(s);
+    VIE_CK(cudaGetLastError());
+    return VIE_OK;
+}
+
+template <class C, bool OCT>
+static int launch_z_reg(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
+    if constexpr (sizeof(C) == 8) {
+        switch (a.lL) {
+            case 2: return launch_zgreen_reg<4>(a, nb, pf, s);
+            case 3: return launch_zgreen_reg<8>(a, nb, pf, s);
+            case 4: return launch_zgreen_reg<16>(a, nb, pf, s);
+            case 5: return launch_zgreen_reg<32>(a, nb, pf, s);
+            default: break;
+        }
+    } else {
+        switch (a.lL) {
+            case 2: return launch_z_pair<C, 2, OCT>(a, nb, pf, s);
+            case 3: return launch_z_pair<C, 4, OCT>(a, nb, pf, s);
+            case 4: return launch_z_pair<C, 8, OCT>(a, nb, pf, s);
+            case 5: return launch_z_pair<C, 16, OCT>(a, nb, pf, s);
+            default: break;
         }
     }
+    switch (a.lL) {
+        case 6: return launch_z_four<C, 8, 8, OCT>(a, nb, pf, s);
+        case 7: return launch_z_four<C, 16, 8, OCT>(a, nb, pf, s);
+        case 8: return launch_z_four<C, 32, 8, OCT>(a, nb, pf, s);
+        default: return launch_z_four<C, 32, 16, OCT>(a, nb, pf, s);
+    }
+}
+
+template <class C>
+static int launch_zgreen(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
+    // Register transforms for 4 to 512 points of the symmetric operator (the box fills at most half of the
+    // axis); the radix-4 form for the rest: one plane, 1024 points, the nine spectra of the rooftop operator,
+    // and complex128 launches of less than two warps' columns per SM, where one thread's serial FP64 work
+    // (a column's parity: 84 us at 16^3 against 30 us) sets the time.
+    const bool few = sizeof(C) == 16 && (int64_t)a.ncols * nb < 152 * 64;
+    if (!a.nine && !few && a.lL >= 2 && a.lL <= 9 && 2 * a.nzb <= (1 << a.lL))
+        return a.oct ? launch_z_reg<C, true>(a, nb, pf, s) : launch_z_reg<C, false>(a, nb, pf, s);
     a.ltc = pick_ltile(a.lL, sizeof(C), 3, 0);
     if ((1 << a.ltc) > a.ncols) a.ltc = ilog2(a.ncols) - ((1 << ilog2(a.ncols)) > a.ncols ? 1 : 0);
     if (a.ltc < 0) a.ltc = 0;
@@ -726,6 +1051,26 @@ static int launch_zgreen(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
     prof_end(s);
     VIE_CK(cudaGetLastError());
     return VIE_OK;
+}
+
+template <class C, bool FWD>
+static int launch_plane(PlaneArgs<C> a, int nplanes, Prof pf, cudaStream_t s) {
+    const size_t smem = (size_t)a.pitch * ((size_t)1 << a.ly) * sizeof(C);
+    VIE_TRY(prep_smem(k_plane<C, FWD>, smem));
+    a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
+    k_plane<C, FWD><<<nplanes, a.lx + a.ly <= 10 ? 128 : a.lx + a.ly <= 12 ? 256 : 512, smem, s>>>(a);
+    prof_end(s);
+    VIE_CK(cudaGetLastError());
+    return VIE_OK;
+}
+
+// x and y transforms of a plane in one launch (k_plane): planes of 4 x 4 to 256 x 256 points that fit shared memory.
+// complex128 planes of more than 32 x 32 points need enough CTAs for the FP64 units of every SM (27 planes of
+// 32 x 256 points: 145 us against 74 in separate passes).
+template <class C> static bool plane_ok(const BoxSet& bs) {
+    if (sizeof(C) == 16 && bs.lx + bs.ly > 10 && (int64_t)bs.nb * 3 * bs.bz < 128) return false;
+    return bs.lx >= 2 && bs.lx <= 8 && bs.ly >= 2 && bs.ly <= 8 &&
+           (size_t)plane_pitch(bs.Mx) * bs.My * sizeof(C) <= (size_t)200 * 1024;
 }
 
 template <class C> static const C* chi_ptr(const BoxSet& bs);
@@ -755,8 +1100,16 @@ int mvm_boxes(const BoxSet& bs, const C* G, const C* x, C* y, const SegState* st
     const Prof piy{PK_Y_INV, b2 + b1, 0};
     const Prof pix{PK_X_INV, b1 + 2 * bv + (bs.mask ? box : 0), 0};
 
-    // pass X: chi * x, zero-padded forward FFT of every row
+    const bool planes = plane_ok<C>(bs);
+    PlaneArgs<C> pa{};
     RowArgs<C> rx{};
+    ColArgs<C> cy{};
+    if (planes) {
+        pa.in = x; pa.out = w2; pa.chi = chi_ptr<C>(bs); pa.st = st; pa.tw = T;
+        pa.bx = bs.bx; pa.by = bs.by; pa.bz = bs.bz; pa.lx = bs.lx; pa.ly = bs.ly; pa.pitch = plane_pitch(bs.Mx);
+        VIE_TRY((launch_plane<C, true>(pa, bs.nb * 3 * bs.bz, Prof{PK_X_FWD, bv + box * es + b2, 0}, s)));
+    } else {
+    // pass X: chi * x, zero-padded forward FFT of every row
     rx.in = x; rx.out = w1; rx.chi = chi_ptr<C>(bs); rx.st = st; rx.tw = T;
     rx.nrows = (int64_t)bs.nb * 3 * bs.bz * bs.by;
     rx.in_stride = bs.bx; rx.out_stride = bs.Mx; rx.n_in = bs.bx; rx.n_out = bs.Mx;
@@ -765,7 +1118,6 @@ int mvm_boxes(const BoxSet& bs, const C* G, const C* x, C* y, const SegState* st
     VIE_TRY((launch_rows<C, ROW_FWD_CHI>(rx, px, s)));
 
     // pass Y forward
-    ColArgs<C> cy{};
     cy.in = w1; cy.out = w2; cy.st = st; cy.tw = T;
     cy.ncols = bs.Mx; cy.n_in = bs.by; cy.n_out = bs.My; cy.lL = bs.ly; cy.twshift = kLogLmax - bs.ly;
     cy.in_axis = bs.Mx; cy.out_axis = bs.Mx;
@@ -773,6 +1125,7 @@ int mvm_boxes(const BoxSet& bs, const C* G, const C* x, C* y, const SegState* st
     cy.in_s2 = (int64_t)bs.bz * bs.by * bs.Mx; cy.out_s2 = (int64_t)bs.bz * planeXY;
     cy.b2_per_box = 3;
     VIE_TRY((launch_cols<C, true>(cy, bs.bz, bs.nb * 3, py, s)));
+    }
 
     // pass Z: forward, Green multiply, inverse
     ZArgs<C> z{};
@@ -785,6 +1138,10 @@ int mvm_boxes(const BoxSet& bs, const C* G, const C* x, C* y, const SegState* st
     if (nine && bs.oct) return fail(VIE_EINVAL, "mvm_boxes: nine spectra need the full layout");
     VIE_TRY(launch_zgreen<C>(z, bs.nb, pz, s));
 
+    if (planes) {
+        pa.in = w2; pa.out = y; pa.xin = xupd ? xupd : x; pa.mask = bs.mask; pa.chi = nullptr;
+        return launch_plane<C, false>(pa, bs.nb * 3 * bs.bz, Prof{PK_X_INV, b2 + 2 * bv + (bs.mask ? box : 0), 0}, s);
+    }
     // pass Y inverse: keep y < by
     ColArgs<C> iy = cy;
     iy.in = w2; iy.out = w1; iy.n_in = bs.My; iy.n_out = bs.by;

@@ -25,6 +25,7 @@
 #include <mutex>
 #include <vector>
 
+#include "dft_small.cuh"
 #include "fft_core.cuh"
 #include "vie_internal.cuh"
 
@@ -67,8 +68,8 @@ __device__ __forceinline__ bool dgood(double2 a) {
     return isfinite(a.x) && isfinite(a.y) && (a.x != 0.0 || a.y != 0.0);
 }
 template <class C> __device__ __forceinline__ void acc_dot(C& acc, C a, C b) {   // acc += conj(a) b
-    acc.x += a.x * b.x + a.y * b.y;
-    acc.y += a.x * b.y - a.y * b.x;
+    acc.x = fma(a.y, b.y, fma(a.x, b.x, acc.x));
+    acc.y = fma(-a.y, b.x, fma(a.x, b.y, acc.y));
 }
 
 // A block is solved by a team: the R CTAs of one thread-block cluster. Every
@@ -231,9 +232,11 @@ __device__ void phase_z(const InnerGroup<C>& g, C* W, C* sm, const C* tw) {
             C gyy = gp[3 * gcomp], gyz = gp[4 * gcomp], gzz = gp[5 * gcomp];
             C* q = sm + i * pitch + c;
             C X = q[0], Y = q[TC], Z = q[2 * TC];
-            q[0] = cmul(gxx, X) + cmul(gxy, Y) + cmul(gxz, Z);
-            q[TC] = cmul(gxy, X) + cmul(gyy, Y) + cmul(gyz, Z);
-            q[2 * TC] = cmul(gxz, X) + cmul(gyz, Y) + cmul(gzz, Z);
+            const C e[6] = {gxx, gxy, gxz, gyy, gyz, gzz};
+            green3<2, false>(X, Y, Z, e);
+            q[0] = X;
+            q[TC] = Y;
+            q[2 * TC] = Z;
         }
         __syncthreads();
         smem_fft<C, false, 3>(sm, g.lz, pitch, g.ltc, tw, kLogLmax - g.lz);

@@ -147,7 +147,7 @@ __device__ __forceinline__ void par_cols(const InnerGroup<C>& g, C* sm, int p) {
             const int pl = (int)fdiv(q, dx);
             s = sm + pl * zp + (q - pl * ex);
         }
-        const R sg = comp == AXIS ? (R)-1 : (R)1;
+        const bool sg = comp == AXIS;
         C a[H];
         if (FWD) {
 #pragma unroll
@@ -158,10 +158,10 @@ __device__ __forceinline__ void par_cols(const InnerGroup<C>& g, C* sm, int p) {
             }
             dft<H, true>(a);
 #pragma unroll
-            for (int j = 0; j < H; ++j) s[j * step] = j >= H / 2 ? cscale(a[j], sg) : a[j];
+            for (int j = 0; j < H; ++j) s[j * step] = j >= H / 2 ? cneg_if(a[j], sg) : a[j];
         } else {
 #pragma unroll
-            for (int j = 0; j < H; ++j) a[j] = j >= H / 2 ? cscale(s[j * step], sg) : s[j * step];
+            for (int j = 0; j < H; ++j) a[j] = j >= H / 2 ? cneg_if(s[j * step], sg) : s[j * step];
             dft<H, false>(a);
             if (p) {
 #pragma unroll
@@ -173,37 +173,6 @@ __device__ __forceinline__ void par_cols(const InnerGroup<C>& g, C* sm, int p) {
         }
     }
     __syncthreads();
-}
-
-template <class C> __device__ __forceinline__ void cmac(C& s, C a, C b) {
-    s.x += a.x * b.x - a.y * b.y;
-    s.y += a.x * b.y + a.y * b.x;
-}
-template <class C> __device__ __forceinline__ void cmacn(C& s, C a, C b) {   // s -= a b
-    s.x -= a.x * b.x - a.y * b.y;
-    s.y -= a.x * b.y + a.y * b.x;
-}
-
-// The symmetric 3x3 multiply of one frequency with the entries v (xx, xy, xz, yy, yz, zz); FLIP: the
-// frequency lies in the upper half of x (xy and xz change sign).
-template <bool FLIP, class C> __device__ __forceinline__ void par_green(C& X, C& Y, C& Z, const C (&v)[6]) {
-    C ox = cmul(v[0], X), oy = cmul(v[3], Y), oz = cmul(v[5], Z);
-    cmac(oy, v[4], Z);
-    cmac(oz, v[4], Y);
-    if (FLIP) {
-        cmacn(ox, v[1], Y);
-        cmacn(ox, v[2], Z);
-        cmacn(oy, v[1], X);
-        cmacn(oz, v[2], X);
-    } else {
-        cmac(ox, v[1], Y);
-        cmac(ox, v[2], Z);
-        cmac(oy, v[1], X);
-        cmac(oz, v[2], X);
-    }
-    X = ox;
-    Y = oy;
-    Z = oz;
 }
 
 // The frequencies kx = 2m + PX of one row: entries of frequency f = min(kx, 2H - kx) at gp[(6 f + c) n].
@@ -220,8 +189,8 @@ template <int H, int PX, class C> __device__ __forceinline__ void par_row_green(
             for (int c = 0; c < 6; ++c) w[c] = gp[(6 * (2 * (m + 1) + PX) + c) * n];
         }
         const int mm = (H - m - PX) % H;          // the mirror frequency
-        par_green<false>(a[0][m], a[1][m], a[2][m], v);
-        if (mm != m) par_green<true>(a[0][mm], a[1][mm], a[2][mm], v);
+        green3<0, false>(a[0][m], a[1][m], a[2][m], v);
+        if (mm != m) green3<0, true>(a[0][mm], a[1][mm], a[2][mm], v);
         if (m + 1 < NF) {
 #pragma unroll
             for (int c = 0; c < 6; ++c) v[c] = w[c];
@@ -588,14 +557,14 @@ __device__ __noinline__ typename real_of<C>::type par_update_cols(const InnerGro
                 }
             }
         }
-        const R sg = k.comp == 2 ? (R)-1 : (R)1;
+        const bool sg = k.comp == 2;
         C b[H];
 #pragma unroll
         for (int j = 0; j < H; ++j) b[j] = a[j];
         dft<H, true>(b);
 #pragma unroll
         for (int j = 0; j < H; ++j) {
-            const C o = j >= H / 2 ? cscale(b[j], sg) : b[j];
+            const C o = j >= H / 2 ? cneg_if(b[j], sg) : b[j];
             dst[0][k.so + j * zp] = o;
             dst[1][k.so + j * zp] = o;
         }
@@ -604,7 +573,7 @@ __device__ __noinline__ typename real_of<C>::type par_update_cols(const InnerGro
         dft<H, true>(a);
 #pragma unroll
         for (int j = 0; j < H; ++j) {
-            const C o = j >= H / 2 ? cscale(a[j], sg) : a[j];
+            const C o = j >= H / 2 ? cneg_if(a[j], sg) : a[j];
             dst[2][k.so + j * zp] = o;
             dst[3][k.so + j * zp] = o;
         }
@@ -631,7 +600,7 @@ __device__ __noinline__ void par_output_cols(const InnerGroup<C>& g, const ParVe
     for (int c = threadIdx.x; c < V.n; c += blockDim.x) {
         const ParCol k = par_col(g, V.n0 + c);
         const int e0 = k.e;
-        const R sg = k.comp == 2 ? (R)-1 : (R)1;
+        const bool sg = k.comp == 2;
         C a[H], b[H];
 #pragma unroll
         for (int j = 0; j < H; ++j) a[j] = src[0][k.so + j * zp] + src[1][k.so + j * zp];
@@ -639,8 +608,8 @@ __device__ __noinline__ void par_output_cols(const InnerGroup<C>& g, const ParVe
         for (int j = 0; j < H; ++j) b[j] = src[2][k.so + j * zp] + src[3][k.so + j * zp];
 #pragma unroll
         for (int j = H / 2; j < H; ++j) {
-            a[j] = cscale(a[j], sg);
-            b[j] = cscale(b[j], sg);
+            a[j] = cneg_if(a[j], sg);
+            b[j] = cneg_if(b[j], sg);
         }
         dft<H, false>(a);
         dft<H, false>(b);
