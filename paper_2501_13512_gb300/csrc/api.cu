@@ -1075,12 +1075,10 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
             Group& gr = g->groups[i];
             Bicg<C>& k = bk[i];
             const C* G = spec_of<C>(sp, 1 + i);
-            VIE_TRY(bicg_rho<C>(k, s));
             VIE_TRY(bicg_update_p<C>(k, s));
             VIE_TRY(mvm_boxes<C>(gr.bs, G, k.v.p, k.v.v, gr.st, s));
             VIE_TRY(bicg_sigma<C>(k, s));
             VIE_TRY(bicg_update_s<C>(k, s));
-            VIE_TRY(bicg_x_half<C>(k, s));
             VIE_TRY(mvm_boxes<C>(gr.bs, G, k.v.s, k.v.t, gr.st, s));
             VIE_TRY(bicg_omega<C>(k, s));
             VIE_TRY(bicg_update_xr<C>(k, s));
@@ -1096,6 +1094,8 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
             if (active == 0) break;
         }
     }
+    // x += alpha p of the blocks that stopped at a half step (nothing of theirs has changed since)
+    for (int i : batched) VIE_TRY(bicg_x_half<C>(bk[i], s));
     if (beside) {
         VIE_CK(cudaEventRecord(g->join_ev, g->s2));
         VIE_CK(cudaStreamWaitEvent(s, g->join_ev, 0));
@@ -1234,14 +1234,12 @@ static int bicgstab_full(vie_grid* g, const vie_spectrum* sp, KrylovVecs<C> v, c
         return VIE_OK;
     };
     for (int it = 0; it < maxit && hs.status == SEG_ACTIVE; ++it) {
-        VIE_TRY(bicg_rho<C>(k, s));
         VIE_TRY(bicg_update_p<C>(k, s));
         if (pre) VIE_TRY(precond(k.v.p, k.v.y));
         VIE_TRY(mvm_full<C>(g, sp, k.v.y, k.v.v, s));
         (prec_of<C>() == VIE_C128 ? acc.mv128 : acc.mv64)++;
         VIE_TRY(bicg_sigma<C>(k, s));
         VIE_TRY(bicg_update_s<C>(k, s));
-        VIE_TRY(bicg_x_half<C>(k, s));
         VIE_TRY(read_outer_state(g, &hs, s, o->wait_timeout_ms));
         if (hs.status != SEG_ACTIVE) break;
         if (pre) VIE_TRY(precond(k.v.s, k.v.z));
@@ -1251,6 +1249,7 @@ static int bicgstab_full(vie_grid* g, const vie_spectrum* sp, KrylovVecs<C> v, c
         VIE_TRY(bicg_update_xr<C>(k, s));
         VIE_TRY(read_outer_state(g, &hs, s, o->wait_timeout_ms));
     }
+    if (hs.status == SEG_HALF_PENDING) VIE_TRY(bicg_x_half<C>(k, s));
     VIE_TRY(read_outer_state(g, &hs, s, o->wait_timeout_ms));
     *final_state = hs;
     return VIE_OK;

@@ -432,12 +432,10 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
             k.red = &b->red;
             VIE_TRY(bicg_init_tols<float2>(k, b->d_tols, o->outer_maxit, s));
             for (int it = 0; it < o->outer_maxit; ++it) {
-                VIE_TRY(bicg_rho<float2>(k, s));
                 VIE_TRY(bicg_update_p<float2>(k, s));
                 VIE_TRY(mvm_boxes<float2>(bs, nullptr, k.v.p, k.v.v, b->st, s, nullptr, b->d_gb64));
                 VIE_TRY(bicg_sigma<float2>(k, s));
                 VIE_TRY(bicg_update_s<float2>(k, s));
-                VIE_TRY(bicg_x_half<float2>(k, s));
                 VIE_TRY(mvm_boxes<float2>(bs, nullptr, k.v.s, k.v.t, b->st, s, nullptr, b->d_gb64));
                 VIE_TRY(bicg_omega<float2>(k, s));
                 VIE_TRY(bicg_update_xr<float2>(k, s));
@@ -448,6 +446,7 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
                     if (*(int*)b->h_scal == 0) break;
                 }
             }
+            VIE_TRY(bicg_x_half<float2>(k, s));   // instances that stopped at a half step
         }
         k_seg_add<<<grid1(nv), 256, 0, s>>>(x, b->k64.x, b->d_rn2, b->d_tols, b->n3, nb);
         VIE_CK(cudaGetLastError());

@@ -11,6 +11,15 @@
 // applies the scalar update, so results are deterministic. Complex64 vectors
 // are multiplied and summed in FP32 within a thread and in FP64 across
 // threads; complex128 vectors use FP64 throughout. Scalars are FP64.
+//
+// On short segments these kernels are bound by FP64 instructions (two lanes a
+// clock and SM, whole warps whatever their active lanes), not by memory: so
+// only the sums an operation has are reduced, halved over the lanes, and every
+// coefficient is computed once, by the thread that finishes the sum (with
+// beta formed by every thread of the p update and 20 additions per warp and
+// sum, 13 to 18 us a launch for 8 segments of 24^3 voxels). The sum <rhat, r>
+// rides in the x/r update, so an iteration takes five launches beside its
+// products.
 #include <math.h>
 
 #include "vie_internal.cuh"
@@ -19,7 +28,11 @@ namespace vie {
 
 constexpr int kRedThreads = 256;
 
-enum VecOp { OP_INIT = 0, OP_P, OP_S, OP_XHALF, OP_XR, OP_RHO, OP_SIGMA, OP_OMEGA };
+enum VecOp { OP_INIT = 0, OP_P, OP_S, OP_XHALF, OP_XR, OP_SIGMA, OP_OMEGA };
+// real sums of an operation
+__host__ __device__ constexpr int op_sums(int op) {
+    return op == OP_INIT || op == OP_S ? 1 : op == OP_SIGMA ? 2 : op == OP_XR || op == OP_OMEGA ? 3 : 0;
+}
 
 template <class C> struct VecArgs {
     KrylovVecs<C> v;
@@ -36,53 +49,52 @@ template <class C> struct VecArgs {
 };
 
 __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-    double d = b.x * b.x + b.y * b.y;
-    return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
+    const double r = 1.0 / (b.x * b.x + b.y * b.y);
+    return make_double2((a.x * b.x + a.y * b.y) * r, (a.y * b.x - a.x * b.y) * r);
 }
+__device__ __forceinline__ float2 to_c64(double2 a) { return make_float2((float)a.x, (float)a.y); }
 __device__ __forceinline__ bool cfinite_nz(double2 a) {
     return isfinite(a.x) && isfinite(a.y) && (a.x != 0.0 || a.y != 0.0);
 }
 
-template <class C> struct Acc;
-template <> struct Acc<double2> {
-    typedef double2 T;
-    static __device__ __forceinline__ double2 widen(double2 a) { return a; }
-};
-template <> struct Acc<float2> {
-    typedef float2 T;
-    static __device__ __forceinline__ double2 widen(float2 a) { return make_double2(a.x, a.y); }
-};
-
 // conj(a) * b accumulated into acc (same precision as the vectors)
 template <class C> __device__ __forceinline__ void cdot_acc(C& acc, C a, C b) {
-    acc.x += a.x * b.x + a.y * b.y;
-    acc.y += a.x * b.y - a.y * b.x;
+    acc.x = fma(a.y, b.y, fma(a.x, b.x, acc.x));
+    acc.y = fma(-a.y, b.x, fma(a.x, b.y, acc.y));
 }
+template <class C> __device__ __forceinline__ C coef(double2 a, float2 a32);
+template <> __device__ __forceinline__ double2 coef<double2>(double2 a, float2) { return a; }
+template <> __device__ __forceinline__ float2 coef<float2>(double2, float2 a32) { return a32; }
 
-__device__ __forceinline__ double2 warp_sum(double2 v) {
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-    }
-    return v;
-}
-
-// Deterministic block sum of two complex values; result valid in thread 0.
-__device__ void block_sum2(double2& a, double2& b) {
-    __shared__ double2 sh[2][kRedThreads / 32];
-    a = warp_sum(a);
-    b = warp_sum(b);
+// Block sums of NV (1, 2 or 4) values of every thread; the total of value i is returned to thread i.
+template <int NV> __device__ double block_sums(double (&x)[NV]) {
+    constexpr int NW = kRedThreads / 32, LG = NV == 4 ? 2 : NV - 1;   // log2 NV
+    __shared__ double sh[NV][NW];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) { sh[0][w] = a; sh[1][w] = b; }
+    int o = 16;
+#pragma unroll
+    for (int h = NV / 2; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (l & o) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const double send = up ? x[k] : x[k + h], keep = up ? x[k + h] : x[k];
+            x[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o >>= 1) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+    // the lane's value index: its upper log2 NV bits
+    if ((l & (31 >> LG)) == 0) sh[l >> (5 - LG)][w] = x[0];
     __syncthreads();
+    double t = 0.0;
     if (w == 0) {
-        const int nw = blockDim.x >> 5;
-        a = l < nw ? sh[0][l] : make_double2(0, 0);
-        b = l < nw ? sh[1][l] : make_double2(0, 0);
-        a = warp_sum(a);
-        b = warp_sum(b);
+        if (l < NV * NW) t = sh[l / NW][l % NW];
+#pragma unroll
+        for (int m = 1; m < NW; m <<= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
+        t = __shfl_sync(0xffffffffu, t, (l & (NV - 1)) * NW);
     }
     __syncthreads();
+    return t;
 }
 
 __device__ __forceinline__ void leave_active(int* n_active) { atomicSub(n_active, 1); }
@@ -95,7 +107,11 @@ __device__ void finalize(SegState& s, double2 d1, double2 d2, int* n_active, dou
         s.bnorm2 = d1.x;
         s.tol2 = tol * tol * d1.x;
         s.res2 = d1.x;
-        s.rho = s.rho_prev = s.alpha = s.omega = make_double2(1.0, 0.0);
+        s.rho = make_double2(d1.x, 0.0);        // <rhat, r> with rhat = r = b
+        s.alpha = s.omega = make_double2(1.0, 0.0);
+        s.alpha32 = s.omega32 = make_float2(1.f, 0.f);
+        s.beta = make_double2(0.0, 0.0);        // p = v = 0 before the first p update
+        s.beta32 = make_float2(0.f, 0.f);
         s.iters = 0.0;
         s.maxit = maxit;
         if (!isfinite(d1.x)) {
@@ -106,18 +122,20 @@ __device__ void finalize(SegState& s, double2 d1, double2 d2, int* n_active, dou
             s.status = SEG_ACTIVE;
             atomicAdd(n_active, 1);
         }
-    } else if (OP == OP_RHO) {
-        s.rho = d1;
-        if (!cfinite_nz(d1)) { s.status = SEG_BREAKDOWN; leave_active(n_active); }
     } else if (OP == OP_SIGMA) {
         if (!cfinite_nz(d1)) { s.status = SEG_BREAKDOWN; leave_active(n_active); }
-        else s.alpha = cdiv(s.rho, d1);
+        else {
+            s.alpha = cdiv(s.rho, d1);
+            s.alpha32 = to_c64(s.alpha);
+        }
     } else if (OP == OP_OMEGA) {
         if (!(d2.x > 0.0) || !isfinite(d2.x) || !isfinite(d1.x) || !isfinite(d1.y)) {
             s.status = SEG_BREAKDOWN;
             leave_active(n_active);
         } else {
-            s.omega = make_double2(d1.x / d2.x, d1.y / d2.x);
+            const double r = 1.0 / d2.x;
+            s.omega = make_double2(d1.x * r, d1.y * r);
+            s.omega32 = to_c64(s.omega);
         }
     } else if (OP == OP_S) {
         s.res2 = d1.x;
@@ -125,14 +143,19 @@ __device__ void finalize(SegState& s, double2 d1, double2 d2, int* n_active, dou
         else if (d1.x <= s.tol2) { s.status = SEG_HALF_PENDING; s.iters += 0.5; leave_active(n_active); }
     } else if (OP == OP_XHALF) {
         s.status = SEG_CONVERGED;
-    } else if (OP == OP_XR) {
-        s.res2 = d1.x;
+    } else if (OP == OP_XR) {                   // d1 = <rhat, r>, d2.x = ||r||^2
+        s.res2 = d2.x;
         s.iters += 1.0;
-        s.rho_prev = s.rho;
-        if (!isfinite(d1.x)) { s.status = SEG_BREAKDOWN; leave_active(n_active); }
-        else if (d1.x <= s.tol2) { s.status = SEG_CONVERGED; leave_active(n_active); }
+        if (!isfinite(d2.x)) { s.status = SEG_BREAKDOWN; leave_active(n_active); }
+        else if (d2.x <= s.tol2) { s.status = SEG_CONVERGED; leave_active(n_active); }
         else if (s.iters >= (double)s.maxit) { s.status = SEG_MAXIT; leave_active(n_active); }
-        else if (s.omega.x == 0.0 && s.omega.y == 0.0) { s.status = SEG_BREAKDOWN; leave_active(n_active); }
+        else if ((s.omega.x == 0.0 && s.omega.y == 0.0) || !cfinite_nz(d1)) { s.status = SEG_BREAKDOWN; leave_active(n_active); }
+        else {
+            // beta = (rho / rho_prev) (alpha / omega)
+            s.beta = cdiv(cmul(d1, s.alpha), cmul(s.rho, s.omega));
+            s.beta32 = to_c64(s.beta);
+            s.rho = d1;
+        }
     }
 }
 
@@ -148,72 +171,100 @@ __global__ void __launch_bounds__(kRedThreads) k_bicg(VecArgs<C> a) {
     if (a.units != nullptr && threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(a.units, 1);
     const int64_t off = (int64_t)seg * a.seglen;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    constexpr int U = 4;                        // elements per thread whose loads are issued together
     C acc1 = czero<C>(), acc2 = czero<C>();
-
-    C alpha = cmk<C>(S.alpha.x, S.alpha.y), omega = cmk<C>(S.omega.x, S.omega.y), beta = czero<C>();
-    if (OP == OP_P) {
-        double2 bt = cmul(cdiv(S.rho, S.rho_prev), cdiv(S.alpha, S.omega));
-        beta = cmk<C>(bt.x, bt.y);
-    }
-    KrylovVecs<C> v = a.v;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.seglen; i += stride) {
-        const int64_t k = off + i;
-        if (OP == OP_INIT) {
-            C b = v.b[k];
-            v.x[k] = czero<C>();
-            v.r[k] = b;
-            v.rhat[k] = b;
-            v.p[k] = czero<C>();
-            v.v[k] = czero<C>();
-            cdot_acc(acc1, b, b);
-        } else if (OP == OP_P) {
-            v.p[k] = v.r[k] + cmul(beta, v.p[k] - cmul(omega, v.v[k]));
-        } else if (OP == OP_S) {
-            C s = v.r[k] - cmul(alpha, v.v[k]);
-            v.s[k] = s;
-            cdot_acc(acc1, s, s);
-        } else if (OP == OP_XHALF) {
-            v.x[k] = v.x[k] + cmul(alpha, v.y[k]);
-        } else if (OP == OP_XR) {
-            v.x[k] = v.x[k] + cmul(alpha, v.y[k]) + cmul(omega, v.z[k]);
-            C r = v.s[k] - cmul(omega, v.t[k]);
-            v.r[k] = r;
-            cdot_acc(acc1, r, r);
-        } else if (OP == OP_RHO) {
-            cdot_acc(acc1, v.rhat[k], v.r[k]);
-        } else if (OP == OP_SIGMA) {
-            cdot_acc(acc1, v.rhat[k], v.v[k]);
-        } else if (OP == OP_OMEGA) {
-            C t = v.t[k];
-            cdot_acc(acc1, t, v.s[k]);
-            cdot_acc(acc2, t, t);
+    const C alpha = coef<C>(S.alpha, S.alpha32), omega = coef<C>(S.omega, S.omega32), beta = coef<C>(S.beta, S.beta32);
+    const KrylovVecs<C> v = a.v;
+    // vectors read by the operation, in order of the argument list of apply
+    const C* in0 = OP == OP_INIT ? v.b : OP == OP_P || OP == OP_S ? v.r : OP == OP_XHALF || OP == OP_XR ? v.x
+                   : OP == OP_SIGMA ? v.rhat : v.t;
+    const C* in1 = OP == OP_P ? v.p : OP == OP_S || OP == OP_SIGMA ? v.v : OP == OP_XHALF || OP == OP_XR ? v.y : v.s;
+    const C* in2 = OP == OP_P ? v.v : v.z;
+    constexpr int NIN = OP == OP_INIT ? 1 : OP == OP_P ? 3 : OP == OP_XR ? 6 : 2;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < a.seglen; i0 += U * stride) {
+        C x[U][NIN];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * stride, k = off + (i < a.seglen ? i : i0);
+            x[u][0] = in0[k];
+            if constexpr (NIN > 1) x[u][1] = in1[k];
+            if constexpr (NIN > 2) x[u][2] = in2[k];
+            if constexpr (NIN == 6) {
+                x[u][3] = v.s[k];
+                x[u][4] = v.t[k];
+                x[u][5] = v.rhat[k];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * stride, k = off + i;
+            if (i >= a.seglen) break;
+            if constexpr (OP == OP_INIT) {
+                const C b = x[u][0];
+                v.x[k] = czero<C>();
+                v.r[k] = b;
+                v.rhat[k] = b;
+                v.p[k] = czero<C>();
+                v.v[k] = czero<C>();
+                cdot_acc(acc1, b, b);
+            } else if constexpr (OP == OP_P) {
+                v.p[k] = x[u][0] + cmul(beta, x[u][1] - cmul(omega, x[u][2]));
+            } else if constexpr (OP == OP_S) {
+                const C s = x[u][0] - cmul(alpha, x[u][1]);
+                v.s[k] = s;
+                cdot_acc(acc1, s, s);
+            } else if constexpr (OP == OP_XHALF) {
+                v.x[k] = x[u][0] + cmul(alpha, x[u][1]);
+            } else if constexpr (OP == OP_XR) {
+                v.x[k] = x[u][0] + cmul(alpha, x[u][1]) + cmul(omega, x[u][2]);
+                const C r = x[u][3] - cmul(omega, x[u][4]);
+                v.r[k] = r;
+                cdot_acc(acc1, x[u][5], r);
+                cdot_acc(acc2, r, r);
+            } else if constexpr (OP == OP_SIGMA) {
+                cdot_acc(acc1, x[u][0], x[u][1]);
+            } else {
+                cdot_acc(acc1, x[u][0], x[u][1]);
+                cdot_acc(acc2, x[u][0], x[u][0]);
+            }
         }
     }
-    double2 d1 = Acc<C>::widen(acc1), d2 = Acc<C>::widen(acc2);
-    block_sum2(d1, d2);
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        double2* pp = a.part + ((int64_t)seg * a.maxcta + blockIdx.x) * 2;
-        pp[0] = d1;
-        pp[1] = d2;
-        __threadfence();
-        unsigned ticket = atomicAdd(&a.count[seg], 1u);
-        last = (ticket == gridDim.x - 1);
+    if constexpr (OP == OP_P) return;
+    constexpr int NV = op_sums(OP) == 3 ? 4 : op_sums(OP) == 0 ? 1 : op_sums(OP);
+    double d[NV], t = 0.0;
+    d[0] = (double)acc1.x;
+    if constexpr (NV > 1) d[1] = (double)acc1.y;
+    if constexpr (NV == 4) {
+        d[2] = (double)acc2.x;
+        d[3] = 0.0;
     }
+    if constexpr (op_sums(OP) > 0) t = block_sums(d);
+    double* part = reinterpret_cast<double*>(a.part + (int64_t)seg * a.maxcta * 2);
+    __shared__ bool last;
+    if (threadIdx.x < NV) {
+        part[4 * blockIdx.x + threadIdx.x] = t;
+        __threadfence();
+    }
+    __syncwarp();
+    if (threadIdx.x == 0) last = atomicAdd(&a.count[seg], 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
     // fixed-order sum of the partials of this segment
-    double2 s1 = make_double2(0, 0), s2 = make_double2(0, 0);
-    const volatile double2* pp = a.part + (int64_t)seg * a.maxcta * 2;
-    for (int c = threadIdx.x; c < (int)gridDim.x; c += blockDim.x) {
-        s1.x += pp[2 * c].x; s1.y += pp[2 * c].y;
-        s2.x += pp[2 * c + 1].x; s2.y += pp[2 * c + 1].y;
+    if constexpr (op_sums(OP) > 0) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+            d[i] = threadIdx.x < gridDim.x ? __ldcg(part + 4 * threadIdx.x + i) : 0.0;
+        t = block_sums(d);
     }
-    block_sum2(s1, s2);
-    if (threadIdx.x == 0) {
-        a.count[seg] = 0;
-        finalize<OP>(S, s1, s2, a.n_active, a.tols ? a.tols[seg] : a.tol, a.maxit);
+    if (threadIdx.x < 32) {
+        const double t0 = __shfl_sync(0xffffffffu, t, 0), t1 = __shfl_sync(0xffffffffu, t, 1 % NV),
+                     t2 = __shfl_sync(0xffffffffu, t, 2 % NV);
+        if (threadIdx.x == 0) {
+            a.count[seg] = 0;
+            finalize<OP>(S, make_double2(t0, NV > 1 ? t1 : 0.0), make_double2(NV == 4 ? t2 : 0.0, 0.0), a.n_active,
+                         a.tols ? a.tols[seg] : a.tol, a.maxit);
+        }
     }
 }
 
@@ -230,12 +281,12 @@ static int launch_bicg(Bicg<C>& k, int op, double tol, int maxit, cudaStream_t s
     a.maxcta = kMaxCtaPerSeg;
     a.tol = tol;
     a.maxit = maxit;
-    int64_t want = (k.seglen + (int64_t)kRedThreads * 8 - 1) / ((int64_t)kRedThreads * 8);
+    int64_t want = (k.seglen + (int64_t)kRedThreads * 4 - 1) / ((int64_t)kRedThreads * 4);
     int nct = (int)std::max<int64_t>(1, std::min<int64_t>(want, kMaxCtaPerSeg));
     dim3 grid(nct, k.nseg);
     // vectors touched per segment by each op (reads + writes)
-    static const int nvec[] = {6, 4, 3, 3, 7, 2, 2, 2};
-    const bool dot = op == OP_RHO || op == OP_SIGMA || op == OP_OMEGA;
+    static const int nvec[] = {6, 4, 3, 3, 8, 2, 2};
+    const bool dot = op == OP_SIGMA || op == OP_OMEGA;
     a.units = prof_begin(s, dot ? PK_BICG_DOT : PK_BICG_UPDATE, sizeof(C) == 16 ? VIE_C128 : VIE_C64,
                          (int64_t)nvec[op] * k.seglen * (int64_t)sizeof(C), 0, true);
     switch (op) {
@@ -244,7 +295,6 @@ static int launch_bicg(Bicg<C>& k, int op, double tol, int maxit, cudaStream_t s
         case OP_S: k_bicg<C, OP_S><<<grid, kRedThreads, 0, s>>>(a); break;
         case OP_XHALF: k_bicg<C, OP_XHALF><<<grid, kRedThreads, 0, s>>>(a); break;
         case OP_XR: k_bicg<C, OP_XR><<<grid, kRedThreads, 0, s>>>(a); break;
-        case OP_RHO: k_bicg<C, OP_RHO><<<grid, kRedThreads, 0, s>>>(a); break;
         case OP_SIGMA: k_bicg<C, OP_SIGMA><<<grid, kRedThreads, 0, s>>>(a); break;
         case OP_OMEGA: k_bicg<C, OP_OMEGA><<<grid, kRedThreads, 0, s>>>(a); break;
         default: prof_end(s); return fail(VIE_EINVAL, "bad BiCGSTAB op");
@@ -262,7 +312,6 @@ template <class C> int bicg_init_tols(Bicg<C>& k, const double* tols, int maxit,
     VIE_CK(cudaMemsetAsync(k.red->n_active, 0, sizeof(int), s));
     return launch_bicg(k, OP_INIT, 0.0, maxit, s, tols);
 }
-template <class C> int bicg_rho(Bicg<C>& k, cudaStream_t s) { return launch_bicg(k, OP_RHO, 0, 0, s); }
 template <class C> int bicg_update_p(Bicg<C>& k, cudaStream_t s) { return launch_bicg(k, OP_P, 0, 0, s); }
 template <class C> int bicg_sigma(Bicg<C>& k, cudaStream_t s) { return launch_bicg(k, OP_SIGMA, 0, 0, s); }
 template <class C> int bicg_update_s(Bicg<C>& k, cudaStream_t s) { return launch_bicg(k, OP_S, 0, 0, s); }
@@ -273,7 +322,6 @@ template <class C> int bicg_update_xr(Bicg<C>& k, cudaStream_t s) { return launc
 #define VIE_INST(C)                                                        \
     template int bicg_init<C>(Bicg<C>&, double, int, cudaStream_t);        \
     template int bicg_init_tols<C>(Bicg<C>&, const double*, int, cudaStream_t); \
-    template int bicg_rho<C>(Bicg<C>&, cudaStream_t);                      \
     template int bicg_update_p<C>(Bicg<C>&, cudaStream_t);                 \
     template int bicg_sigma<C>(Bicg<C>&, cudaStream_t);                    \
     template int bicg_update_s<C>(Bicg<C>&, cudaStream_t);                 \
@@ -320,28 +368,27 @@ int vec_residual128(const double2* b, const double2* ax, double2* r, int64_t n, 
 
 // ||a||^2 in FP64 into d_out[0] (single segment, deterministic two-level sum).
 __global__ void __launch_bounds__(kRedThreads) k_norm2(const double2* a, int64_t n, double2* part, unsigned* count, double* out) {
-    double2 acc = make_double2(0, 0), zero = make_double2(0, 0);
+    double acc[1] = {0.0};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         double2 v = a[i];
-        acc.x += v.x * v.x + v.y * v.y;
+        acc[0] = fma(v.y, v.y, fma(v.x, v.x, acc[0]));
     }
-    block_sum2(acc, zero);
+    double t = block_sums(acc);
     __shared__ bool last;
+    double* pp = reinterpret_cast<double*>(part);
     if (threadIdx.x == 0) {
-        part[2 * blockIdx.x] = acc;
+        pp[blockIdx.x] = t;
         __threadfence();
         last = atomicAdd(count, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double2 s1 = make_double2(0, 0), s2 = make_double2(0, 0);
-    const volatile double2* pp = part;
-    for (int c = threadIdx.x; c < (int)gridDim.x; c += blockDim.x) s1.x += pp[2 * c].x;
-    block_sum2(s1, s2);
+    acc[0] = threadIdx.x < gridDim.x ? __ldcg(pp + threadIdx.x) : 0.0;
+    t = block_sums(acc);
     if (threadIdx.x == 0) {
         *count = 0;
-        *out = s1.x;
+        *out = t;
     }
 }
 int vec_norm2_128(const double2* a, int64_t n, ReduceScratch* red, double* d_out, cudaStream_t s) {

@@ -380,13 +380,11 @@ extern "C" int vie_rooftop_solve(vie_rooftop* r, const void* b_dev, void* w_dev,
     SegState hs;
     VIE_TRY(read_state(r, &hs, s, wait_timeout_ms));
     for (int it = 0; it < maxit && hs.status == SEG_ACTIVE; ++it) {
-        VIE_TRY(bicg_rho<double2>(k, s));
         VIE_TRY(bicg_update_p<double2>(k, s));
         VIE_TRY(rooftop_mvm<double2>(r, k.v.y, k.v.v, s));
         ++mv;
         VIE_TRY(bicg_sigma<double2>(k, s));
         VIE_TRY(bicg_update_s<double2>(k, s));
-        VIE_TRY(bicg_x_half<double2>(k, s));
         VIE_TRY(read_state(r, &hs, s, wait_timeout_ms));
         if (hs.status != SEG_ACTIVE) break;
         VIE_TRY(rooftop_mvm<double2>(r, k.v.z, k.v.t, s));
@@ -395,6 +393,7 @@ extern "C" int vie_rooftop_solve(vie_rooftop* r, const void* b_dev, void* w_dev,
         VIE_TRY(bicg_update_xr<double2>(k, s));
         VIE_TRY(read_state(r, &hs, s, wait_timeout_ms));
     }
+    if (hs.status == SEG_HALF_PENDING) VIE_TRY(bicg_x_half<double2>(k, s));
     VIE_TRY(read_state(r, &hs, s, wait_timeout_ms));
     int rc = hs.status == SEG_CONVERGED ? VIE_OK : (hs.status == SEG_BREAKDOWN ? VIE_EBREAKDOWN : VIE_ENOTCONV);
     if (stats) {

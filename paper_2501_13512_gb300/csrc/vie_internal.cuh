@@ -172,7 +172,8 @@ enum SegStatus : int {
 };
 
 struct SegState {
-    double2 rho, rho_prev, alpha, omega;
+    double2 rho, alpha, omega, beta;
+    float2 alpha32, omega32, beta32;   // the same, rounded, for complex64 vectors
     double bnorm2, res2, tol2;
     double iters;          // half-steps counted as 0.5
     int status;
@@ -353,7 +354,6 @@ struct Bicg {
 };
 template <class C> int bicg_init(Bicg<C>& k, double tol, int maxit, cudaStream_t s);
 template <class C> int bicg_init_tols(Bicg<C>& k, const double* tols, int maxit, cudaStream_t s);
-template <class C> int bicg_rho(Bicg<C>& k, cudaStream_t s);
 template <class C> int bicg_update_p(Bicg<C>& k, cudaStream_t s);
 template <class C> int bicg_sigma(Bicg<C>& k, cudaStream_t s);
 template <class C> int bicg_update_s(Bicg<C>& k, cudaStream_t s);
