@@ -613,31 +613,41 @@ extern "C" int vie_green_spectrum_near(vie_grid* g, double k0, int mask, int32_t
 }
 
 static void free_par(vie_spectrum* sp) {
-    for (auto& v : sp->par)
-        for (ParSpec& p : v) {
-            dfree(p.g128);
-            dfree(p.g64);
-        }
+    for (void* p : sp->par_alloc) dfree(p);
 }
 
-// Spectra of the parity-split MVM for one group: the lengths of its box (they hold every block, so the
-// spectrum serves any grid of the same shape signature), then those of its smaller classes.
-static int par_spectra(const Group& gr, const double2* K, int mask, std::vector<ParSpec>& out, cudaStream_t s) {
+// Allocates the spectra of the parity-split MVM for one group: the lengths of its box (they hold every block,
+// so the spectrum serves any grid of the same shape signature), then those of its smaller classes.
+static int alloc_par(vie_spectrum* sp, const Group& gr, int mask, std::vector<ParSpec>& out) {
     if (gr.par.empty()) return VIE_OK;
-    auto add = [&](int hx, int hy, int hz) -> int {
+    auto add = [&](int hx, int hy, int hz) {
         for (const ParSpec& p : out)
-            if (p.hx == hx && p.hy == hy && p.hz == hz) return VIE_OK;
+            if (p.hx == hx && p.hy == hy && p.hz == hz) return;
         ParSpec p;
         p.hx = hx; p.hy = hy; p.hz = hz;
         out.push_back(p);
-        const int64_t n = par_spectrum_elems(hx, hy, hz);
-        ParSpec& q = out.back();
-        if (mask & VIE_C128) VIE_TRY(dmalloc((void**)&q.g128, n * sizeof(double2), "vie_green_spectrum"));
-        if (mask & VIE_C64) VIE_TRY(dmalloc((void**)&q.g64, n * sizeof(float2), "vie_green_spectrum"));
-        return par_spectrum(gr.bs, K, hx, hy, hz, q.g128, q.g64, s);
     };
-    VIE_TRY(add(par_len(gr.bs.bx), par_len(gr.bs.by), par_len(gr.bs.bz)));
-    for (const ParClass& c : gr.par) VIE_TRY(add(c.hx, c.hy, c.hz));
+    add(par_len(gr.bs.bx), par_len(gr.bs.by), par_len(gr.bs.bz));
+    for (const ParClass& c : gr.par) add(c.hx, c.hy, c.hz);
+    int64_t n = 0;
+    for (const ParSpec& p : out) n += par_spectrum_elems(p.hx, p.hy, p.hz);
+    double2* b128 = nullptr;
+    float2* b64 = nullptr;
+    if (mask & VIE_C128) {
+        VIE_TRY(dmalloc((void**)&b128, n * sizeof(double2), "vie_green_spectrum"));
+        sp->par_alloc.push_back(b128);
+    }
+    if (mask & VIE_C64) {
+        VIE_TRY(dmalloc((void**)&b64, n * sizeof(float2), "vie_green_spectrum"));
+        sp->par_alloc.push_back(b64);
+    }
+    for (ParSpec& p : out) {
+        p.g128 = b128;
+        p.g64 = b64;
+        const int64_t e = par_spectrum_elems(p.hx, p.hy, p.hz);
+        if (b128) b128 += e;
+        if (b64) b64 += e;
+    }
     return VIE_OK;
 }
 
@@ -662,55 +672,29 @@ static int green_spectrum(vie_grid* g, double k0, int mask, const NearRule& near
         delete sp;
         return rc;
     };
-    std::vector<const BoxSet*> sets;
-    sets.push_back(&g->full);
-    for (auto& gr : g->groups) sets.push_back(&gr.bs);
-    {
-        // full grid: octant-compressed spectra, built from an FP64 temporary
-        const int64_t n = 6 * g->full.oct_elems();
+    // full grid: octant-compressed spectra; block groups: full layout and the parity-split one
+    auto one = [&](const BoxSet& bs, bool oct, const std::vector<ParSpec>* par) -> int {
+        const int64_t n = 6 * (oct ? bs.oct_elems() : bs.spec_elems());
         double2* G = nullptr;
         float2* G64 = nullptr;
-        int arc = VIE_OK;
-        if (mask & VIE_C128) arc = dmalloc((void**)&G, n * sizeof(double2), "vie_green_spectrum");
-        if (!arc && (mask & VIE_C64)) arc = dmalloc((void**)&G64, n * sizeof(float2), "vie_green_spectrum");
-        if (arc) {
-            dfree(G);
-            return bail(arc);
-        }
+        if (mask & VIE_C128) VIE_TRY(dmalloc((void**)&G, n * sizeof(double2), "vie_green_spectrum"));
         sp->g128.push_back(G);
+        const int rc = mask & VIE_C64 ? dmalloc((void**)&G64, n * sizeof(float2), "vie_green_spectrum") : VIE_OK;
         sp->g64.push_back(G64);
-        int rc = spectrum_build(g->full, k0, g->h, G, G64, nullptr, s, &near);
-        if (rc) return bail(rc);
-    }
-    sets.erase(sets.begin());
-    for (const BoxSet* bs : sets) {
-        const int64_t n = 6 * bs->spec_elems();
-        double2* G = nullptr;
-        int arc = dmalloc((void**)&G, n * sizeof(double2), "vie_green_spectrum");
-        if (arc) return bail(arc);
-        sp->g128.push_back(G);
-        int rc = green_sample(*bs, k0, g->h, G, s, &near);
+        if (rc) return rc;
+        SpecOut so;
+        (oct ? so.oct128 : so.full128) = G;
+        (oct ? so.oct64 : so.full64) = G64;
+        so.par = par;
+        return spectrum_build(bs, k0, g->h, so, s, &near);
+    };
+    int rc = one(g->full, true, nullptr);
+    if (rc) return bail(rc);
+    for (const Group& gr : g->groups) {
         sp->par.emplace_back();
-        if (!rc) rc = par_spectra(g->groups[sp->par.size() - 1], G, mask, sp->par.back(), s);
-        if (!rc) rc = spectrum_fft<double2>(*bs, G, s);
+        rc = alloc_par(sp, gr, mask, sp->par.back());
+        if (!rc) rc = one(gr.bs, false, &sp->par.back());
         if (rc) return bail(rc);
-        float2* G64 = nullptr;
-        if (mask & VIE_C64) {
-            if ((arc = dmalloc((void**)&G64, n * sizeof(float2), "vie_green_spectrum"))) return bail(arc);
-            if ((rc = convert_c128_to_c64(G, G64, n, s))) {
-                sp->g64.push_back(G64);
-                return bail(rc);
-            }
-        }
-        sp->g64.push_back(G64);
-    }
-    if (!(mask & VIE_C128)) {
-        // the FP64 spectrum was only the source of the complex64 copy
-        if (cudaStreamSynchronize(s) != cudaSuccess) return bail(fail(VIE_ECUDA, "spectrum generation failed"));
-        for (auto& p : sp->g128) {
-            dfree(p);
-            p = nullptr;
-        }
     }
     *out = sp;
     return VIE_OK;

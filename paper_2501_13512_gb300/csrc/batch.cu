@@ -300,8 +300,18 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
             if (!arc) {
                 BoxSet one = bs;
                 one.nb = 1;
-                arc = spectrum_build(one, k0s[i], b->h, g.g128, par ? nullptr : g.g64, g.full64, s, nullptr,
-                                     par ? g.g64 : nullptr);
+                SpecOut so;
+                std::vector<ParSpec> ps(par ? 1 : 0);
+                so.oct128 = g.g128;
+                so.full64 = g.full64;
+                if (par) {
+                    ps[0].hx = hx; ps[0].hy = hy; ps[0].hz = hz;
+                    ps[0].g64 = g.g64;
+                    so.par = &ps;
+                } else {
+                    so.oct64 = g.g64;
+                }
+                arc = spectrum_build(one, k0s[i], b->h, so, s);
                 if (arc) cudaStreamSynchronize(s);
             }
             if (arc) {

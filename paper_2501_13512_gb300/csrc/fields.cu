@@ -53,7 +53,32 @@ __device__ __forceinline__ void add_k2G(double rx, double ry, double rz, double 
 // (1 / (Mx My Mz), the inverse-FFT normalisation folded into the spectrum);
 // offsets with 0 < max|D| <= near.radius take the mean of k0^2 G over the cube
 // of side h around D h instead (tensor Gauss-Legendre rule of order near.q).
-// Output: natural order [6][Mz][My][Mx], components xx, xy, xz, yy, yz, zz.
+// Components xx, xy, xz, yy, yz, zz.
+__device__ __forceinline__ void green_entry(int dx, int dy, int dz, double k0, double h, double scale, double2 self,
+                                            const NearRule& near, double2 (&K)[6]) {
+    for (int c = 0; c < 6; ++c) K[c] = make_double2(0.0, 0.0);
+    if (dx == 0 && dy == 0 && dz == 0) {
+        const double2 sd = make_double2(self.x * scale, self.y * scale);
+        K[0] = sd;
+        K[3] = sd;
+        K[5] = sd;
+        return;
+    }
+    const double hs = h * h * h * scale;
+    const int dmax = max(abs(dx), max(abs(dy), abs(dz)));
+    if (dmax <= near.radius) {
+        // mean over the cube: weights w_i w_j w_l / 8 of the rule on [-1, 1]^3
+        for (int l = 0; l < near.q; ++l)
+            for (int j = 0; j < near.q; ++j)
+                for (int i = 0; i < near.q; ++i)
+                    add_k2G((dx + 0.5 * near.t[i]) * h, (dy + 0.5 * near.t[j]) * h, (dz + 0.5 * near.t[l]) * h, k0, hs,
+                            0.125 * near.w[i] * near.w[j] * near.w[l], K);
+    } else {
+        add_k2G(dx * h, dy * h, dz * h, k0, hs, 1.0, K);
+    }
+}
+
+// Natural order [6][Mz][My][Mx], zero at offsets that no product uses.
 __global__ void k_green_sample(double2* G, int Mx, int My, int Mz, int bx, int by, int bz,
                                double k0, double h, double scale, double2 self, NearRule near) {
     const int64_t vol = (int64_t)Mx * My * Mz;
@@ -65,29 +90,20 @@ __global__ void k_green_sample(double2* G, int Mx, int My, int Mz, int bx, int b
         int dx, dy, dz;
         double2 K[6];
         for (int c = 0; c < 6; ++c) K[c] = make_double2(0.0, 0.0);
-        bool used = wrap_offset(ix, Mx, bx, dx) & wrap_offset(iy, My, by, dy) & wrap_offset(iz, Mz, bz, dz);
-        if (used) {
-            if (dx == 0 && dy == 0 && dz == 0) {
-                double2 sd = make_double2(self.x * scale, self.y * scale);
-                K[0] = sd;
-                K[3] = sd;
-                K[5] = sd;
-            } else {
-                const double hs = h * h * h * scale;
-                const int dmax = max(abs(dx), max(abs(dy), abs(dz)));
-                if (dmax <= near.radius) {
-                    // mean over the cube: weights w_i w_j w_l / 8 of the rule on [-1, 1]^3
-                    for (int l = 0; l < near.q; ++l)
-                        for (int j = 0; j < near.q; ++j)
-                            for (int i = 0; i < near.q; ++i)
-                                add_k2G((dx + 0.5 * near.t[i]) * h, (dy + 0.5 * near.t[j]) * h,
-                                        (dz + 0.5 * near.t[l]) * h, k0, hs,
-                                        0.125 * near.w[i] * near.w[j] * near.w[l], K);
-                } else {
-                    add_k2G(dx * h, dy * h, dz * h, k0, hs, 1.0, K);
-                }
-            }
-        }
+        if (wrap_offset(ix, Mx, bx, dx) & wrap_offset(iy, My, by, dy) & wrap_offset(iz, Mz, bz, dz))
+            green_entry(dx, dy, dz, k0, h, scale, self, near, K);
+        for (int c = 0; c < 6; ++c) G[c * vol + idx] = K[c];
+    }
+}
+
+// The octant of non-negative offsets alone, [6][bz][by][bx]: every component is even or odd along each axis.
+__global__ void k_green_octant(double2* G, int bx, int by, int bz, double k0, double h, double scale, double2 self,
+                               NearRule near) {
+    const int64_t vol = (int64_t)bx * by * bz;
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < vol;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        double2 K[6];
+        green_entry((int)(idx % bx), (int)((idx / bx) % by), (int)(idx / ((int64_t)bx * by)), k0, h, scale, self, near, K);
         for (int c = 0; c < 6; ++c) G[c * vol + idx] = K[c];
     }
 }
@@ -137,18 +153,30 @@ int near_rule(int radius, int q, NearRule* out) {
     return VIE_OK;
 }
 
-int green_sample(const BoxSet& bs, double k0, double h, double2* G, cudaStream_t s, const NearRule* near) {
-    // equivalent-sphere self term: (2/3)[(1 + jka) e^{-jka} - 1] - 1/3
-    const double a = h * cbrt(3.0 / (4.0 * 3.14159265358979323846));
-    const double ka = k0 * a;
+// equivalent-sphere self term: (2/3)[(1 + jka) e^{-jka} - 1] - 1/3
+static double2 self_term(double k0, double h) {
+    const double ka = k0 * h * cbrt(3.0 / (4.0 * 3.14159265358979323846));
     const double c = cos(ka), sn = sin(ka);
     // (1 + j ka)(c - j sn) = c + ka sn + j (ka c - sn)
-    double2 self = make_double2((2.0 / 3.0) * (c + ka * sn - 1.0) - 1.0 / 3.0, (2.0 / 3.0) * (ka * c - sn));
+    return make_double2((2.0 / 3.0) * (c + ka * sn - 1.0) - 1.0 / 3.0, (2.0 / 3.0) * (ka * c - sn));
+}
+
+int green_sample(const BoxSet& bs, double k0, double h, double2* G, cudaStream_t s, const NearRule* near) {
     const double scale = 1.0 / ((double)bs.Mx * bs.My * bs.Mz);
     prof_begin(s, PK_SPECTRUM, VIE_C128, 0, 6 * bs.spec_elems() * 16, false);
     const NearRule rule = near ? *near : NearRule();
     k_green_sample<<<grid_1d(bs.spec_elems()), 256, 0, s>>>(G, bs.Mx, bs.My, bs.Mz, bs.bx, bs.by, bs.bz,
-                                                            k0, h, scale, self, rule);
+                                                            k0, h, scale, self_term(k0, h), rule);
+    prof_end(s);
+    VIE_CK(cudaGetLastError());
+    return VIE_OK;
+}
+
+int green_octant(const BoxSet& bs, double k0, double h, double2* G, cudaStream_t s, const NearRule* near) {
+    const double scale = 1.0 / ((double)bs.Mx * bs.My * bs.Mz);
+    prof_begin(s, PK_SPECTRUM, VIE_C128, 0, 6 * bs.box_elems() * 16, false);
+    const NearRule rule = near ? *near : NearRule();
+    k_green_octant<<<grid_1d(bs.box_elems()), 256, 0, s>>>(G, bs.bx, bs.by, bs.bz, k0, h, scale, self_term(k0, h), rule);
     prof_end(s);
     VIE_CK(cudaGetLastError());
     return VIE_OK;

@@ -727,13 +727,20 @@ template int inner_persistent<float2>(const std::vector<InnerJob<float2>>&, cons
 // array); 1: y; 2: z, into the layout of the block solver.
 struct ParAxis {
     int hx, hy, hz;          // transform lengths
-    int n, ny, nz;           // offsets of this axis; of y and z (rows beyond them are never read)
-    int64_t sy, sz, sc;      // strides of K (AXIS 0)
-    double scale;            // AXIS 0: normalisation of the inverse transforms over that of K
+    int nx, ny, nz;          // offsets of each axis (rows beyond them are never read)
+    double scale;            // normalisation of the inverse transforms over that of K
+    int64_t t1, t2;          // first element of this spectrum in the temporaries of pass x and y
+    double2* o128;
+    float2* o64;
+};
+constexpr int kParSetMax = 27;   // lengths 10, 12 or 16 on each axis
+struct ParAxisSet {
+    ParAxis a[kParSetMax];
 };
 template <int AXIS>
-__global__ void k_par_axis(const double2* __restrict__ in, double2* out, double2* o128, float2* o64, ParAxis a) {
-    const int H = AXIS == 0 ? a.hx : AXIS == 1 ? a.hy : a.hz;
+__global__ void k_par_axis(const double2* __restrict__ in, double2* out, int64_t sy, int64_t sz, int64_t sc, ParAxisSet set) {
+    const ParAxis a = set.a[blockIdx.y];
+    const int H = AXIS == 0 ? a.hx : AXIS == 1 ? a.hy : a.hz, na = AXIS == 0 ? a.nx : AXIS == 1 ? a.ny : a.nz;
     __shared__ double2 tw[32];                      // exp(-i pi j / H), j < 2H
     if ((int)threadIdx.x < 2 * H) {
         double sn, cs;
@@ -741,6 +748,8 @@ __global__ void k_par_axis(const double2* __restrict__ in, double2* out, double2
         tw[threadIdx.x] = make_double2(cs, -sn);
     }
     __syncthreads();
+    if (AXIS > 0) in += AXIS == 1 ? a.t1 : a.t2;
+    if (AXIS < 2) out += AXIS == 0 ? a.t1 : a.t2;
     const int nx = a.hx + 1, ny = AXIS == 0 ? a.hy : a.hy + 1, nz = AXIS == 2 ? a.hz + 1 : a.hz;
     const int total = 6 * nz * ny * nx;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
@@ -750,11 +759,11 @@ __global__ void k_par_axis(const double2* __restrict__ in, double2* out, double2
         const int f = AXIS == 0 ? fx : AXIS == 1 ? y : z;
         const double2* p;
         int64_t st;
-        if (AXIS == 0) { p = in + c * a.sc + z * a.sz + y * a.sy; st = 1; }
+        if (AXIS == 0) { p = in + c * sc + z * sz + y * sy; st = 1; }
         else if (AXIS == 1) { p = in + ((int64_t)(c * a.hz + z) * a.hy) * nx + fx; st = nx; }
         else { p = in + ((int64_t)c * a.hz * ny + y) * nx + fx; st = (int64_t)ny * nx; }
         double2 s = odd ? make_double2(0.0, 0.0) : p[0];
-        for (int d = 1; d < a.n; ++d) {
+        for (int d = 1; d < na; ++d) {
             const double2 w = tw[(f * d) % (2 * H)], k = p[d * st];
             // even: 2 K cos; odd: -2i K sin (w.y = -sin)
             if (odd) s = make_double2(s.x - 2.0 * w.y * k.y, s.y + 2.0 * w.y * k.x);
@@ -768,39 +777,48 @@ __global__ void k_par_axis(const double2* __restrict__ in, double2* out, double2
             const int pz = z & 1, py = y & 1, iz = z >> 1, iy = y >> 1;
             const int my = a.hy / 2 + 1, mz = a.hz / 2 + 1;
             const int64_t o = ((((int64_t)(2 * pz + py) * nx + fx) * 6 + c) * mz + iz) * my + iy;
-            if (o128) o128[o] = s;
-            if (o64) o64[o] = make_float2((float)s.x, (float)s.y);
+            if (a.o128) a.o128[o] = s;
+            if (a.o64) a.o64[o] = make_float2((float)s.x, (float)s.y);
         }
     }
 }
 
 int64_t par_spectrum_elems(int hx, int hy, int hz) { return 4LL * (hx + 1) * 6 * (hz / 2 + 1) * (hy / 2 + 1); }
 
-// K: lattice samples of the box set's shape (green_sample: natural order [6][Mz][My][Mx], scaled by
-// 1 / (Mx My Mz)); the spectrum of transform lengths (hx, hy, hz) into g128 and / or g64.
-int par_spectrum(const BoxSet& bs, const double2* K, int hx, int hy, int hz, double2* g128, float2* g64, cudaStream_t s) {
-    const int64_t n1 = 6LL * hz * hy * (hx + 1), n2 = 6LL * hz * (hy + 1) * (hx + 1);
+// K: lattice samples of the box set's shape (green_octant: [6][bz][by][bx], scaled by 1 / (Mx My Mz)); fills
+// the spectra of `out`, all of them in one launch per axis.
+int par_spectra(const BoxSet& bs, const double2* K, const std::vector<ParSpec>& out, cudaStream_t s) {
+    if (out.empty()) return VIE_OK;
+    if ((int)out.size() > kParSetMax) return fail(VIE_EINVAL, "par_spectra: too many classes");
+    ParAxisSet set{};
+    int64_t n1 = 0, n2 = 0, m1 = 0, m2 = 0, m3 = 0;
+    for (size_t k = 0; k < out.size(); ++k) {
+        const ParSpec& p = out[k];
+        ParAxis& a = set.a[k];
+        a.hx = p.hx; a.hy = p.hy; a.hz = p.hz;
+        a.nx = std::min(p.hx, bs.bx); a.ny = std::min(p.hy, bs.by); a.nz = std::min(p.hz, bs.bz);
+        a.scale = (double)bs.spec_elems() / (8.0 * p.hx * p.hy * p.hz);
+        a.t1 = n1; a.t2 = n2;
+        a.o128 = p.g128; a.o64 = p.g64;
+        const int64_t e1 = 6LL * p.hz * p.hy * (p.hx + 1), e2 = 6LL * p.hz * (p.hy + 1) * (p.hx + 1);
+        n1 += e1;
+        n2 += e2;
+        m1 = std::max(m1, e1);
+        m2 = std::max(m2, e2);
+        m3 = std::max<int64_t>(m3, 6LL * (p.hz + 1) * (p.hy + 1) * (p.hx + 1));
+    }
     double2* tmp = nullptr;
     VIE_CK(cudaMallocAsync((void**)&tmp, (n1 + n2) * sizeof(double2), s));
-    ParAxis a{};
-    a.hx = hx; a.hy = hy; a.hz = hz;
-    a.sy = bs.Mx; a.sz = (int64_t)bs.Mx * bs.My; a.sc = bs.spec_elems();
-    a.scale = (double)bs.spec_elems() / (8.0 * hx * hy * hz);
-    auto blocks = [](int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, 152 * 8)); };
-    const int64_t es = sizeof(double2), n3 = 6LL * (hz + 1) * (hy + 1) * (hx + 1);
-    a.n = std::min(hx, bs.bx);
-    a.ny = std::min(hy, bs.by);
-    a.nz = std::min(hz, bs.bz);
+    const int64_t es = sizeof(double2), sy = bs.bx, sz = (int64_t)bs.bx * bs.by, sc = bs.box_elems();
+    auto grid = [&](int64_t n) { return dim3((unsigned)((n + 127) / 128), (unsigned)out.size()); };
     prof_begin(s, PK_SPECTRUM, VIE_C128, 0, 2 * n1 * es, false);
-    k_par_axis<0><<<blocks(n1), 128, 0, s>>>(K, tmp, nullptr, nullptr, a);
+    k_par_axis<0><<<grid(m1), 128, 0, s>>>(K, tmp, sy, sz, sc, set);
     prof_end(s);
-    a.n = a.ny;
     prof_begin(s, PK_SPECTRUM, VIE_C128, 0, 2 * n2 * es, false);
-    k_par_axis<1><<<blocks(n2), 128, 0, s>>>(tmp, tmp + n1, nullptr, nullptr, a);
+    k_par_axis<1><<<grid(m2), 128, 0, s>>>(tmp, tmp + n1, sy, sz, sc, set);
     prof_end(s);
-    a.n = a.nz;
-    prof_begin(s, PK_SPECTRUM, VIE_C128, 0, (n2 + n3) * es, false);
-    k_par_axis<2><<<blocks(n3), 128, 0, s>>>(tmp + n1, nullptr, g128, g64, a);
+    prof_begin(s, PK_SPECTRUM, VIE_C128, 0, 2 * n2 * es, false);
+    k_par_axis<2><<<grid(m3), 128, 0, s>>>(tmp + n1, nullptr, sy, sz, sc, set);
     prof_end(s);
     const cudaError_t le = cudaGetLastError(), e = cudaFreeAsync(tmp, s);
     if (le != cudaSuccess) return cuda_fail(le, "k_par_axis launch", __FILE__, __LINE__);

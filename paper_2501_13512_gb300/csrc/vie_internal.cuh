@@ -238,6 +238,7 @@ struct vie_spectrum {
     // index g: spectra of group g for the parity-split MVM: the lengths of the group's box first (they
     // serve every block of the group), then those of its smaller classes
     std::vector<std::vector<vie::ParSpec>> par;
+    std::vector<void*> par_alloc;         // their device memory
 };
 
 struct vie_grid {
@@ -316,9 +317,10 @@ int mvm_boxes(const BoxSet& bs, const C* G, const C* x, C* y, const SegState* st
 template <class C>
 int spectrum_fft(const BoxSet& bs, C* G, cudaStream_t s, const Twiddles* tw = nullptr,
                  int ncomp = 6);   // in place, ncomp components
-// Green spectrum of one box shape at wavenumber k0 (FP64 samples and FFT in a
-// stream-ordered temporary), written to any of: oct128 / oct64 (octant
-// layout [6][Mz/2+1][My/2+1][Mx/2+1]), full64 (full layout [6][Mz][My][Mx]).
+// Green spectrum of one box shape at wavenumber k0: FP64 samples of the octant of non-negative offsets and
+// its transform to the octant of non-negative frequencies (every component is even or odd along every axis),
+// in stream-ordered temporaries, written to any of the layouts of SpecOut: octant
+// [6][Mz/2+1][My/2+1][Mx/2+1], full [6][Mz][My][Mx] (both in bit-reversed order), parity-split.
 // Cube-integrated near-neighbour entries (an accuracy variant; the paper does not say how
 // near couplings are integrated): K(D) = mean over the cube of side h centred at D h of
 // k0^2 G, times h^3, for 0 < max|D| <= radius, by tensor Gauss-Legendre quadrature of order q.
@@ -329,12 +331,19 @@ struct NearRule {
     double t[kNearMaxOrder], w[kNearMaxOrder];   // nodes and weights on [-1, 1]
 };
 int near_rule(int radius, int q, NearRule* out);   // VIE_EINVAL outside radius [0, 8], q [1, 16]
-// or par64 (parity-split layout of the lengths holding the box, par_spectrum).
-int spectrum_build(const BoxSet& bs, double k0, double h, double2* oct128, float2* oct64, float2* full64,
-                   cudaStream_t s, const NearRule* near = nullptr, float2* par64 = nullptr);
+// Any of them may be null; `par`: spectra of the parity-split MVM to fill (allocated).
+struct SpecOut {
+    double2* oct128 = nullptr;
+    float2* oct64 = nullptr;
+    double2* full128 = nullptr;
+    float2* full64 = nullptr;
+    const std::vector<ParSpec>* par = nullptr;
+};
+int spectrum_build(const BoxSet& bs, double k0, double h, const SpecOut& out, cudaStream_t s, const NearRule* near = nullptr);
 
 // ---------------------------------------------------------------- green.cu
 int green_sample(const BoxSet& bs, double k0, double h, double2* G, cudaStream_t s, const NearRule* near = nullptr);
+int green_octant(const BoxSet& bs, double k0, double h, double2* G, cudaStream_t s, const NearRule* near = nullptr);   // [6][bz][by][bx]
 int convert_c128_to_c64(const double2* a, float2* b, int64_t n, cudaStream_t s);
 // Bistatic RCS of sum_j wts_j E_j h^3 exp(j k0 u . r_j) over voxel centres r_j, component c shifted by
 // shift[c] along its own axis (shift may be null). Synchronises s.
@@ -386,12 +395,12 @@ template <class C> struct InnerJob {
 };
 bool inner_persistent_ok(const BoxSet& bs, size_t es, bool force);
 // Parity-split MVM (inner_parity.cuh): smallest transform length holding b voxels (0: none), whether a
-// box set takes it, and its spectra from the lattice samples K of green_sample.
+// box set takes it, and its spectra from the lattice samples K of green_octant.
 int par_len(int b);
 int par_least(int h);                   // smallest extent that takes length h
 bool par_path_ok(const BoxSet& bs);
 int64_t par_spectrum_elems(int hx, int hy, int hz);
-int par_spectrum(const BoxSet& bs, const double2* K, int hx, int hy, int hz, double2* g128, float2* g64, cudaStream_t s);
+int par_spectra(const BoxSet& bs, const double2* K, const std::vector<ParSpec>& out, cudaStream_t s);
 size_t inner_group_desc_bytes();
 // cluster: CTAs per block (1, 2, 4, 8; 0 = 2) of launches without parity-split jobs (those take 4),
 // unless VIE_INNER_CLUSTER forces one.
