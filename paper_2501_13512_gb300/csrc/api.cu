@@ -976,10 +976,9 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
     std::vector<int> batched;
     const bool merged = mm != nullptr && mm->live;
     bool any_fit = false;
+    VIE_TRY(precond_gather<C>(g, b, s));
     for (int i = 0; i < ng; ++i) {
         Group& gr = g->groups[i];
-        KrylovVecs<C>& v = group_vecs<C>(gr);
-        VIE_TRY(precond_gather<C>(g, gr, b, v.b, s));
         // in a session, blocks that fit go to the merged launch; the rest run as they would alone
         if (merged && gr.fit[c128 ? 0 : 1]) any_fit = true;
         else if (c128 ? gr.persistent128 : gr.persistent64) group_jobs<C>(g, sp, i, jobs);
@@ -1088,8 +1087,7 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
         guard.armed = false;
         VIE_TRY(merge_wait(mm, &req, s));
     }
-    VIE_TRY(precond_copy_unblocked<C>(g, b, y, s));
-    for (int i = 0; i < ng; ++i) VIE_TRY(precond_scatter_group<C>(g, g->groups[i], group_vecs<C>(g->groups[i]).x, y, s));
+    VIE_TRY(precond_scatter<C>(g, b, y, s));
     std::vector<int2>& wh = g->work_host[c128 ? 0 : 1];
     const bool reorder = !jobs.empty() && wh.size() > 1;
     if (stats || reorder || merged) {

@@ -55,6 +55,7 @@ template <class C> struct RowArgs {
 
 template <class C, int MODE>
 __global__ void __launch_bounds__(kThreads) k_rows(RowArgs<C> a) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     const int TR = 1 << a.ltr;
@@ -124,6 +125,7 @@ template <class C> struct ColArgs {
 
 template <class C, bool FWD>
 __global__ void __launch_bounds__(kThreads) k_cols(ColArgs<C> a) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     const int TC = 1 << a.ltc;
@@ -167,6 +169,7 @@ template <class C> struct ZArgs {
 
 template <class C>
 __global__ void __launch_bounds__(kThreads) k_zgreen(ZArgs<C> a) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     const int TC = 1 << a.ltc;
@@ -245,6 +248,7 @@ constexpr int kZRegThreads = 3 * kZRegCols;
 
 template <int LZ>
 __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
+    pdl_wait();
     typedef float2 F;
     constexpr int H = LZ / 2 > 0 ? LZ / 2 : 1;
     constexpr int LGZ = ILog2<LZ>::v;
@@ -442,6 +446,7 @@ __device__ __forceinline__ void z_parity(const ZArgs<C>& a, const ZColumn<C, OCT
 
 template <class C, int H, bool OCT>
 __global__ void __launch_bounds__(2 * kZPairCols, 2) k_z_pair(ZArgs<C> a) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* sm = reinterpret_cast<C*>(smem_raw);      // [3 H][kZPairCols]: the odd parity's results
     const int b = blockIdx.y;
@@ -490,6 +495,7 @@ template <class C, int A, int B> struct ZFour {
 
 template <class C, int A, int B, bool OCT>
 __global__ void __launch_bounds__((ZFour<C, A, B>::threads), (ZFour<C, A, B>::ctas)) k_z_four(ZArgs<C> a) {
+    pdl_wait();
     constexpr int L = A * B, HA = A / 2, NC = ZFour<C, A, B>::NC, TS = kLmax / A, LG = ILog2<L>::v;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* sm = reinterpret_cast<C*>(smem_raw);      // [3][k1 B + n2][NC]
@@ -643,6 +649,7 @@ constexpr int kRows4 = 8;   // rows per CTA (256 threads: 8 rows x 32)
 // Pass X forward: rows of bx -> chi * x, zero-padded to L = 32 A, forward transform.
 template <int A>
 __global__ void __launch_bounds__(256) k_rows4_fwd(RowArgs<float2> a) {
+    pdl_wait();
     constexpr int L = kB4 * A, LP = L + L / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* sm = reinterpret_cast<float2*>(smem_raw);     // [kRows4][LP]
@@ -696,6 +703,7 @@ __global__ void __launch_bounds__(256) k_rows4_fwd(RowArgs<float2> a) {
 // Pass X inverse: rows of L = 32 A spectrum positions -> keep x < bx, y = mask (x - u).
 template <int A>
 __global__ void __launch_bounds__(256) k_rows4_inv(RowArgs<float2> a) {
+    pdl_wait();
     constexpr int L = kB4 * A, LP = L + L / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* sm = reinterpret_cast<float2*>(smem_raw);     // [kRows4][LP]
@@ -750,6 +758,7 @@ constexpr int kCols4 = 16;   // columns per CTA (512 threads: 16 columns x 32)
 // Pass Y (forward or inverse) over columns of L = 32 A, 16 adjacent columns per CTA.
 template <int A, bool FWD>
 __global__ void __launch_bounds__(512) k_cols4(ColArgs<float2> a) {
+    pdl_wait();
     constexpr int L = kB4 * A;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* sm = reinterpret_cast<float2*>(smem_raw);     // [L][kCols4]
@@ -850,9 +859,9 @@ static int launch_rows4(RowArgs<float2> a, Prof pf, cudaStream_t s) {
     const int64_t grid = (a.nrows + kRows4 - 1) / kRows4;
     if (grid <= 0) return VIE_OK;
     a.units = prof_begin(s, pf.kind, VIE_C64, pf.bpu, pf.fixed, true);
-    kern<<<(unsigned)grid, 256, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(kern, dim3((unsigned)grid), 256, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -875,9 +884,9 @@ static int launch_line_rows(RowArgs<C> a, Prof pf, cudaStream_t s) {
     const int64_t grid = (a.nrows + NR - 1) / NR;
     if (grid <= 0) return VIE_OK;
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_line_rows<C, A, B, FWD><<<(unsigned)grid, kLineThreadsRow, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_line_rows<C, A, B, FWD>, dim3((unsigned)grid), kLineThreadsRow, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -888,9 +897,9 @@ static int launch_line_cols(ColArgs<C> a, int nb1, int nb2, Prof pf, cudaStream_
     VIE_TRY(prep_smem(k_line_cols<C, A, B, FWD>, smem));
     dim3 grid((a.ncols + NC - 1) / NC, nb1, nb2);
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_line_cols<C, A, B, FWD><<<grid, line_threads_col<C>(), smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_line_cols<C, A, B, FWD>, grid, line_threads_col<C>(), smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -921,9 +930,9 @@ static int launch_rows(RowArgs<C> a, Prof pf, cudaStream_t s) {
     int64_t grid = (a.nrows + TR - 1) / TR;
     if (grid <= 0) return VIE_OK;
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_rows<C, MODE><<<(unsigned)grid, kThreads, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_rows<C, MODE>, dim3((unsigned)grid), kThreads, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -933,9 +942,9 @@ static int launch_cols4(ColArgs<float2> a, int nb1, int nb2, Prof pf, cudaStream
     VIE_TRY(prep_smem(k_cols4<A, FWD>, smem));
     dim3 grid((a.ncols + kCols4 - 1) / kCols4, nb1, nb2);
     a.units = prof_begin(s, pf.kind, VIE_C64, pf.bpu, pf.fixed, true);
-    k_cols4<A, FWD><<<grid, kB4 * kCols4, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_cols4<A, FWD>, grid, kB4 * kCols4, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -961,9 +970,9 @@ static int launch_cols(ColArgs<C> a, int nb1, int nb2, Prof pf, cudaStream_t s) 
     VIE_TRY(prep_smem(k_cols<C, FWD>, smem));
     dim3 grid((a.ncols + TC - 1) / TC, nb1, nb2);
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_cols<C, FWD><<<grid, kThreads, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_cols<C, FWD>, grid, kThreads, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -973,9 +982,9 @@ static int launch_zgreen_reg(ZArgs<float2> a, int nb, Prof pf, cudaStream_t s) {
     VIE_TRY(prep_smem(k_zgreen_reg<LZ>, smem));
     dim3 grid((a.ncols + kZRegCols - 1) / kZRegCols, nb);
     a.units = prof_begin(s, pf.kind, VIE_C64, pf.bpu, pf.fixed, true);
-    k_zgreen_reg<LZ><<<grid, kZRegThreads, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_zgreen_reg<LZ>, grid, kZRegThreads, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -985,9 +994,9 @@ static int launch_z_pair(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
     VIE_TRY(prep_smem(k_z_pair<C, H, OCT>, smem));
     dim3 grid((a.ncols + kZPairCols - 1) / kZPairCols, nb);
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_z_pair<C, H, OCT><<<grid, 2 * kZPairCols, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_z_pair<C, H, OCT>, grid, 2 * kZPairCols, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -997,9 +1006,9 @@ static int launch_z_four(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
     VIE_TRY(prep_smem(k_z_four<C, A, B, OCT>, Z::smem));
     dim3 grid((a.ncols + Z::NC - 1) / Z::NC, nb);
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_z_four<C, A, B, OCT><<<grid, Z::threads, Z::smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_z_four<C, A, B, OCT>, grid, Z::threads, Z::smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -1047,9 +1056,9 @@ static int launch_zgreen(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
     VIE_TRY(prep_smem(k_zgreen<C>, smem));
     dim3 grid((a.ncols + TC - 1) / TC, nb);
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_zgreen<C><<<grid, kThreads, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_zgreen<C>, grid, kThreads, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 
@@ -1058,9 +1067,9 @@ static int launch_plane(PlaneArgs<C> a, int nplanes, Prof pf, cudaStream_t s) {
     const size_t smem = (size_t)a.pitch * ((size_t)1 << a.ly) * sizeof(C);
     VIE_TRY(prep_smem(k_plane<C, FWD>, smem));
     a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
-    k_plane<C, FWD><<<nplanes, a.lx + a.ly <= 10 ? 128 : a.lx + a.ly <= 12 ? 256 : 512, smem, s>>>(a);
+    const cudaError_t e = launch_dependent(k_plane<C, FWD>, dim3((unsigned)nplanes), a.lx + a.ly <= 10 ? 128 : a.lx + a.ly <= 12 ? 256 : 512, smem, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 

@@ -202,6 +202,7 @@ template <int A, int B, class C> __device__ __forceinline__ void plane_cols_inv(
 
 template <class C, bool FWD>
 __global__ void __launch_bounds__(512) k_plane(PlaneArgs<C> a) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* sm = reinterpret_cast<C*>(smem_raw);          // [My][pitch]
     const int pl = blockIdx.x, b = pl / (3 * a.bz), z = pl % a.bz;
@@ -234,6 +235,7 @@ template <class C> struct LineCols { static constexpr int n = sizeof(C) == 8 ? 1
 
 template <class C, int A, int B, bool FWD>
 __global__ void __launch_bounds__(kLineThreadsRow) k_line_rows(RowArgs<C> a) {
+    pdl_wait();
     constexpr int L = A * B, NR = LineRows<L>::n, P = L + L / 8 + 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* sm = reinterpret_cast<C*>(smem_raw);          // [NR][P]
@@ -304,6 +306,7 @@ __global__ void __launch_bounds__(kLineThreadsRow) k_line_rows(RowArgs<C> a) {
 
 template <class C, int A, int B, bool FWD>
 __global__ void __launch_bounds__(line_threads_col<C>()) k_line_cols(ColArgs<C> a) {
+    pdl_wait();
     constexpr int NC = LineCols<C>::n;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* sm = reinterpret_cast<C*>(smem_raw);          // [L][NC]

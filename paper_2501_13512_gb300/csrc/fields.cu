@@ -229,98 +229,116 @@ int plane_wave_launch(const vie_grid* g, double k0, const double* khat, const do
 }
 
 // ---------------------------------------------------------------- block restriction / prolongation
-// b_k = b restricted to the voxels S_k of block k, laid out in the block's box
-// [nb][3][bz][by][bx]; zero outside S_k.
+// Groups of blocks of one launch, their box elements numbered one after another from first[i].
+constexpr int kBlockTabMax = 16;
+template <class C> struct BlockTab {
+    int n, nx, ny, nz;
+    int64_t first[kBlockTabMax + 1];
+    C* vec[kBlockTabMax];                 // b (gather) or x (scatter) of the group, [nb][3][bz][by][bx]
+    const uint8_t* mask[kBlockTabMax];
+    const int32_t* origin[kBlockTabMax];
+    int bx[kBlockTabMax], by[kBlockTabMax], bz[kBlockTabMax];
+};
+
+// Element idx of the table: its group i, index j in the group's vectors, mask value and place in the grid.
 template <class C>
-__global__ void k_gather(const C* src, C* out, const uint8_t* mask, const int32_t* origin,
-                         int nb, int bx, int by, int bz, int nx, int ny, int nz) {
-    const int64_t box = (int64_t)bx * by * bz;
-    const int64_t total = (int64_t)nb * 3 * box;
-    const int64_t N = (int64_t)nx * ny * nz;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+__device__ __forceinline__ uint8_t block_elem(const BlockTab<C>& t, int64_t idx, int& i, int64_t& j, int64_t& place) {
+    i = 0;
+    while (i + 1 < t.n && idx >= t.first[i + 1]) ++i;
+    j = idx - t.first[i];
+    const int bx = t.bx[i], by = t.by[i];
+    const int64_t box = (int64_t)bx * by * t.bz[i], bc = j / box;
+    const int l = (int)(j - bc * box), c = (int)(bc % 3), b = (int)(bc / 3);
+    const uint8_t m = t.mask[i][b * box + l];
+    const int32_t* o = t.origin[i] + 3 * b;
+    place = c * ((int64_t)t.nx * t.ny * t.nz) +
+            ((int64_t)(o[2] + l / (bx * by)) * t.ny + o[1] + (l / bx) % by) * t.nx + o[0] + l % bx;
+    return m;
+}
+
+// b_k = b restricted to the voxels S_k of block k; zero outside S_k.
+template <class C> __global__ void k_gather(const C* src, BlockTab<C> t) {
+    pdl_wait();
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < t.first[t.n];
          idx += (int64_t)gridDim.x * blockDim.x) {
-        int64_t l = idx % box;
-        int64_t bc = idx / box;
-        int c = (int)(bc % 3), b = (int)(bc / 3);
-        C v = czero<C>();
-        if (mask[(int64_t)b * box + l]) {
-            int lx = (int)(l % bx), ly = (int)((l / bx) % by), lz = (int)(l / ((int64_t)bx * by));
-            int gx = origin[3 * b] + lx, gy = origin[3 * b + 1] + ly, gz = origin[3 * b + 2] + lz;
-            v = src[c * N + ((int64_t)gz * ny + gy) * nx + gx];
-        }
-        out[idx] = v;
+        int i;
+        int64_t j, p;
+        const uint8_t m = block_elem(t, idx, i, j, p);
+        t.vec[i][j] = m ? src[p] : czero<C>();
     }
 }
 
 // y = x_k on the voxels of block k (mask 1; the blocks are disjoint, so no write conflicts). Halo
 // voxels of an expanded block (mask 2) belong to another block or to none and are not written.
-template <class C>
-__global__ void k_scatter(const C* xk, C* y, const uint8_t* mask, const int32_t* origin,
-                          int nb, int bx, int by, int bz, int nx, int ny, int nz) {
-    const int64_t box = (int64_t)bx * by * bz;
-    const int64_t total = (int64_t)nb * 3 * box;
-    const int64_t N = (int64_t)nx * ny * nz;
+// y = b on voxels that belong to no block (identity part of K2), when block_id is given.
+template <class C> __global__ void k_scatter(C* y, BlockTab<C> t, const C* b, const int32_t* block_id) {
+    pdl_wait();
+    const int64_t N = (int64_t)t.nx * t.ny * t.nz, total = t.first[t.n] + (block_id ? N : 0);
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        int64_t l = idx % box;
-        int64_t bc = idx / box;
-        int c = (int)(bc % 3), b = (int)(bc / 3);
-        if (mask[(int64_t)b * box + l] != 1) continue;
-        int lx = (int)(l % bx), ly = (int)((l / bx) % by), lz = (int)(l / ((int64_t)bx * by));
-        int gx = origin[3 * b] + lx, gy = origin[3 * b + 1] + ly, gz = origin[3 * b + 2] + lz;
-        y[c * N + ((int64_t)gz * ny + gy) * nx + gx] = xk[idx];
-    }
-}
-
-// y = b on voxels that belong to no block (identity part of K2).
-template <class C>
-__global__ void k_copy_unblocked(const C* b, C* y, const int32_t* block_id, int64_t N) {
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        if (block_id[idx] < 0) {
-            y[idx] = b[idx];
-            y[N + idx] = b[N + idx];
-            y[2 * N + idx] = b[2 * N + idx];
+        if (idx < t.first[t.n]) {
+            int i;
+            int64_t j, p;
+            if (block_elem(t, idx, i, j, p) == 1) y[p] = t.vec[i][j];
+        } else {
+            const int64_t v = idx - t.first[t.n];
+            if (block_id[v] < 0) {
+                y[v] = b[v];
+                y[N + v] = b[N + v];
+                y[2 * N + v] = b[2 * N + v];
+            }
         }
     }
 }
 
-template <class C>
-int precond_gather(const vie_grid* g, const Group& gr, const C* b, C* out, cudaStream_t s) {
-    const BoxSet& bs = gr.bs;
-    prof_begin(s, PK_FIELD, sizeof(C) == 16 ? VIE_C128 : VIE_C64, 0, 2 * bs.nb * bs.vec_elems() * (int64_t)sizeof(C), false);
-    k_gather<C><<<grid_1d(bs.nb * bs.vec_elems()), 256, 0, s>>>(b, out, bs.mask, bs.origin, bs.nb, bs.bx, bs.by,
-                                                                bs.bz, g->nx, g->ny, g->nz);
-    prof_end(s);
-    VIE_CK(cudaGetLastError());
+template <class C> static KrylovVecs<C>& vecs_of(Group& gr);
+template <> KrylovVecs<double2>& vecs_of<double2>(Group& gr) { return gr.k128; }
+template <> KrylovVecs<float2>& vecs_of<float2>(Group& gr) { return gr.k64; }
+
+template <class C> static BlockTab<C> block_tab(vie_grid* g, size_t g0, bool gather) {
+    BlockTab<C> t{};
+    t.nx = g->nx; t.ny = g->ny; t.nz = g->nz;
+    for (size_t i = g0; i < g->groups.size() && t.n < kBlockTabMax; ++i) {
+        const BoxSet& bs = g->groups[i].bs;
+        const KrylovVecs<C>& v = vecs_of<C>(g->groups[i]);
+        t.vec[t.n] = gather ? v.b : v.x;
+        t.mask[t.n] = bs.mask;
+        t.origin[t.n] = bs.origin;
+        t.bx[t.n] = bs.bx; t.by[t.n] = bs.by; t.bz[t.n] = bs.bz;
+        t.first[t.n + 1] = t.first[t.n] + bs.nb * bs.vec_elems();
+        ++t.n;
+    }
+    return t;
+}
+
+template <class C> int precond_gather(vie_grid* g, const C* b, cudaStream_t s) {
+    for (size_t g0 = 0; g0 < g->groups.size(); g0 += kBlockTabMax) {
+        const BlockTab<C> t = block_tab<C>(g, g0, true);
+        prof_begin(s, PK_FIELD, sizeof(C) == 16 ? VIE_C128 : VIE_C64, 0, 2 * t.first[t.n] * (int64_t)sizeof(C), false);
+        const cudaError_t e = launch_dependent(k_gather<C>, dim3(grid_1d(t.first[t.n])), 256, 0, s, b, t);
+        prof_end(s);
+        VIE_CK(e);
+    }
     return VIE_OK;
 }
 
-template <class C>
-int precond_scatter_group(const vie_grid* g, const Group& gr, const C* xk, C* y, cudaStream_t s) {
-    const BoxSet& bs = gr.bs;
-    prof_begin(s, PK_FIELD, sizeof(C) == 16 ? VIE_C128 : VIE_C64, 0, 2 * bs.nb * bs.vec_elems() * (int64_t)sizeof(C), false);
-    k_scatter<C><<<grid_1d(bs.nb * bs.vec_elems()), 256, 0, s>>>(xk, y, bs.mask, bs.origin, bs.nb, bs.bx, bs.by,
-                                                                 bs.bz, g->nx, g->ny, g->nz);
-    prof_end(s);
-    VIE_CK(cudaGetLastError());
+template <class C> int precond_scatter(vie_grid* g, const C* b, C* y, cudaStream_t s) {
+    for (size_t g0 = 0; g0 < g->groups.size(); g0 += kBlockTabMax) {
+        const BlockTab<C> t = block_tab<C>(g, g0, false);
+        const int64_t n = t.first[t.n] + (g0 == 0 ? g->N : 0);
+        prof_begin(s, PK_FIELD, sizeof(C) == 16 ? VIE_C128 : VIE_C64, 0,
+                   2 * t.first[t.n] * (int64_t)sizeof(C) + (g0 == 0 ? g->N * (4 + 6 * (int64_t)sizeof(C)) : 0), false);
+        const cudaError_t e = launch_dependent(k_scatter<C>, dim3(grid_1d(n)), 256, 0, s, y, t, b,
+                                               g0 == 0 ? (const int32_t*)g->block_id : (const int32_t*)nullptr);
+        prof_end(s);
+        VIE_CK(e);
+    }
     return VIE_OK;
 }
 
-template <class C>
-int precond_copy_unblocked(const vie_grid* g, const C* b, C* y, cudaStream_t s) {
-    prof_begin(s, PK_FIELD, sizeof(C) == 16 ? VIE_C128 : VIE_C64, 0, g->N * 4 + 6 * g->N * (int64_t)sizeof(C), false);
-    k_copy_unblocked<C><<<grid_1d(g->N), 256, 0, s>>>(b, y, g->block_id, g->N);
-    prof_end(s);
-    VIE_CK(cudaGetLastError());
-    return VIE_OK;
-}
-
-template int precond_gather<double2>(const vie_grid*, const Group&, const double2*, double2*, cudaStream_t);
-template int precond_gather<float2>(const vie_grid*, const Group&, const float2*, float2*, cudaStream_t);
-template int precond_scatter_group<double2>(const vie_grid*, const Group&, const double2*, double2*, cudaStream_t);
-template int precond_scatter_group<float2>(const vie_grid*, const Group&, const float2*, float2*, cudaStream_t);
-template int precond_copy_unblocked<double2>(const vie_grid*, const double2*, double2*, cudaStream_t);
-template int precond_copy_unblocked<float2>(const vie_grid*, const float2*, float2*, cudaStream_t);
+template int precond_gather<double2>(vie_grid*, const double2*, cudaStream_t);
+template int precond_gather<float2>(vie_grid*, const float2*, cudaStream_t);
+template int precond_scatter<double2>(vie_grid*, const double2*, double2*, cudaStream_t);
+template int precond_scatter<float2>(vie_grid*, const float2*, float2*, cudaStream_t);
 
 }  // namespace vie

@@ -162,6 +162,7 @@ __device__ void finalize(SegState& s, double2 d1, double2 d2, int* n_active, dou
 // One fused pass over a segment: vector update and/or up to two inner products.
 template <class C, int OP>
 __global__ void __launch_bounds__(kRedThreads) k_bicg(VecArgs<C> a) {
+    pdl_wait();
     const int seg = blockIdx.y;
     SegState& S = a.st[seg];
     if (OP != OP_INIT) {
@@ -289,18 +290,20 @@ static int launch_bicg(Bicg<C>& k, int op, double tol, int maxit, cudaStream_t s
     const bool dot = op == OP_SIGMA || op == OP_OMEGA;
     a.units = prof_begin(s, dot ? PK_BICG_DOT : PK_BICG_UPDATE, sizeof(C) == 16 ? VIE_C128 : VIE_C64,
                          (int64_t)nvec[op] * k.seglen * (int64_t)sizeof(C), 0, true);
+    auto kern = k_bicg<C, OP_INIT>;
     switch (op) {
-        case OP_INIT: k_bicg<C, OP_INIT><<<grid, kRedThreads, 0, s>>>(a); break;
-        case OP_P: k_bicg<C, OP_P><<<grid, kRedThreads, 0, s>>>(a); break;
-        case OP_S: k_bicg<C, OP_S><<<grid, kRedThreads, 0, s>>>(a); break;
-        case OP_XHALF: k_bicg<C, OP_XHALF><<<grid, kRedThreads, 0, s>>>(a); break;
-        case OP_XR: k_bicg<C, OP_XR><<<grid, kRedThreads, 0, s>>>(a); break;
-        case OP_SIGMA: k_bicg<C, OP_SIGMA><<<grid, kRedThreads, 0, s>>>(a); break;
-        case OP_OMEGA: k_bicg<C, OP_OMEGA><<<grid, kRedThreads, 0, s>>>(a); break;
+        case OP_INIT: break;
+        case OP_P: kern = k_bicg<C, OP_P>; break;
+        case OP_S: kern = k_bicg<C, OP_S>; break;
+        case OP_XHALF: kern = k_bicg<C, OP_XHALF>; break;
+        case OP_XR: kern = k_bicg<C, OP_XR>; break;
+        case OP_SIGMA: kern = k_bicg<C, OP_SIGMA>; break;
+        case OP_OMEGA: kern = k_bicg<C, OP_OMEGA>; break;
         default: prof_end(s); return fail(VIE_EINVAL, "bad BiCGSTAB op");
     }
+    const cudaError_t e = launch_dependent(kern, grid, kRedThreads, 0, s, a);
     prof_end(s);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(e);
     return VIE_OK;
 }
 

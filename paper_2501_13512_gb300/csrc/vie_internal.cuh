@@ -86,6 +86,34 @@ template <class C> __device__ __forceinline__ C from_c128(double2 a);
 template <> __device__ __forceinline__ double2 from_c128<double2>(double2 a) { return a; }
 template <> __device__ __forceinline__ float2 from_c128<float2>(double2 a) { return make_float2((float)a.x, (float)a.y); }
 
+// ---------------------------------------------------------------- dependent launches
+// The kernels of a product and of a BiCGSTAB step follow one another on a stream and take a few microseconds
+// each on small grids. They are launched with programmatic stream serialization: a kernel's CTAs may be placed
+// while the last CTAs of its predecessor run, and wait in pdl_wait, before their first access to memory, until
+// the predecessor has finished and its writes are visible. Each kernel lets its successor be placed once its own
+// wait is over. (Plain launches -> these: 16^3 complex64 product 17.8 -> 14.6 us, preconditioner with 16 coarse
+// blocks 6.15 -> 5.46 ms, 8 particles of 24^3 15.7 -> 12.8 ms.)
+__device__ __forceinline__ void pdl_wait() {
+#ifdef __CUDA_ARCH__
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------- FFT plan pieces
 constexpr int kLmax = 1024;   // largest padded FFT length per axis
 constexpr int kLogLmax = 10;
@@ -481,11 +509,9 @@ template <> inline const double2* tw_of<double2>(const Twiddles& t) { return t.d
 template <> inline const float2* tw_of<float2>(const Twiddles& t) { return t.d64; }
 
 // ---------------------------------------------------------------- precond.cu
-template <class C>
-int precond_gather(const vie_grid* g, const Group& gr, const C* b, C* out, cudaStream_t s);
-template <class C>
-int precond_scatter_group(const vie_grid* g, const Group& gr, const C* xk, C* y, cudaStream_t s);
-template <class C>
-int precond_copy_unblocked(const vie_grid* g, const C* b, C* y, cudaStream_t s);
+// The groups' right-hand sides from b, and y from the groups' solutions (and from b on voxels of no block),
+// each in one launch per kBlockTabMax groups.
+template <class C> int precond_gather(vie_grid* g, const C* b, cudaStream_t s);
+template <class C> int precond_scatter(vie_grid* g, const C* b, C* y, cudaStream_t s);
 
 }  // namespace vie
