@@ -208,6 +208,7 @@ static void release_grid(vie_grid* g) {
     for (void* p : g->allocations) dfree(p);
     g->allocations.clear();
     if (g->h_ring) cudaFreeHost(g->h_ring);
+    if (g->h_st) cudaFreeHost(g->h_st);
     for (int i = 0; i < 2; ++i) {
         if (g->ev[i]) cudaEventDestroy(g->ev[i]);
         if (g->tev[i]) cudaEventDestroy(g->tev[i]);
@@ -230,18 +231,20 @@ static bool is_device_pointer(const void* p) {
 }
 
 // Bounded host wait for an event (no device-side spin exists in this library;
-// the bound protects callers from a device that stopped answering).
+// the bound protects callers from a device that stopped answering). Polls for
+// the first 2 ms, the length of a preconditioner apply or a product on the
+// served grids (a sleep of 20 us costs the timer's slack of 50 us on top, twice
+// or four times per outer iteration), then sleeps between polls.
 static int wait_event(cudaEvent_t ev, double timeout_ms) {
     if (timeout_ms <= 0) timeout_ms = 60000.0;
     auto t0 = std::chrono::steady_clock::now();
-    int spins = 0;
     for (;;) {
         cudaError_t e = cudaEventQuery(ev);
         if (e == cudaSuccess) return VIE_OK;
         if (e != cudaErrorNotReady) return cuda_fail(e, "cudaEventQuery", __FILE__, __LINE__);
-        if (++spins > 64) std::this_thread::sleep_for(std::chrono::microseconds(20));
         double el = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         if (el > timeout_ms) return fail(VIE_ETIMEOUT, "device did not finish within the wait bound");
+        if (el > 2.0) std::this_thread::sleep_for(std::chrono::microseconds(20));
     }
 }
 
@@ -427,6 +430,11 @@ extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
             .push_back(b);
     std::vector<int32_t> h_group(K), h_index(K), h_origin(3 * K);
     g->groups.resize(bykey.size());
+    // the states of all blocks in one array, read back in one copy to pinned memory after an apply
+    if ((rc = dalloc(g, &g->st_all, K))) return bail(rc);
+    if (K > 0 && cudaHostAlloc((void**)&g->h_st, K * sizeof(SegState), cudaHostAllocDefault) != cudaSuccess)
+        return bail(fail(VIE_ENOMEM, "pinned host allocation failed"));
+    int64_t st_off = 0;
     int gi = 0;
     for (auto& kv : bykey) {
         Group& gr = g->groups[gi];
@@ -484,7 +492,8 @@ extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
         const int64_t nv = gr.bs.nb * gr.bs.vec_elems();
         if ((rc = alloc_krylov(g, gr.k128, nv, true, false))) return bail(rc);
         if ((rc = alloc_krylov(g, gr.k64, nv, true, false))) return bail(rc);
-        if ((rc = dalloc(g, &gr.st, gr.bs.nb))) return bail(rc);
+        gr.st = g->st_all + st_off;
+        st_off += gr.bs.nb;
         if ((rc = alloc_reduce(g, gr.red, gr.bs.nb))) return bail(rc);
         ++gi;
     }
@@ -1091,26 +1100,25 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
     std::vector<int2>& wh = g->work_host[c128 ? 0 : 1];
     const bool reorder = !jobs.empty() && wh.size() > 1;
     if (stats || reorder || merged) {
-        std::vector<std::vector<SegState>> hs(ng);
-        for (int i = 0; i < ng; ++i) {
-            Group& gr = g->groups[i];
-            hs[i].resize(gr.bs.nb);
-            VIE_CK(cudaMemcpyAsync(hs[i].data(), gr.st, gr.bs.nb * sizeof(SegState), cudaMemcpyDeviceToHost, s));
-        }
+        VIE_CK(cudaMemcpyAsync(g->h_st, g->st_all, g->nblocks * sizeof(SegState), cudaMemcpyDeviceToHost, s));
         VIE_CK(cudaEventRecord(g->ev[0], s));
         VIE_TRY(wait_event(g->ev[0], timeout_ms));
-        for (int i = 0; i < ng; ++i)
-            for (int k = 0; k < g->groups[i].bs.nb; ++k) g->groups[i].last_iters[c128 ? 0 : 1][k] = (float)hs[i][k].iters;
+        std::vector<const SegState*> hs(ng);
+        for (int i = 0; i < ng; ++i) {
+            Group& gr = g->groups[i];
+            hs[i] = g->h_st + (gr.st - g->st_all);
+            for (int k = 0; k < gr.bs.nb; ++k) gr.last_iters[c128 ? 0 : 1][k] = (float)hs[i][k].iters;
+        }
         if (stats) {
             double sum = 0.0;
             stats->nblocks = g->nblocks;
-            for (int i = 0; i < ng; ++i)
-                for (auto& st : hs[i]) {
-                    sum += st.iters;
-                    stats->max_iters = std::max(stats->max_iters, (int32_t)std::ceil(st.iters));
-                    if (st.status == SEG_MAXIT) stats->not_converged++;
-                    if (st.status == SEG_BREAKDOWN) stats->breakdowns++;
-                }
+            for (int k = 0; k < g->nblocks; ++k) {
+                const SegState& st = g->h_st[k];
+                sum += st.iters;
+                stats->max_iters = std::max(stats->max_iters, (int32_t)std::ceil(st.iters));
+                if (st.status == SEG_MAXIT) stats->not_converged++;
+                if (st.status == SEG_BREAKDOWN) stats->breakdowns++;
+            }
             stats->mean_iters = sum / std::max(1, g->nblocks);
         }
         if (reorder) {

@@ -245,7 +245,7 @@ struct Group {
     BoxSet bs;
     KrylovVecs<double2> k128;
     KrylovVecs<float2> k64;
-    SegState* st = nullptr;            // [nb]
+    SegState* st = nullptr;            // [nb], part of the grid's st_all
     ReduceScratch red;
 };
 
@@ -289,6 +289,8 @@ struct vie_grid {
     double2* host_io[2] = {nullptr, nullptr};   // vie_solve_host: E_inc and E on the device (first use)
     float2* tmp64 = nullptr;
     vie::SegState* ost = nullptr;         // outer state [1]
+    vie::SegState* st_all = nullptr;      // states of all blocks [nblocks], group after group
+    vie::SegState* h_st = nullptr;        // pinned host copy
     vie::ReduceScratch ored;
     double* dscal = nullptr;              // device scalars: [0] ||b||^2, [1] ||r||^2
     char* h_ring = nullptr;               // pinned host: active counts, state, scalar
