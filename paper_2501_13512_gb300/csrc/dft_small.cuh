@@ -23,11 +23,10 @@ template <bool FWD, class C> VIE_HD void dft2(C& a, C& b) {
 template <bool FWD, class C> VIE_HD void dft3(C& a, C& b, C& c) {
     typedef typename real_of<C>::type R;
     const R h = (R)0.86602540378443864676;               // sin(pi / 3)
-    const C s = b + c, d = rot<FWD>(cscale(b - c, h));
-    const C m = mk(a.x - (R)0.5 * s.x, a.y - (R)0.5 * s.y);
+    const C s = b + c, d = rot<FWD>(b - c), m = cfmas(s, (R)-0.5, a);
     a = a + s;
-    b = m + d;
-    c = m - d;
+    b = cfmas(d, h, m);
+    c = cfmas(d, -h, m);
 }
 
 template <bool FWD, class C> VIE_HD void dft4(C& a, C& b, C& c, C& d) {
@@ -43,8 +42,7 @@ template <bool FWD, class C> VIE_HD void dft5(C& a, C& b, C& c, C& d, C& e) {
     const R c1 = (R)0.30901699437494742410, c2 = (R)-0.80901699437494742410;   // cos(2 pi / 5), cos(4 pi / 5)
     const R s1 = (R)0.95105651629515357212, s2 = (R)0.58778525229247312917;    // sin of the same
     const C p = b + e, q = c + d, u = b - e, v = c - d;
-    const C m1 = mk(a.x + c1 * p.x + c2 * q.x, a.y + c1 * p.y + c2 * q.y);
-    const C m2 = mk(a.x + c2 * p.x + c1 * q.x, a.y + c2 * p.y + c1 * q.y);
+    const C m1 = cfmas(q, c2, cfmas(p, c1, a)), m2 = cfmas(q, c1, cfmas(p, c2, a));
     const C n1 = rot<FWD>(mk(s1 * u.x + s2 * v.x, s1 * u.y + s2 * v.y));
     const C n2 = rot<FWD>(mk(s2 * u.x - s1 * v.x, s2 * u.y - s1 * v.y));
     a = a + p + q;
