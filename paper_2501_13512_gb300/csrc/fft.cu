@@ -713,12 +713,24 @@ __global__ void __launch_bounds__(256) k_rows4_inv(RowArgs<float2> a) {
         for (int64_t b = (row0 + rpb - 1) / rpb; b * rpb < row0 + kRows4 && b * rpb < a.nrows; ++b)
             if (box_active(a.st, (int)b)) atomicAdd(a.units, 1);
     }
-    for (int idx = threadIdx.x; idx < kRows4 * L; idx += blockDim.x) {
-        const int r = idx / L, p = idx - r * L;
-        const int64_t row = row0 + r;
-        float2 v = czero<float2>();
-        if (row < a.nrows && box_active(a.st, (int)(row / a.rows_per_box))) v = a.in[row * a.in_stride + p];
-        sm[r * LP + pad32(p)] = v;
+    // 16-byte loads (rows of w1 start 16-byte aligned), all of a thread's in flight at once
+    {
+        constexpr int NV = kRows4 * L / 2 / 256 > 0 ? kRows4 * L / 2 / 256 : 1;
+        float4 q[NV];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int idx = threadIdx.x + 256 * i, r = idx / (L / 2), p = 2 * (idx - r * (L / 2));
+            const int64_t row = row0 + r;
+            q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < a.nrows && box_active(a.st, (int)(row / a.rows_per_box)))
+                q[i] = *reinterpret_cast<const float4*>(a.in + row * a.in_stride + p);
+        }
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int idx = threadIdx.x + 256 * i, r = idx / (L / 2), p = 2 * (idx - r * (L / 2));
+            sm[r * LP + pad32(p)] = make_float2(q[i].x, q[i].y);
+            sm[r * LP + pad32(p + 1)] = make_float2(q[i].z, q[i].w);
+        }
     }
     __syncthreads();
     for (int t = threadIdx.x; t < kRows4 * A; t += blockDim.x) {
@@ -737,19 +749,25 @@ __global__ void __launch_bounds__(256) k_rows4_inv(RowArgs<float2> a) {
     if (row >= a.nrows) return;
     const int b = (int)(row / a.rows_per_box);
     if (!box_active(a.st, b)) return;
+    // x and the mask before the last step: loads behind the stores of y would wait for one another
+    const int64_t mrow = (int64_t)b * a.plane + (row % a.plane);
+    float2 xv[A / 2];
+    bool in[A / 2];
+#pragma unroll
+    for (int m = 0; m < A / 2; ++m) {
+        const int p = j + kB4 * m;
+        const bool live = p < a.n_out;
+        xv[m] = live ? a.xin[row * a.out_stride + p] : czero<float2>();
+        in[m] = live && (a.mask == nullptr || a.mask[mrow * a.bx + p]);
+    }
     float2 v[A];
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = sm[r * LP + pad32(j + kB4 * m)];
     step_a_inv<A>(v, j, a.tw);
-    const int64_t mrow = (int64_t)b * a.plane + (row % a.plane);
 #pragma unroll
     for (int m = 0; m < A / 2; ++m) {
         const int p = j + kB4 * m;
-        if (p >= a.n_out) continue;
-        const int64_t o = row * a.out_stride + p;
-        float2 y = a.xin[o] - v[m];
-        if (a.mask != nullptr && !a.mask[mrow * a.bx + p]) y = czero<float2>();
-        a.out[o] = y;
+        if (p < a.n_out) a.out[row * a.out_stride + p] = in[m] ? xv[m] - v[m] : czero<float2>();
     }
 }
 

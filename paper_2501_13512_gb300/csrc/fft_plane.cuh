@@ -144,12 +144,25 @@ __device__ __forceinline__ void plane_rows_inv(const PlaneArgs<C>& a, C* sm, C* 
     for (int t = threadIdx.x; t < a.by * B; t += blockDim.x) {
         const int n2 = t & (B - 1), y = t / B;
         const C* row = sm + y * a.pitch;
+        // x and the mask first: loads behind the stores of y would wait for one another
+        // (complex64; complex128 has no registers left for them)
+        constexpr bool AHEAD = sizeof(C) == 8;
+        C xv[A / 2];
+        bool in[A / 2];
+        if (AHEAD) {
+#pragma unroll
+            for (int j = 0; j < A / 2; ++j) {
+                const int x = j * B + n2, o = y * a.bx + x;
+                xv[j] = x < a.bx ? xin[o] : czero<C>();
+                in[j] = x < a.bx && (mask == nullptr || mask[o]);
+            }
+        }
         line_a_inv<A, B>(n2, a.tw, [&](int p) { return row[plane_pad(p)]; },
                          [&](int x, C u) {
                              if (x >= a.bx) return;
                              const int o = y * a.bx + x;
-                             C v = xin[o] - u;
-                             if (mask != nullptr && !mask[o]) v = czero<C>();
+                             C v = (AHEAD ? xv[x / B] : xin[o]) - u;
+                             if (AHEAD ? !in[x / B] : mask != nullptr && !mask[o]) v = czero<C>();
                              out[o] = v;
                          });
     }
@@ -293,12 +306,17 @@ __global__ void __launch_bounds__(kLineThreadsRow) k_line_rows(RowArgs<C> a) {
             const C* xin = a.xin + (row0 + r) * a.out_stride;
             C* out = a.out + (row0 + r) * a.out_stride;
             const uint8_t* mask = a.mask ? a.mask + vox(r) : nullptr;
+            C xv[A / 2];
+            bool in[A / 2];
+#pragma unroll
+            for (int j = 0; j < A / 2; ++j) {
+                const int x = j * B + n2;
+                xv[j] = x < a.n_out ? xin[x] : czero<C>();
+                in[j] = x < a.n_out && (mask == nullptr || mask[x]);
+            }
             line_a_inv<A, B>(n2, a.tw, [&](int p) { return row[plane_pad(p)]; },
                              [&](int x, C u) {
-                                 if (x >= a.n_out) return;
-                                 C v = xin[x] - u;
-                                 if (mask != nullptr && !mask[x]) v = czero<C>();
-                                 out[x] = v;
+                                 if (x < a.n_out) out[x] = in[x / B] ? xv[x / B] - u : czero<C>();
                              });
         }
     }
