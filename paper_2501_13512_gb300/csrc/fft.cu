@@ -236,124 +236,6 @@ __global__ void __launch_bounds__(kThreads) k_zgreen(ZArgs<C> a) {
     }
 }
 
-// Pass Z of complex64 MVMs with Mz <= 32, register-resident: each thread
-// transforms one (component, column) pencil in registers (pruned: the box
-// fills at most the lower half of the padded axis), the three transformed
-// components of kZRegCols columns meet in shared memory for the 3x3 Green
-// multiply, and each thread transforms its pencil back, keeping z < bz. The
-// spectrum is even in z for xx, xy, yy, zz and odd for xz, yz, so one load of
-// its six entries serves the z positions of frequencies f and -f.
-constexpr int kZRegCols = 64;
-constexpr int kZRegThreads = 3 * kZRegCols;
-
-template <int LZ>
-__global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
-    pdl_wait();
-    typedef float2 F;
-    constexpr int H = LZ / 2 > 0 ? LZ / 2 : 1;
-    constexpr int LGZ = ILog2<LZ>::v;
-    constexpr int NC = kZRegCols;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    F* sm = reinterpret_cast<F*>(smem_raw);          // [3][LZ][NC]
-    const int b = blockIdx.y;
-    if (!box_active(a.st, b)) return;
-    if (a.units != nullptr && threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(a.units, 1);
-    const int P = a.ncols, bz = a.nzb, c0 = blockIdx.x * NC, t = threadIdx.x;
-    const int nc = min(NC, P - c0);
-    F* W = a.w + (int64_t)b * a.box_stride + c0;
-    const int64_t cs = a.comp_stride;
-    {
-        const int comp = t / NC, c = t - comp * NC;
-        if (c < nc) {
-            const F* src = W + comp * cs + c;
-            F* S = sm + comp * LZ * NC + c;
-            if (LZ == 1) {
-                S[0] = src[0];
-            } else {
-                F v[H];
-#pragma unroll
-                for (int j = 0; j < H; ++j) v[j] = j < bz ? src[(int64_t)j * P] : czero<F>();
-                F q[H];
-#pragma unroll
-                for (int j = 0; j < H; ++j) q[j] = twc<true>(v[j], j * (kLmax / LZ));
-                rfft<H, true>(q, (const F*)nullptr);
-#pragma unroll
-                for (int j = 0; j < H; ++j) S[(H + j) * NC] = q[j];
-                rfft<H, true>(v, (const F*)nullptr);
-#pragma unroll
-                for (int j = 0; j < H; ++j) S[j * NC] = v[j];
-            }
-        }
-    }
-    __syncthreads();
-    const F* G = a.Gb ? a.Gb[b] : a.G;
-    const int hx = (1 << a.lx) / 2 + 1, hy = (1 << a.ly) / 2 + 1;
-    const int cst = LZ * NC;
-    for (int task = t; task < LZ * NC; task += kZRegThreads) {
-        const int i = task / NC, c = task - i * NC;
-        if (c >= nc) continue;
-        const int f = LGZ ? (int)(__brev((unsigned)i) >> (32 - LGZ)) : 0;
-        const int fm = (LZ - f) & (LZ - 1);
-        const int im = LGZ ? (int)(__brev((unsigned)fm) >> (32 - LGZ)) : 0;
-        if (im < i) continue;
-        const int col = c0 + c;
-        bool ux = false, uy = false, uz = false;
-        const F* gp;
-        if (a.oct) {
-            const int qx = octant_slot(col & ((1 << a.lx) - 1), a.lx, ux);
-            const int qy = octant_slot(col >> a.lx, a.ly, uy);
-            const int qz = octant_slot(i, LGZ, uz);
-            gp = G + ((int64_t)qz * hy + qy) * hx + qx;
-        } else {
-            gp = G + (int64_t)i * P + col;
-        }
-        const F gxx = gp[0], gyy = gp[3 * a.gcomp], gzz = gp[5 * a.gcomp];
-        F gxy = gp[a.gcomp], gxz = gp[2 * a.gcomp], gyz = gp[4 * a.gcomp];
-        if (ux != uy) gxy = mk(-gxy.x, -gxy.y);
-        if (ux != uz) gxz = mk(-gxz.x, -gxz.y);
-        if (uy != uz) gyz = mk(-gyz.x, -gyz.y);
-        const F e[6] = {gxx, gxy, gxz, gyy, gyz, gzz};
-        {
-            F* q = sm + i * NC + c;
-            F X = q[0], Y = q[cst], Z = q[2 * cst];
-            green3<2, false>(X, Y, Z, e);
-            q[0] = X;
-            q[cst] = Y;
-            q[2 * cst] = Z;
-        }
-        if (im != i) {   // frequency -f: xz and yz change sign
-            F* q = sm + im * NC + c;
-            F X = q[0], Y = q[cst], Z = q[2 * cst];
-            green3<2, true>(X, Y, Z, e);
-            q[0] = X;
-            q[cst] = Y;
-            q[2 * cst] = Z;
-        }
-    }
-    __syncthreads();
-    {
-        const int comp = t / NC, c = t - comp * NC;
-        if (c < nc) {
-            F* S = sm + comp * LZ * NC + c;
-            F* dst = W + comp * cs + c;
-            if (LZ == 1) {
-                dst[0] = S[0];
-            } else {
-                F u[H], v[H];
-#pragma unroll
-                for (int j = 0; j < H; ++j) v[j] = S[(H + j) * NC];
-                rfft<H, false>(v, (const F*)nullptr);
-#pragma unroll
-                for (int j = 0; j < H; ++j) u[j] = S[j * NC];
-                rfft<H, false>(u, (const F*)nullptr);
-#pragma unroll
-                for (int j = 0; j < H; ++j)
-                    if (j < bz) dst[(int64_t)j * P] = u[j] + twc<false>(v[j], j * (kLmax / LZ));
-            }
-        }
-    }
-}
-
 // Where a column's spectrum entries lie: octant (OCT) or full layout (bit-reversed positions). entry(f) is
 // the offset of component xx at the z frequency f in [0, M/2]; the six components are gcomp apart. sxy, sx,
 // sy: whether xy, xz and yz change sign with the column's x and y frequencies (octant).
@@ -390,6 +272,118 @@ template <class C, bool OCT> struct ZColumn {
         }
     }
 };
+
+// Pass Z of complex64 MVMs with Mz <= 32, register-resident: each thread
+// transforms one (component, column) pencil in registers (pruned: the box
+// fills at most the lower half of the padded axis), the three transformed
+// components of kZRegCols columns meet in shared memory for the 3x3 Green
+// multiply, and each thread transforms its pencil back, keeping z < bz. The
+// spectrum is even in z for xx, xy, yy, zz and odd for xz, yz, so one load of
+// its six entries serves the z positions of frequencies f and -f. Bound by the
+// latency of those loads: entries of two frequencies in flight, 84 -> 68 us at
+// 256x256x16 (three 80, six 90: fewer CTAs fit).
+constexpr int kZRegCols = 64;
+constexpr int kZRegThreads = 3 * kZRegCols;
+
+template <int LZ, bool OCT>
+__global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
+    pdl_wait();
+    typedef float2 F;
+    constexpr int H = LZ / 2 > 0 ? LZ / 2 : 1;
+    constexpr int LGZ = ILog2<LZ>::v;
+    constexpr int NC = kZRegCols;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    F* sm = reinterpret_cast<F*>(smem_raw);          // [3][LZ][NC]
+    const int b = blockIdx.y;
+    if (!box_active(a.st, b)) return;
+    if (a.units != nullptr && threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(a.units, 1);
+    const int P = a.ncols, bz = a.nzb, c0 = blockIdx.x * NC, t = threadIdx.x;
+    const int nc = min(NC, P - c0);
+    F* W = a.w + (int64_t)b * a.box_stride + c0;
+    const int64_t cs = a.comp_stride;
+    const int comp = t / NC, c = t - comp * NC;
+    {
+        if (c < nc) {
+            const F* src = W + comp * cs + c;
+            F* S = sm + comp * LZ * NC + c;
+            if (LZ == 1) {
+                S[0] = src[0];
+            } else {
+                F v[H];
+#pragma unroll
+                for (int j = 0; j < H; ++j) v[j] = j < bz ? src[(int64_t)j * P] : czero<F>();
+                F q[H];
+#pragma unroll
+                for (int j = 0; j < H; ++j) q[j] = twc<true>(v[j], j * (kLmax / LZ));
+                rfft<H, true>(q, (const F*)nullptr);
+#pragma unroll
+                for (int j = 0; j < H; ++j) S[(H + j) * NC] = q[j];
+                rfft<H, true>(v, (const F*)nullptr);
+#pragma unroll
+                for (int j = 0; j < H; ++j) S[j * NC] = v[j];
+            }
+        }
+    }
+    // Green multiply: thread (comp, c) takes the frequencies f = comp, comp + 3, ... <= LZ / 2 of column c
+    // and their mirrors, the spectrum entries of ZU frequencies in flight at once (the first ones before the wait).
+    constexpr int NF = (LZ / 2 + 1 + 2) / 3, cst = LZ * NC;
+    constexpr int ZU = NF < 2 ? NF : 2;
+    const ZColumn<F, OCT> zc(a, b, c0 + (c < nc ? c : 0));
+#pragma unroll
+    for (int k0 = 0; k0 < NF; k0 += ZU) {
+        F e[ZU][6];
+#pragma unroll
+        for (int k = 0; k < ZU; ++k) {
+            const int f = min(comp + 3 * (k0 + k), LZ / 2);
+            const int i = LGZ ? (int)(__brev((unsigned)f) >> (32 - LGZ)) : 0;
+            const int q = !OCT ? i : f == LZ / 2 ? LZ / 2 : LGZ >= 2 ? (int)(__brev((unsigned)f) >> (33 - LGZ)) : 0;
+            zc.load(e[k], q, a.gcomp);
+        }
+        if (k0 == 0) __syncthreads();
+#pragma unroll
+        for (int k = 0; k < ZU; ++k) {
+            const int f = comp + 3 * (k0 + k);
+            if (c >= nc || f > LZ / 2) continue;
+            const int i = LGZ ? (int)(__brev((unsigned)f) >> (32 - LGZ)) : 0;
+            const int im = LGZ ? (int)(__brev((unsigned)((LZ - f) & (LZ - 1))) >> (32 - LGZ)) : 0;
+            F* q = sm + i * NC + c;
+            F X = q[0], Y = q[cst], Z = q[2 * cst];
+            green3<2, false>(X, Y, Z, e[k]);
+            q[0] = X;
+            q[cst] = Y;
+            q[2 * cst] = Z;
+            if (im != i) {   // frequency -f: xz and yz change sign
+                F* m = sm + im * NC + c;
+                F X = m[0], Y = m[cst], Z = m[2 * cst];
+                green3<2, true>(X, Y, Z, e[k]);
+                m[0] = X;
+                m[cst] = Y;
+                m[2 * cst] = Z;
+            }
+        }
+    }
+    __syncthreads();
+    {
+        if (c < nc) {
+            F* S = sm + comp * LZ * NC + c;
+            F* dst = W + comp * cs + c;
+            if (LZ == 1) {
+                dst[0] = S[0];
+            } else {
+                F u[H], v[H];
+#pragma unroll
+                for (int j = 0; j < H; ++j) v[j] = S[(H + j) * NC];
+                rfft<H, false>(v, (const F*)nullptr);
+#pragma unroll
+                for (int j = 0; j < H; ++j) u[j] = S[j * NC];
+                rfft<H, false>(u, (const F*)nullptr);
+#pragma unroll
+                for (int j = 0; j < H; ++j)
+                    if (j < bz) dst[(int64_t)j * P] = u[j] + twc<false>(v[j], j * (kLmax / LZ));
+            }
+        }
+    }
+}
 
 // exp(-2 pi i m / 1024) at a compile-time m, times or conjugated times v.
 template <bool FWD> __device__ __forceinline__ float2 ztw(float2 v, int m, const float2*) { return twc<FWD>(v, m); }
@@ -483,7 +477,8 @@ __global__ void __launch_bounds__(2 * kZPairCols, 2) k_z_pair(ZArgs<C> a) {
 //            Green multiply of its B frequencies, inverse transform, twiddles;   to shared memory
 //   step A'  the inverse of step A, planes z < bz kept.
 // Four shared-memory accesses per value and no stage over padding, against 2 log4(L) + 4 of the radix-4 form:
-// complex64, 128^3 voxels (256 points) 525 -> 231 us, 64^3 (128 points) 62 -> 29 us, 100x37x60 113 -> 57 us;
+// complex64, 128^3 voxels (256 points) 525 -> 194 us, 64^3 (128 points) 62 -> 27 us, 100x37x60 113 -> 45 us (the
+// first four frequencies' spectrum entries on their way before the B-point transform: 209 -> 194 us);
 // complex128, bound by the FP64 units, 128^3 5970 -> 5220 us with sums as multiply-adds (radd).
 template <class C, int A, int B> struct ZFour {
     static constexpr int L = A * B;
@@ -496,6 +491,8 @@ template <class C, int A, int B> struct ZFour {
 template <class C, int A, int B, bool OCT>
 __global__ void __launch_bounds__((ZFour<C, A, B>::threads), (ZFour<C, A, B>::ctas)) k_z_four(ZArgs<C> a) {
     pdl_wait();
+    constexpr int ZP = sizeof(C) == 8 ? 4 : 1;   // frequencies whose entries are in flight
+    constexpr bool AHEAD = sizeof(C) == 8;
     constexpr int L = A * B, HA = A / 2, NC = ZFour<C, A, B>::NC, TS = kLmax / A, LG = ILog2<L>::v;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* sm = reinterpret_cast<C*>(smem_raw);      // [3][k1 B + n2][NC]
@@ -529,6 +526,18 @@ __global__ void __launch_bounds__((ZFour<C, A, B>::threads), (ZFour<C, A, B>::ct
         const int c = task % NC, k1 = task / NC;
         if (c >= nc) continue;
         const ZColumn<C, OCT> zc(a, b, col0 + c);
+        const auto entries = [&](C (&e)[6], int k2) {
+            const int k = k1 + A * k2, f = k > L / 2 ? L - k : k;
+            const int q = !OCT ? (int)(__brev((unsigned)f) >> (32 - LG)) : f == L / 2 ? L / 2 : (int)(__brev((unsigned)f) >> (33 - LG));
+            zc.load(e, q, a.gcomp);
+            e[2] = cneg_if(e[2], k > L / 2);
+            e[4] = cneg_if(e[4], k > L / 2);
+        };
+        C e[ZP][6];
+        if (AHEAD) {
+#pragma unroll
+            for (int k2 = 0; k2 < ZP; ++k2) entries(e[k2], k2);
+        }
         C w[B], v[3][B];
 #pragma unroll
         for (int n2 = 1; n2 < B; ++n2) w[n2] = __ldg(a.tw + ((n2 * k1) << (kLogLmax - LG)));
@@ -541,17 +550,8 @@ __global__ void __launch_bounds__((ZFour<C, A, B>::threads), (ZFour<C, A, B>::ct
         }
 #pragma unroll
         for (int k2 = 0; k2 < B; ++k2) {
-            const int k = k1 + A * k2;
-            const bool up = k > L / 2;
-            const int f = up ? L - k : k;
-            int q;
-            if (OCT) q = f == L / 2 ? L / 2 : (int)(__brev((unsigned)f) >> (33 - LG));
-            else q = (int)(__brev((unsigned)f) >> (32 - LG));
-            C e[6];
-            zc.load(e, q, a.gcomp);
-            e[2] = cneg_if(e[2], up);
-            e[4] = cneg_if(e[4], up);
-            green3<2, false>(v[0][k2], v[1][k2], v[2][k2], e);
+            if (!AHEAD || k2 >= ZP) entries(e[k2 % ZP], k2);
+            green3<2, false>(v[0][k2], v[1][k2], v[2][k2], e[k2 % ZP]);
         }
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -994,13 +994,13 @@ static int launch_cols(ColArgs<C> a, int nb1, int nb2, Prof pf, cudaStream_t s) 
     return VIE_OK;
 }
 
-template <int LZ>
+template <int LZ, bool OCT>
 static int launch_zgreen_reg(ZArgs<float2> a, int nb, Prof pf, cudaStream_t s) {
     const size_t smem = (size_t)3 * LZ * kZRegCols * sizeof(float2);
-    VIE_TRY(prep_smem(k_zgreen_reg<LZ>, smem));
+    VIE_TRY(prep_smem(k_zgreen_reg<LZ, OCT>, smem));
     dim3 grid((a.ncols + kZRegCols - 1) / kZRegCols, nb);
     a.units = prof_begin(s, pf.kind, VIE_C64, pf.bpu, pf.fixed, true);
-    const cudaError_t e = launch_dependent(k_zgreen_reg<LZ>, grid, kZRegThreads, smem, s, a);
+    const cudaError_t e = launch_dependent(k_zgreen_reg<LZ, OCT>, grid, kZRegThreads, smem, s, a);
     prof_end(s);
     VIE_CK(e);
     return VIE_OK;
@@ -1034,10 +1034,10 @@ template <class C, bool OCT>
 static int launch_z_reg(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
     if constexpr (sizeof(C) == 8) {
         switch (a.lL) {
-            case 2: return launch_zgreen_reg<4>(a, nb, pf, s);
-            case 3: return launch_zgreen_reg<8>(a, nb, pf, s);
-            case 4: return launch_zgreen_reg<16>(a, nb, pf, s);
-            case 5: return launch_zgreen_reg<32>(a, nb, pf, s);
+            case 2: return launch_zgreen_reg<4, OCT>(a, nb, pf, s);
+            case 3: return launch_zgreen_reg<8, OCT>(a, nb, pf, s);
+            case 4: return launch_zgreen_reg<16, OCT>(a, nb, pf, s);
+            case 5: return launch_zgreen_reg<32, OCT>(a, nb, pf, s);
             default: break;
         }
     } else {
