@@ -648,7 +648,7 @@ constexpr int kRows4 = 8;   // rows per CTA (256 threads: 8 rows x 32)
 
 // Pass X forward: rows of bx -> chi * x, zero-padded to L = 32 A, forward transform.
 template <int A>
-__global__ void __launch_bounds__(256) k_rows4_fwd(RowArgs<float2> a) {
+__global__ void __launch_bounds__(256, A <= 16 ? 3 : 2) k_rows4_fwd(RowArgs<float2> a) {
     pdl_wait();
     constexpr int L = kB4 * A, LP = L + L / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -659,16 +659,13 @@ __global__ void __launch_bounds__(256) k_rows4_fwd(RowArgs<float2> a) {
         for (int64_t b = (row0 + rpb - 1) / rpb; b * rpb < row0 + kRows4 && b * rpb < a.nrows; ++b)
             if (box_active(a.st, (int)b)) atomicAdd(a.units, 1);
     }
+    // warp r owns row r at both ends
+    const int r = threadIdx.x >> 5, j = threadIdx.x & 31;
+    const int64_t row = row0 + r;
+    const int b = row < a.nrows ? (int)(row / a.rows_per_box) : 0;
+    const bool live = row < a.nrows && box_active(a.st, b);
     {
-        const int r = threadIdx.x >> 5, j = threadIdx.x & 31;
-        const int64_t row = row0 + r;
         float2 v[A];
-        bool live = row < a.nrows;
-        int b = 0;
-        if (live) {
-            b = (int)(row / a.rows_per_box);
-            live = box_active(a.st, b);
-        }
         const int64_t crow = live ? (int64_t)b * a.plane + (row % a.plane) : 0;
 #pragma unroll
         for (int m = 0; m < A; ++m) {
@@ -692,17 +689,19 @@ __global__ void __launch_bounds__(256) k_rows4_fwd(RowArgs<float2> a) {
         for (int i = 0; i < kB4; ++i) q[i] = u[i];
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < kRows4 * L; idx += blockDim.x) {
-        const int r = idx / L, p = idx - r * L;
-        const int64_t row = row0 + r;
-        if (row >= a.nrows || !box_active(a.st, (int)(row / a.rows_per_box))) continue;
-        a.out[row * a.out_stride + p] = sm[r * LP + pad32(p)];
+    if (!live) return;
+    float2* out = a.out + row * a.out_stride;
+#pragma unroll
+    for (int m = 0; m < A / 2; ++m) {
+        const int p = 2 * (j + 32 * m);
+        const float2 u = sm[r * LP + pad32(p)], v = sm[r * LP + pad32(p + 1)];
+        *reinterpret_cast<float4*>(out + p) = make_float4(u.x, u.y, v.x, v.y);
     }
 }
 
 // Pass X inverse: rows of L = 32 A spectrum positions -> keep x < bx, y = mask (x - u).
 template <int A>
-__global__ void __launch_bounds__(256) k_rows4_inv(RowArgs<float2> a) {
+__global__ void __launch_bounds__(256, A <= 16 ? 3 : 2) k_rows4_inv(RowArgs<float2> a) {
     pdl_wait();
     constexpr int L = kB4 * A, LP = L + L / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -713,23 +712,22 @@ __global__ void __launch_bounds__(256) k_rows4_inv(RowArgs<float2> a) {
         for (int64_t b = (row0 + rpb - 1) / rpb; b * rpb < row0 + kRows4 && b * rpb < a.nrows; ++b)
             if (box_active(a.st, (int)b)) atomicAdd(a.units, 1);
     }
-    // 16-byte loads (rows of w1 start 16-byte aligned), all of a thread's in flight at once
+    // Warp r owns row r at both ends; 16-byte loads, all of a thread's in flight at once. (Element by element,
+    // with the box looked up for each, 48 us at 256x256x16; so, 25.)
+    const int r = threadIdx.x >> 5, j = threadIdx.x & 31;
+    const int64_t row = row0 + r;
+    const int b = row < a.nrows ? (int)(row / a.rows_per_box) : 0;
+    const bool live = row < a.nrows && box_active(a.st, b);
     {
-        constexpr int NV = kRows4 * L / 2 / 256 > 0 ? kRows4 * L / 2 / 256 : 1;
-        float4 q[NV];
+        const float2* in = a.in + (live ? row : row0) * a.in_stride;
+        float4 q[A / 2];
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int idx = threadIdx.x + 256 * i, r = idx / (L / 2), p = 2 * (idx - r * (L / 2));
-            const int64_t row = row0 + r;
-            q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < a.nrows && box_active(a.st, (int)(row / a.rows_per_box)))
-                q[i] = *reinterpret_cast<const float4*>(a.in + row * a.in_stride + p);
-        }
+        for (int m = 0; m < A / 2; ++m) q[m] = *reinterpret_cast<const float4*>(in + 2 * (j + 32 * m));
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int idx = threadIdx.x + 256 * i, r = idx / (L / 2), p = 2 * (idx - r * (L / 2));
-            sm[r * LP + pad32(p)] = make_float2(q[i].x, q[i].y);
-            sm[r * LP + pad32(p + 1)] = make_float2(q[i].z, q[i].w);
+        for (int m = 0; m < A / 2; ++m) {
+            const int p = 2 * (j + 32 * m);
+            sm[r * LP + pad32(p)] = make_float2(q[m].x, q[m].y);
+            sm[r * LP + pad32(p + 1)] = make_float2(q[m].z, q[m].w);
         }
     }
     __syncthreads();
@@ -744,11 +742,7 @@ __global__ void __launch_bounds__(256) k_rows4_inv(RowArgs<float2> a) {
         for (int i = 0; i < kB4; ++i) q[i] = u[i];
     }
     __syncthreads();
-    const int r = threadIdx.x >> 5, j = threadIdx.x & 31;
-    const int64_t row = row0 + r;
-    if (row >= a.nrows) return;
-    const int b = (int)(row / a.rows_per_box);
-    if (!box_active(a.st, b)) return;
+    if (!live) return;
     // x and the mask before the last step: loads behind the stores of y would wait for one another
     const int64_t mrow = (int64_t)b * a.plane + (row % a.plane);
     float2 xv[A / 2];
