@@ -279,17 +279,19 @@ template <bool STG, class C> __device__ __noinline__ void par_mid(const InnerGro
 // Team-wide sums of the N complex values v of every thread; fn(sums) runs in warp 0 of every CTA with
 // identical arguments and writes the shared state the closing barrier publishes. Each warp halves its
 // values over the lanes (2N real values take 2N - 1 + (5 - log2 2N) shuffles, in the vectors' precision),
-// its lanes store them into the slot of all four ranks, and after one cluster barrier warp 0 adds the
-// warps' and ranks' sums in FP64, lanes in parallel: an FP64 instruction holds its unit for the whole warp
-// whatever the number of active lanes, so the serial form (thread 0 adding 12 warps x 8 values, then 4
-// ranks) cost 9 us of a 22 us product. Two slots alternate: a slot is rewritten two sums later, after the
-// cluster barrier of the sum in between.
+// its lanes store them into the slot of all four ranks, and after one cluster barrier N warps add the
+// warps' and ranks' sums in FP64, one complex value each. What counts there is the number of FP64
+// instructions: each holds a quarter SM's unit for 64 clocks whatever the number of active lanes (a serial
+// form, thread 0 adding everything, cost 9 us of a 22 us product), so the additions are spread over the
+// quarters and lanes, and fn works on real and imaginary parts in different lanes. Two slots alternate: a
+// slot is rewritten two sums later, after the cluster barrier of the sum in between.
 constexpr int kParWarpsMax = 12;
 template <class C> struct ParSums {
     typename real_of<C>::type v[2][kParRanks][kParWarpsMax][8];
+    double2 tot[4];
 };
 
-template <int N, class C, class Fn>
+template <int NW, int N, class C, class Fn>
 __device__ __forceinline__ void par_sum(C (&v)[N], ParSums<C>& xs, int& slot, Fn fn) {
     typedef typename real_of<C>::type R;
     constexpr int NV = 2 * N;
@@ -300,7 +302,7 @@ __device__ __forceinline__ void par_sum(C (&v)[N], ParSums<C>& xs, int& slot, Fn
         x[2 * i] = v[i].x;
         x[2 * i + 1] = v[i].y;
     }
-    const int l = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
     int o = 16;
 #pragma unroll
     for (int h = NV / 2; h >= 1; h >>= 1, o >>= 1) {
@@ -320,49 +322,46 @@ __device__ __forceinline__ void par_sum(C (&v)[N], ParSums<C>& xs, int& slot, Fn
     slot ^= 1;
     if (dst < kParRanks) *cl.map_shared_rank(&xs.v[slot][rk][w][vi], (unsigned)dst) = x[0];
     cl.sync();
-    if (w == 0) {
-        constexpr int G = 32 / NV;              // lanes per value
-        const int q = l & (NV - 1);
-        double s = 0.0;
-        for (int k = l / NV; k < kParRanks * nw; k += G) {
-            const int r = k & (kParRanks - 1), ww = k / kParRanks;
-            s += (double)xs.v[slot][r][ww][q];
+    if (w < N) {
+        // warp w: complex value w; lane l: component l & 1 of every 16th partial sum, added as a tree
+        constexpr int ALL = kParRanks * NW, PER = (ALL + 15) / 16;
+        double u[PER];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int k = (l >> 1) + 16 * i;
+            u[i] = ALL % 16 == 0 || k < ALL ? (double)xs.v[slot][k & (kParRanks - 1)][k / kParRanks][2 * w + (l & 1)] : 0.0;
         }
 #pragma unroll
-        for (int m = NV; m < 32; m <<= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-        double2 t[N];
+        for (int h = PER; h > 1; h = (h + 1) / 2) {
 #pragma unroll
-        for (int i = 0; i < N; ++i)
-            t[i] = make_double2(__shfl_sync(0xffffffffu, s, 2 * i), __shfl_sync(0xffffffffu, s, 2 * i + 1));
-        fn(t);
+            for (int i = 0; i < h / 2; ++i) u[i] += u[i + (h + 1) / 2];
+        }
+        double s = u[0];
+#pragma unroll
+        for (int m = 2; m < 32; m <<= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+        if (l < 2) (l ? xs.tot[w].y : xs.tot[w].x) = s;
+        if (N > 1) asm volatile("bar.sync 15, %0;" ::"n"(32 * N) : "memory");
+        else __syncwarp();
+        if (w == 0) fn(xs.tot, l);
     }
     __syncthreads();
 }
 
+// Finite, and not zero: integer tests, an FP64 comparison takes 64 clocks.
+__device__ __forceinline__ bool par_finite(double a) { return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool par_zero(double a) { return ((__double2hiint(a) & 0x7fffffff) | __double2loint(a)) == 0; }
+__device__ __forceinline__ double par_lane(double a, int lane) { return __shfl_sync(0xffffffffu, a, lane); }
+// component c (0, 1) of a complex number
+template <class C2, class T> __device__ __forceinline__ void par_put(C2& z, int c, T v) { (c ? z.y : z.x) = v; }
+
 // Scalars of the iteration, written by warp 0 inside par_sum.
 template <class C> struct ParState {
-    double2 rho, rho_prev, alpha, omega;
-    double tol2, bn2, res2, iters;
+    double2 rho, iq;                            // iq = 1 / <rhat, v>
+    double tol2, bn2, res2;
+    int halves;                                 // half steps done
     int status, half, pend;                     // pend: the last full step's x update is pending
     C cbeta, comega, calpha;                    // coefficients of the vector updates
 };
-
-// a / b with one reciprocal (an FP64 division is about ten dependent FP64 instructions).
-__device__ __forceinline__ double2 par_cdiv(double2 a, double2 b) {
-    const double r = 1.0 / (b.x * b.x + b.y * b.y);
-    return make_double2((a.x * b.x + a.y * b.y) * r, (a.y * b.x - a.x * b.y) * r);
-}
-
-// beta = (rho / rho_prev) (alpha / omega) as one division, or a breakdown.
-template <class C> __device__ __forceinline__ void par_beta(ParState<C>& S, double2 rho, double2 rho_prev, double2 alpha,
-                                                            double2 omega) {
-    if (!dgood(rho)) {
-        S.status = SEG_BREAKDOWN;
-        return;
-    }
-    const double2 beta = par_cdiv(cmul(rho, alpha), cmul(rho_prev, omega));
-    S.cbeta = cmk<C>(beta.x, beta.y);
-}
 
 // Where the Krylov vectors of this rank's quarter live while a block is solved. Each thread works on the
 // same elements in every phase, so nothing here is shared between threads. CHIP: in shared memory behind
@@ -658,6 +657,7 @@ template <bool CHIP, class C>
 __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double tol, int maxit, C* sm, int* units) {
     typedef typename real_of<C>::type R;
     constexpr bool STG = sizeof(C) == 8, COLS = par_by_column<C>();
+    constexpr int NW = par_threads<C, CHIP>() / 32;
     __shared__ ParState<C> S;
     __shared__ ParSums<C> xs;
     __shared__ ParVecs<C, CHIP> V;
@@ -727,14 +727,13 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             zmask[c] = m;
         }
     }
-    par_sum(a0, xs, slot, [&](const double2 (&q)[1]) {
+    par_sum<NW>(a0, xs, slot, [&](const double2* q, int) {
         const double bn2 = q[0].x;
         S.bn2 = bn2;
         S.tol2 = tol * tol * bn2;
         S.rho = make_double2(bn2, 0.0);
-        S.alpha = S.omega = make_double2(1, 0);
         S.comega = cmk<C>(1.0, 0.0);
-        S.iters = 0.0;
+        S.halves = 0;
         S.res2 = bn2;
         S.half = 0;
         S.pend = 0;
@@ -764,15 +763,20 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             par_output<false>(g, V, sm, q4);
         }
         C p1[1] = {q4[0]};
-        par_sum(p1, xs, slot, [&](const double2 (&q)[1]) {
+        par_sum<NW>(p1, xs, slot, [&](const double2* q, int l) {
+            const double2 z = q[0], rho = S.rho;
+            const int c = l & 1;                // real and imaginary parts in lanes
             S.pend = 0;                         // the p update took the previous step's x update
-            if (!dgood(q[0])) {
+            if (!par_finite(z.x) || !par_finite(z.y) || (par_zero(z.x) && par_zero(z.y))) {
                 S.status = SEG_BREAKDOWN;
                 return;
             }
-            const double2 alpha = par_cdiv(S.rho, q[0]);
-            S.alpha = alpha;
-            S.calpha = cmk<C>(alpha.x, alpha.y);
+            const double d = 1.0 / (z.x * z.x + z.y * z.y), iq = (c ? -z.y : z.x) * d;
+            const double alpha = fma(rho.x, iq, (c ? rho.y : -rho.y) * __shfl_xor_sync(0xffffffffu, iq, 1));
+            if (l < 2) {
+                par_put(S.iq, c, iq);
+                par_put(S.calpha, c, (R)alpha);
+            }
         });
         if (S.status != SEG_ACTIVE) break;
         R sn = 0;
@@ -792,35 +796,55 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             par_output<true>(g, V, sm, q4);
         }
         q4[1].y = sn;                           // the deferred ||s||^2 rides in the unused slot
-        par_sum(q4, xs, slot, [&](const double2 (&q)[4]) {
-            const double2 ts = q[0], rs = q[2], rt = q[3];
-            const double tt = q[1].x, sn2 = q[1].y;
-            if (sn2 <= S.tol2) {
+        // omega = <t, s> / ||t||^2, rho, ||r||^2 and beta: with alpha = rho_prev / <rhat, v>, beta = (rho / rho_prev)
+        // (alpha / omega) = (rho / omega) iq = (<rhat, s> / omega - <rhat, t>) iq. Lanes 0, 1: rho; 2, 3: beta;
+        // 4: ||r||^2 (15 FP64 instructions a warp where one thread's scalars took about 60 and 1.3 us).
+        par_sum<NW>(q4, xs, slot, [&](const double2* q, int l) {
+            const double2 ts = q[0], rs = q[2], rt = q[3], iq = S.iq;
+            const double tt = q[1].x, sn2 = q[1].y, tol2 = S.tol2;
+            const int c = l & 1, g = l >> 1;
+            const double d = 1.0 / (c ? ts.x * ts.x + ts.y * ts.y : tt);
+            const double itt = par_lane(d, 0), inn = par_lane(d, 1);
+            const double m = (g == 1 ? tt : c ? ts.y : ts.x) * (g == 1 ? inn : itt);     // omega; tt / |ts|^2
+            const double ox = par_lane(m, 0), oy = par_lane(m, 1), io = par_lane(m, 2);
+            const double w = (c ? -ts.y : ts.x) * io;                                    // 1 / omega
+            const double wx = par_lane(w, 0), wy = par_lane(w, 1);
+            const double base = g == 0 ? (c ? rs.y : rs.x) : g == 1 ? (c ? -rt.y : -rt.x) : sn2;
+            const double m1 = g == 0 ? -ox : g == 1 ? rs.x : -ts.x;
+            const double k1 = g == 0 ? (c ? rt.y : rt.x) : g == 1 ? (c ? wy : wx) : ox;
+            const double m2 = g == 0 ? (c ? -oy : oy) : g == 1 ? (c ? rs.y : -rs.y) : -ts.y;
+            const double k2 = g == 0 ? (c ? rt.x : rt.y) : g == 1 ? (c ? wx : wy) : oy;
+            const double v = fma(m2, k2, fma(m1, k1, base));                             // rho; rho / omega; ||r||^2
+            const double beta = fma(v, iq.x, (c ? iq.y : -iq.y) * __shfl_xor_sync(0xffffffffu, v, 1));
+            const double rhox = par_lane(v, 0), rhoy = par_lane(v, 1);
+            double res2 = par_lane(v, 4);
+            if ((unsigned)__double2hiint(res2) > 0x7ff00000u) res2 = 0.0;               // negative or NaN (fmax)
+            const R coef = (R)(g == 0 ? m : beta);
+            const unsigned le = __ballot_sync(0xffffffffu, (l == 0 ? sn2 : l == 1 ? res2 : tt) <= (l < 2 ? tol2 : 0.0));
+            if (le & 1u) {
                 S.half = 1;
                 S.res2 = sn2;
-                S.iters += 0.5;
+                if (l == 0) S.halves += 1;
                 S.status = SEG_CONVERGED;
                 return;
             }
-            if (!(tt > 0.0) || !isfinite(tt)) {
+            if ((le & 4u) || !par_finite(tt)) {
                 S.status = SEG_BREAKDOWN;
                 return;
             }
-            const double itt = 1.0 / tt;
-            const double2 omega = make_double2(ts.x * itt, ts.y * itt), rho_prev = S.rho, alpha = S.alpha;
-            const double2 rho = make_double2(rs.x - (omega.x * rt.x - omega.y * rt.y),
-                                             rs.y - (omega.x * rt.y + omega.y * rt.x));
-            const double res2 = fmax(sn2 - (ts.x * omega.x + ts.y * omega.y), 0.0);
-            S.omega = omega;
-            S.comega = cmk<C>(omega.x, omega.y);
+            if (g == 0) {
+                par_put(S.comega, c, coef);
+                par_put(S.rho, c, v);
+            } else if (g == 1) {
+                par_put(S.cbeta, c, coef);
+            }
             S.pend = 1;
-            S.rho = rho;
             S.res2 = res2;
-            S.iters += 1.0;
-            if (!isfinite(res2)) S.status = SEG_BREAKDOWN;
-            else if (res2 <= S.tol2) S.status = SEG_CONVERGED;
-            else if (omega.x == 0.0 && omega.y == 0.0) S.status = SEG_BREAKDOWN;
-            else par_beta(S, rho, rho_prev, alpha, omega);
+            if (l == 0) S.halves += 2;
+            if (!par_finite(res2)) S.status = SEG_BREAKDOWN;
+            else if (le & 2u) S.status = SEG_CONVERGED;
+            else if ((par_zero(ox) && par_zero(oy)) || !par_finite(rhox) || !par_finite(rhoy) || (par_zero(rhox) && par_zero(rhoy)))
+                S.status = SEG_BREAKDOWN;
         });
     }
     // x of a half step (x += alpha p) or of the last full step (no p update followed it)
@@ -835,7 +859,7 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
         SegState& St = g.st[b];
         St.bnorm2 = S.bn2;
         St.res2 = S.res2;
-        St.iters = S.iters;
+        St.iters = 0.5 * S.halves;
         St.status = S.status == SEG_ACTIVE ? SEG_MAXIT : S.status;
         St.maxit = maxit;
     }
