@@ -34,6 +34,28 @@ int cuda_fail(cudaError_t e, const char* what, const char* file, int line) {
     return fail(VIE_ECUDA, m);
 }
 
+// ---------------------------------------------------------------- dynamic shared memory opt-in
+int raise_dynamic_smem(const void* kernel, size_t bytes) {
+    struct Entry {
+        const void* kernel;
+        int dev;
+        size_t bytes;
+    };
+    constexpr int kEntries = 4096;              // kernels x devices; about 100 kernels opt in
+    static std::mutex mu;
+    static Entry tab[kEntries];
+    static int used = 0;
+    int dev = 0, i = 0;
+    VIE_CK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    while (i < used && (tab[i].kernel != kernel || tab[i].dev != dev)) ++i;
+    if (i < used && tab[i].bytes >= bytes) return VIE_OK;
+    VIE_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    if (i == used && used < kEntries) ++used;
+    if (i < used) tab[i] = Entry{kernel, dev, bytes};
+    return VIE_OK;
+}
+
 // ---------------------------------------------------------------- twiddles (per device)
 static std::mutex g_tw_mutex;
 static std::map<int, Twiddles> g_tw;

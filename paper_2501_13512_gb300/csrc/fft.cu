@@ -849,11 +849,7 @@ template <> const float2* tw_ptr<float2>(const Twiddles& t) { return t.d64; }
 
 template <class K>
 static int prep_smem(K kernel, size_t bytes) {
-    if (bytes > 46 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute", __FILE__, __LINE__);
-    }
-    return VIE_OK;
+    return bytes > 46 * 1024 ? raise_dynamic_smem(reinterpret_cast<const void*>(kernel), bytes) : VIE_OK;
 }
 
 struct Prof {

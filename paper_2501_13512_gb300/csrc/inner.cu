@@ -668,8 +668,8 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
     // one block per cluster of R CTAs; as many clusters as fit at once, pulling blocks from the queue
     auto launch = [&](const int2* work, int n, int* next, int R, cudaStream_t st, int* units) -> int {
         if (any_par) R = kParRanks;
-        // opt in to the exact dynamic size: the default 48 KB limit also counts the static shared memory
-        VIE_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // whatever the size: the default 48 KB limit also counts the static shared memory
+        VIE_TRY(raise_dynamic_smem(reinterpret_cast<const void*>(kern), smem));
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = R;

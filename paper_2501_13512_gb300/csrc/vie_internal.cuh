@@ -144,6 +144,11 @@ __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
 }
+// Opt-in of a kernel to dynamic shared memory of up to bytes on the current device. The limit is shared by all
+// threads of the process, which launch the same kernel with different sizes, so it is only ever raised: set to
+// the size of each launch, one thread could lower it between another's call and launch.
+int raise_dynamic_smem(const void* kernel, size_t bytes);
+
 template <class... P, class... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchAttribute attr[1];
