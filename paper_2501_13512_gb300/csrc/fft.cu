@@ -16,7 +16,9 @@
 //   pass Y' inverse, keep y < by                             -> w1
 //   pass X' inverse, keep x < bx, y = x - u (masked)         -> y
 // Each pass stages a tile of pencils in shared memory; global accesses are
-// along the contiguous x axis in every pass.
+// along the contiguous x axis in every pass. Most lengths use the two-step
+// register transforms of fft_plane.cuh (which also joins x and y of small
+// planes) and the z passes below; the radix-4 kernels take the rest.
 #include <algorithm>
 #include <type_traits>
 
@@ -289,8 +291,8 @@ template <int LZ, bool OCT>
 __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
     pdl_wait();
     typedef float2 F;
-    constexpr int H = LZ / 2 > 0 ? LZ / 2 : 1;
-    constexpr int LGZ = ILog2<LZ>::v;
+    constexpr int H = LZ / 2, LGZ = ILog2<LZ>::v;
+    static_assert(LZ >= 4, "shorter axes use k_zgreen");
     constexpr int NC = kZRegCols;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     F* sm = reinterpret_cast<F*>(smem_raw);          // [3][LZ][NC]
@@ -302,32 +304,25 @@ __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
     F* W = a.w + (int64_t)b * a.box_stride + c0;
     const int64_t cs = a.comp_stride;
     const int comp = t / NC, c = t - comp * NC;
-    {
-        if (c < nc) {
-            const F* src = W + comp * cs + c;
-            F* S = sm + comp * LZ * NC + c;
-            if (LZ == 1) {
-                S[0] = src[0];
-            } else {
-                F v[H];
+    F* S = sm + comp * LZ * NC + c;
+    // (radix 2: with the radix-4 transforms of dft_small.cuh 72 us in place of 68 at 256x256x16)
+    if (c < nc) {
+        const F* src = W + comp * cs + c;
+        F v[H], q[H];
 #pragma unroll
-                for (int j = 0; j < H; ++j) v[j] = j < bz ? src[(int64_t)j * P] : czero<F>();
-                F q[H];
+        for (int j = 0; j < H; ++j) v[j] = j < bz ? src[(int64_t)j * P] : czero<F>();
 #pragma unroll
-                for (int j = 0; j < H; ++j) q[j] = twc<true>(v[j], j * (kLmax / LZ));
-                rfft<H, true>(q, (const F*)nullptr);
+        for (int j = 0; j < H; ++j) q[j] = twc<true>(v[j], j * (kLmax / LZ));
+        rfft<H, true>(q, (const F*)nullptr);
 #pragma unroll
-                for (int j = 0; j < H; ++j) S[(H + j) * NC] = q[j];
-                rfft<H, true>(v, (const F*)nullptr);
+        for (int m = 0; m < H; ++m) S[(H + m) * NC] = q[m];
+        rfft<H, true>(v, (const F*)nullptr);
 #pragma unroll
-                for (int j = 0; j < H; ++j) S[j * NC] = v[j];
-            }
-        }
+        for (int m = 0; m < H; ++m) S[m * NC] = v[m];
     }
     // Green multiply: thread (comp, c) takes the frequencies f = comp, comp + 3, ... <= LZ / 2 of column c
     // and their mirrors, the spectrum entries of ZU frequencies in flight at once (the first ones before the wait).
-    constexpr int NF = (LZ / 2 + 1 + 2) / 3, cst = LZ * NC;
-    constexpr int ZU = NF < 2 ? NF : 2;
+    constexpr int NF = (LZ / 2 + 1 + 2) / 3, cst = LZ * NC, ZU = NF < 2 ? NF : 2;
     const ZColumn<F, OCT> zc(a, b, c0 + (c < nc ? c : 0));
 #pragma unroll
     for (int k0 = 0; k0 < NF; k0 += ZU) {
@@ -335,8 +330,8 @@ __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
 #pragma unroll
         for (int k = 0; k < ZU; ++k) {
             const int f = min(comp + 3 * (k0 + k), LZ / 2);
-            const int i = LGZ ? (int)(__brev((unsigned)f) >> (32 - LGZ)) : 0;
-            const int q = !OCT ? i : f == LZ / 2 ? LZ / 2 : LGZ >= 2 ? (int)(__brev((unsigned)f) >> (33 - LGZ)) : 0;
+            const int i = (int)(__brev((unsigned)f) >> (32 - LGZ));
+            const int q = !OCT ? i : f == LZ / 2 ? LZ / 2 : (int)(__brev((unsigned)f) >> (33 - LGZ));
             zc.load(e[k], q, a.gcomp);
         }
         if (k0 == 0) __syncthreads();
@@ -344,8 +339,8 @@ __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
         for (int k = 0; k < ZU; ++k) {
             const int f = comp + 3 * (k0 + k);
             if (c >= nc || f > LZ / 2) continue;
-            const int i = LGZ ? (int)(__brev((unsigned)f) >> (32 - LGZ)) : 0;
-            const int im = LGZ ? (int)(__brev((unsigned)((LZ - f) & (LZ - 1))) >> (32 - LGZ)) : 0;
+            const int i = (int)(__brev((unsigned)f) >> (32 - LGZ));
+            const int im = (int)(__brev((unsigned)((LZ - f) & (LZ - 1))) >> (32 - LGZ));
             F* q = sm + i * NC + c;
             F X = q[0], Y = q[cst], Z = q[2 * cst];
             green3<2, false>(X, Y, Z, e[k]);
@@ -363,26 +358,18 @@ __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
         }
     }
     __syncthreads();
-    {
-        if (c < nc) {
-            F* S = sm + comp * LZ * NC + c;
-            F* dst = W + comp * cs + c;
-            if (LZ == 1) {
-                dst[0] = S[0];
-            } else {
-                F u[H], v[H];
+    if (c >= nc) return;
+    F* dst = W + comp * cs + c;
+    F u[H], v[H];
 #pragma unroll
-                for (int j = 0; j < H; ++j) v[j] = S[(H + j) * NC];
-                rfft<H, false>(v, (const F*)nullptr);
+    for (int m = 0; m < H; ++m) v[m] = S[(H + m) * NC];
+    rfft<H, false>(v, (const F*)nullptr);
 #pragma unroll
-                for (int j = 0; j < H; ++j) u[j] = S[j * NC];
-                rfft<H, false>(u, (const F*)nullptr);
+    for (int m = 0; m < H; ++m) u[m] = S[m * NC];
+    rfft<H, false>(u, (const F*)nullptr);
 #pragma unroll
-                for (int j = 0; j < H; ++j)
-                    if (j < bz) dst[(int64_t)j * P] = u[j] + twc<false>(v[j], j * (kLmax / LZ));
-            }
-        }
-    }
+    for (int j = 0; j < H; ++j)
+        if (j < bz) dst[(int64_t)j * P] = u[j] + twc<false>(v[j], j * (kLmax / LZ));
 }
 
 // exp(-2 pi i m / 1024) at a compile-time m, times or conjugated times v.
@@ -771,7 +758,6 @@ constexpr int kCols4 = 16;   // columns per CTA (512 threads: 16 columns x 32)
 template <int A, bool FWD>
 __global__ void __launch_bounds__(512) k_cols4(ColArgs<float2> a) {
     pdl_wait();
-    constexpr int L = kB4 * A;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* sm = reinterpret_cast<float2*>(smem_raw);     // [L][kCols4]
     const int col0 = blockIdx.x * kCols4;

@@ -1,7 +1,7 @@
-// Register-resident FFTs shared by the full-grid z pass (fft.cu) and the
-// persistent block solver (inner.cu). Each translation unit that includes
-// this header has its own constant-memory twiddle table and calls
-// reg_twiddles_ready() on the host before its first launch that uses them.
+// Register-resident radix-2 FFTs of the complex64 passes (fft.cu). The
+// translation unit that includes this header has its own constant-memory
+// twiddle table and calls reg_twiddles_ready() on the host before its first
+// launch that uses them.
 #pragma once
 
 #include <algorithm>
@@ -98,59 +98,6 @@ template <> struct TwSel<float2> {
         return twc<FWD>(v, m);
     }
 };
-
-// Pruned transforms. A box of b voxels is padded to L >= 2b - 1, a power of
-// two, so b <= L/2: forward inputs beyond L/2 are zero and inverse outputs
-// beyond L/2 are discarded. The first DIF stage then splits the L-point
-// transform into FFT_{L/2}(x) (positions [0, L/2)) and FFT_{L/2}(x_j W_L^j)
-// (positions [L/2, L)); the last DIT stage of the inverse combines
-// u = iFFT_{L/2}(lower half) and v = iFFT_{L/2}(upper half) as
-// u_j + conj(W_L^j) v_j. Only L/2 values are live in registers at a time.
-
-// Forward: get(j) gives input j < L/2 (zero where the box ends); put(k, v)
-// receives output position k (bit-reversed order).
-template <int L, class Get, class Put>
-__device__ __forceinline__ void fwd_half(Get get, Put put, const F* __restrict__ tw) {
-    if (L == 1) {
-        put(0, get(0));
-        return;
-    }
-    constexpr int H = L / 2 > 0 ? L / 2 : 1;
-    F a[H];
-#pragma unroll
-    for (int j = 0; j < H; ++j) a[j] = twc<true>(get(j), j * (kLmax / L));
-    rfft<H, true>(a, tw);
-#pragma unroll
-    for (int j = 0; j < H; ++j) put(H + j, a[j]);
-#pragma unroll
-    for (int j = 0; j < H; ++j) a[j] = get(j);
-    rfft<H, true>(a, tw);
-#pragma unroll
-    for (int j = 0; j < H; ++j) put(j, a[j]);
-}
-
-// Inverse keeping outputs [0, L/2): get(k) gives input position k;
-// stash(j, v) / unstash(j) hold conj(W_L^j) v_j between the two halves;
-// put(j, v) receives output j (called for every j < L/2).
-template <int L, class Get, class Stash, class Unstash, class Put>
-__device__ __forceinline__ void inv_half(Get get, Stash stash, Unstash unstash, Put put, const F* __restrict__ tw) {
-    if (L == 1) {
-        put(0, get(0));
-        return;
-    }
-    constexpr int H = L / 2 > 0 ? L / 2 : 1;
-    F a[H];
-#pragma unroll
-    for (int j = 0; j < H; ++j) a[j] = get(H + j);
-    rfft<H, false>(a, tw);
-#pragma unroll
-    for (int j = 0; j < H; ++j) stash(j, twc<false>(a[j], j * (kLmax / L)));
-#pragma unroll
-    for (int j = 0; j < H; ++j) a[j] = get(j);
-    rfft<H, false>(a, tw);
-#pragma unroll
-    for (int j = 0; j < H; ++j) put(j, a[j] + unstash(j));
-}
 
 // Copies the complex64 twiddles into this translation unit's constant table, once per device.
 static int reg_twiddles_ready(const Twiddles& tw) {

@@ -59,7 +59,6 @@ template <class C> struct InnerGroup {
 
 constexpr int kInnerThreads = 256;
 
-
 __device__ __forceinline__ double2 dcdiv(double2 a, double2 b) {
     double d = b.x * b.x + b.y * b.y;
     return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
@@ -96,11 +95,10 @@ template <class T> __device__ __forceinline__ T shfl_dn(T v, int o) { return __s
 // computes identical sums. Two rank slots alternate between consecutive sums: a
 // slot is rewritten two sums later, after every rank has passed the cluster
 // barrier of the sum in between, so one cluster barrier per sum suffices.
-constexpr int kTeamSumMax = 4;                 // complex values one team sum carries
-
-template <int N, class C, class Fn>
-__device__ __forceinline__ void team_sum_n(C (&v)[N], double2* red, Fn fn) {
-    static_assert(N <= kTeamSumMax, "team_sum_n: too many values");
+template <class C, class Fn>
+__device__ __forceinline__ void team_sum(C a, C b, double2* red, Fn fn) {
+    constexpr int N = 2;
+    C v[N] = {a, b};
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -115,7 +113,7 @@ __device__ __forceinline__ void team_sum_n(C (&v)[N], double2* red, Fn fn) {
     __syncthreads();
     cg::cluster_group cl = cg::this_cluster();
     const unsigned R = cl.num_blocks();
-    __shared__ double2 xred[2][kTeamSumMax];
+    __shared__ double2 xred[2][N];
     double2 sum[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) sum[i] = make_double2(0, 0);
@@ -147,14 +145,8 @@ __device__ __forceinline__ void team_sum_n(C (&v)[N], double2* red, Fn fn) {
             }
         }
     }
-    if (threadIdx.x == 0) fn(sum);
+    if (threadIdx.x == 0) fn(sum[0], sum[1]);
     __syncthreads();
-}
-
-template <class C, class Fn>
-__device__ __forceinline__ void team_sum(C a, C b, double2* red, Fn fn) {
-    C v[2] = {a, b};
-    team_sum_n<2>(v, red, [&](const double2 (&s)[2]) { fn(s[0], s[1]); });
 }
 
 enum { IN_P = 0, IN_S = 1 };
@@ -498,7 +490,7 @@ __global__ void __launch_bounds__((inner_threads<C, PAR>()), (PAR == PAR_NONE ? 
             int* units) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* sm = reinterpret_cast<C*>(smem_raw);
-    __shared__ double2 red[kTeamSumMax * (inner_threads<C, PAR>() / 32)];   // per-warp sums
+    __shared__ double2 red[2 * (inner_threads<C, PAR>() / 32)];   // per-warp sums
     __shared__ int item;
     cg::cluster_group cl = cg::this_cluster();
     if (threadIdx.x == 0) team_slot = 0;
