@@ -36,9 +36,9 @@ namespace vie {
 
 constexpr int kParRanks = 4;
 // Two shapes in complex64. On chip: one CTA of 12 warps per SM, the Krylov vectors and the rank's spectrum in
-// shared memory: the shortest iteration of a block (28.6 us for a 12 x 12 x 16 box, 36 us in the other
+// shared memory: the shortest iteration of a block (26.4 us for a 12 x 12 x 16 box, 33 us in the other
 // shape). L2: two CTAs of 6 warps per SM, which hide each other's barriers, vectors in L2: the higher rate
-// when many blocks queue (0.61 us per block iteration of the 256 metasurface pillars against 0.75).
+// when many blocks queue (0.52 us per block iteration of the 256 metasurface pillars against 0.65).
 // complex128 (FP64-bound): one CTA of 8 warps of 255 registers. The row stage pairs warps: a multiple of 64.
 template <class C, bool CHIP> __host__ __device__ constexpr int par_threads() {
     return sizeof(C) == 16 ? 256 : CHIP ? 384 : 192;
