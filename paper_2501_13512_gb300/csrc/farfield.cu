@@ -5,9 +5,16 @@
 //   sigma(u) = k0^4 / (4 pi) |(I - u u) P(u)|^2
 // over voxel centres r_j = ((i + 1/2) h - n h / 2) per axis. The phase is
 // separable, exp(j k0 (ux x + uy y + uz z)) = ex(x) ey(y) ez(z), so each CTA
-// (one direction, one slab of z planes) tabulates the three 1D factors in
-// shared memory and the voxel loop is two complex multiplies per voxel;
-// partial sums are FP64 and are added on the host in a fixed order.
+// (ND directions, one slab of z planes) tabulates the three 1D factors in
+// shared memory; partial sums are FP64 and are added on the host in a fixed
+// order.
+//
+// Bound by the FP64 units. A thread sums along one axis (y, or z within the
+// slab where that is longer) with that axis's factor alone and applies the
+// other two factors once per line, and forms chi E once for its ND directions:
+// 12 + 12 / ND FP64 instructions per voxel and direction in place of 30
+// (64^3 voxels, 181 directions 2.92 -> 1.52 ms; 256 x 256 x 16, 361
+// directions 20.6 -> 10.2 ms, on the host with the read-back).
 #include <math.h>
 
 #include <algorithm>
@@ -22,57 +29,107 @@ namespace {
 constexpr int kFfThreads = 256;
 constexpr int kFfSlabs = 16;   // z slabs per direction (CTAs per direction)
 
+// acc += a b
+__device__ __forceinline__ void cfma_acc(double2& acc, double2 a, double2 b) {
+    acc.x = fma(-a.y, b.y, fma(a.x, b.x, acc.x));
+    acc.y = fma(a.y, b.x, fma(a.x, b.y, acc.y));
+}
+
+template <int ND>
 __global__ void __launch_bounds__(kFfThreads) k_far_field(const double2* E, const double2* chi, const double3* dirs,
-                                                           int nx, int ny, int nz, double h, double k0,
+                                                           int ndir, int nx, int ny, int nz, double h, double k0,
                                                            double2* partial) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* ex = reinterpret_cast<double2*>(smem_raw);    // [nx]
-    double2* ey = ex + nx;                                  // [ny]
-    double2* ez = ey + ny;                                  // [nz]
-    double2* red = ez + nz;                                 // [3][kFfThreads / 32]
-    const int d = blockIdx.x, slab = blockIdx.y;
-    const double3 u = dirs[d];
+    const int nf = nx + ny + nz;
+    double2* fac = reinterpret_cast<double2*>(smem_raw);    // [ND][ex nx | ey ny | ez nz]
+    double2* red = fac + ND * nf;                            // [ND][3][kFfThreads / 32]
+    const int d0 = blockIdx.x * ND, slab = blockIdx.y;
     const double kh = k0 * h;
-    for (int i = threadIdx.x; i < nx + ny + nz; i += blockDim.x) {
+    for (int t = threadIdx.x; t < ND * nf; t += blockDim.x) {
+        const int dd = t / nf, i = t - dd * nf;
+        const double3 u = dirs[min(d0 + dd, ndir - 1)];
         double w, n, c;
         if (i < nx) { w = u.x; n = nx; c = i; }
         else if (i < nx + ny) { w = u.y; n = ny; c = i - nx; }
         else { w = u.z; n = nz; c = i - nx - ny; }
         double sn, cs;
         sincos(kh * w * (c + 0.5 - 0.5 * n), &sn, &cs);
-        ex[i] = make_double2(cs, sn);
+        fac[t] = make_double2(cs, sn);
     }
     __syncthreads();
     const int z0 = (int)((int64_t)nz * slab / gridDim.y), z1 = (int)((int64_t)nz * (slab + 1) / gridDim.y);
     const int64_t N = (int64_t)nx * ny * nz;
     const int64_t plane = (int64_t)nx * ny;
-    double2 acc[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-    for (int64_t l = (int64_t)z0 * plane + threadIdx.x; l < (int64_t)z1 * plane; l += blockDim.x) {
-        const int z = (int)(l / plane);
-        const int64_t r = l - z * plane;
-        const int y = (int)(r / nx), x = (int)(r - (int64_t)y * nx);
-        const double2 ph = cmul(cmul(ex[x], ey[y]), ez[z]);
-        const double2 w = cmul(chi[l], ph);
+    // lines along y or z; where they are fewer than threads, each is cut into parts
+    const bool alongy = ny >= z1 - z0;
+    const int nl = alongy ? ny : z1 - z0, lines = nx * (alongy ? z1 - z0 : ny);
+    const int parts = max(1, min(nl, (int)blockDim.x / lines));
+    const int64_t step = alongy ? nx : plane;
+    double2 acc[ND][3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) acc[c] = acc[c] + cmul(w, E[c * N + l]);
+    for (int dd = 0; dd < ND; ++dd)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[dd][c] = make_double2(0, 0);
+    for (int t = threadIdx.x; t < lines * parts; t += blockDim.x) {
+        const int part = t / lines, line = t - part * lines, o = line / nx, x = line - o * nx;
+        const int64_t l0 = alongy ? (z0 + o) * plane + x : z0 * plane + (int64_t)o * nx + x;
+        const double2* fl = fac + (alongy ? nx : nx + ny + z0);                 // factor along the line
+        const double2* fo = fac + (alongy ? nx + ny + z0 : nx) + o;             // the other axis's
+        double2 sum[ND][3];
+#pragma unroll
+        for (int dd = 0; dd < ND; ++dd)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sum[dd][c] = make_double2(0, 0);
+        const int j1 = nl * (part + 1) / parts;
+        for (int j = nl * part / parts; j < j1; ++j) {
+            const int64_t l = l0 + j * step;
+            const double2 ch = chi[l];
+            const double2 w[3] = {cmul(ch, E[l]), cmul(ch, E[N + l]), cmul(ch, E[2 * N + l])};
+#pragma unroll
+            for (int dd = 0; dd < ND; ++dd) {
+                const double2 f = fl[dd * nf + j];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) cfma_acc(sum[dd][c], f, w[c]);
+            }
+        }
+#pragma unroll
+        for (int dd = 0; dd < ND; ++dd) {
+            const double2 f = cmul(fac[dd * nf + x], fo[dd * nf]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) cfma_acc(acc[dd][c], f, sum[dd][c]);
+        }
     }
-    // CTA sum in a fixed order: warp shuffles, then warp 0 over the warps
+    // CTA sums in a fixed order: warp shuffles, then one thread per component over the warps
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        double2 v = acc[c];
-        for (int o = 16; o > 0; o >>= 1) {
-            v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-            v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+    for (int dd = 0; dd < ND; ++dd) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double2 v = acc[dd][c];
+            for (int o = 16; o > 0; o >>= 1) {
+                v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+                v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+            }
+            if (lane == 0) red[(dd * 3 + c) * nw + warp] = v;
         }
-        if (lane == 0) red[c * nw + warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 3) {
+    if (threadIdx.x < 3 * ND && d0 + (int)threadIdx.x / 3 < ndir) {
         double2 v = make_double2(0, 0);
         for (int k = 0; k < nw; ++k) v = v + red[threadIdx.x * nw + k];
-        partial[((int64_t)d * gridDim.y + slab) * 3 + threadIdx.x] = v;
+        const int dd = threadIdx.x / 3, c = threadIdx.x - 3 * dd;
+        partial[((int64_t)(d0 + dd) * gridDim.y + slab) * 3 + c] = v;
     }
+}
+
+template <int ND>
+int launch_far_field(const double2* E, const double2* chi, const double3* dirs, int ndir, int slabs, int nx, int ny, int nz,
+                     double h, double k0, double2* partial, cudaStream_t s) {
+    const size_t smem = (size_t)ND * (nx + ny + nz + 3 * (kFfThreads / 32)) * sizeof(double2);
+    if (smem > 46 * 1024) VIE_TRY(raise_dynamic_smem(reinterpret_cast<const void*>(k_far_field<ND>), smem));
+    k_far_field<ND><<<dim3((ndir + ND - 1) / ND, slabs), kFfThreads, smem, s>>>(E, chi, dirs, ndir, nx, ny, nz, h, k0, partial);
+    VIE_CK(cudaGetLastError());
+    return VIE_OK;
 }
 
 }  // namespace
@@ -117,12 +174,12 @@ int far_field_rcs_impl(int nx, int ny, int nz, double h, double k0, const double
         if (e != cudaSuccess) rc = cuda_fail(e, "cudaMemcpyAsync", __FILE__, __LINE__);
     }
     if (!rc) {
-        const size_t smem = (size_t)(nx + ny + nz + 3 * (kFfThreads / 32)) * sizeof(double2);
         prof_begin(s, PK_FIELD, VIE_C128, 0, (int64_t)ndir * nx * ny * nz * 64, false);
-        k_far_field<<<dim3(ndir, slabs), kFfThreads, smem, s>>>(e_dev, wts, d_dirs, nx, ny, nz, h, k0, d_part);
+        // four directions per CTA while that leaves two CTAs for each SM (below, the last wave would be uneven)
+        rc = (int64_t)((ndir + 3) / 4) * slabs >= 2 * 152
+                 ? launch_far_field<4>(e_dev, wts, d_dirs, ndir, slabs, nx, ny, nz, h, k0, d_part, s)
+                 : launch_far_field<1>(e_dev, wts, d_dirs, ndir, slabs, nx, ny, nz, h, k0, d_part, s);
         prof_end(s);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) rc = cuda_fail(e, "k_far_field launch", __FILE__, __LINE__);
     }
     if (!rc) {
         e = cudaMemcpyAsync(part.data(), d_part, part_n * sizeof(double2), cudaMemcpyDeviceToHost, s);
