@@ -658,6 +658,8 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
     typedef typename real_of<C>::type R;
     constexpr bool STG = sizeof(C) == 8, COLS = par_by_column<C>();
     constexpr int NW = par_threads<C, CHIP>() / 32;
+    // a lone warp would wait in pair_sync for ever; par_sum has a slot for each warp, and four of them add
+    static_assert(par_threads<C, CHIP>() % 64 == 0 && NW >= 4 && NW <= kParWarpsMax, "par_solve: threads per CTA");
     __shared__ ParState<C> S;
     __shared__ ParSums<C> xs;
     __shared__ ParVecs<C, CHIP> V;
