@@ -356,10 +356,11 @@ template <class C2, class T> __device__ __forceinline__ void par_put(C2& z, int 
 
 // Scalars of the iteration, written by warp 0 inside par_sum.
 template <class C> struct ParState {
-    double2 rho, iq;                            // iq = 1 / <rhat, v>
+    double2 rho, iq, omega;                     // iq = 1 / <rhat, v>
     double tol2, bn2, res2;
     int halves;                                 // half steps done
     int status, half, pend;                     // pend: the last full step's x update is pending
+    int check;                                  // the recurrence's ||r||^2 meets the tolerance, r's own is due
     C cbeta, comega, calpha;                    // coefficients of the vector updates
 };
 
@@ -652,7 +653,9 @@ __device__ __noinline__ void par_output_cols(const InnerGroup<C>& g, const ParVe
 
 // One block's BiCGSTAB from x = 0 to ||r|| <= tol ||b|| on a cluster of kParRanks CTAs, in the merged form:
 // r = s - omega t and x += alpha p + omega s are applied in the next p update, and <rhat, r> = <rhat, s> -
-// omega <rhat, t> and ||r||^2 = ||s||^2 - |<t, s>|^2 / ||t||^2 come from the sums of the t pass.
+// omega <rhat, t> and ||r||^2 = ||s||^2 - |<t, s>|^2 / ||t||^2 come from the sums of the t pass. That difference
+// carries the rounding of ||s||^2 (in complex64 it can be negative where r is 2e-4 of s), so it only says when to
+// look: a block stops on ||r||^2 summed over r = s - omega t itself, once per solve as a rule.
 template <bool CHIP, class C>
 __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double tol, int maxit, C* sm, int* units) {
     typedef typename real_of<C>::type R;
@@ -739,6 +742,7 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
         S.res2 = bn2;
         S.half = 0;
         S.pend = 0;
+        S.check = 0;
         S.status = SEG_ACTIVE;
         if (!(bn2 > 0.0) || !isfinite(bn2)) S.status = bn2 == 0.0 ? SEG_CONVERGED : SEG_BREAKDOWN;
         else S.cbeta = cmk<C>(bn2, 0.0);        // (rho / 1) (1 / 1); p = v = 0
@@ -819,8 +823,7 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             const double v = fma(m2, k2, fma(m1, k1, base));                             // rho; rho / omega; ||r||^2
             const double beta = fma(v, iq.x, (c ? iq.y : -iq.y) * __shfl_xor_sync(0xffffffffu, v, 1));
             const double rhox = par_lane(v, 0), rhoy = par_lane(v, 1);
-            double res2 = par_lane(v, 4);
-            if ((unsigned)__double2hiint(res2) > 0x7ff00000u) res2 = 0.0;               // negative or NaN (fmax)
+            const double res2 = par_lane(v, 4);
             const R coef = (R)(g == 0 ? m : beta);
             const unsigned le = __ballot_sync(0xffffffffu, (l == 0 ? sn2 : l == 1 ? res2 : tt) <= (l < 2 ? tol2 : 0.0));
             if (le & 1u) {
@@ -836,6 +839,7 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             }
             if (g == 0) {
                 par_put(S.comega, c, coef);
+                par_put(S.omega, c, m);
                 par_put(S.rho, c, v);
             } else if (g == 1) {
                 par_put(S.cbeta, c, coef);
@@ -844,10 +848,32 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             S.res2 = res2;
             if (l == 0) S.halves += 2;
             if (!par_finite(res2)) S.status = SEG_BREAKDOWN;
-            else if (le & 2u) S.status = SEG_CONVERGED;
+            else if (le & 2u) S.check = 1;
             else if ((par_zero(ox) && par_zero(oy)) || !par_finite(rhox) || !par_finite(rhoy) || (par_zero(rhox) && par_zero(rhoy)))
                 S.status = SEG_BREAKDOWN;
         });
+        if (S.check) {
+            const C oc = S.comega;
+            q4[0] = q4[1] = q4[2] = q4[3] = czero<C>();
+            own([&](int e, int, int) {
+                const C r = V.s[e] - cmul(oc, V.t[e]);
+                acc_dot(q4[0], V.rhat[e], r);
+                q4[1].x += r.x * r.x + r.y * r.y;
+            });
+            par_sum<NW>(q4, xs, slot, [&](const double2* q, int) {
+                const double2 rho = q[0], om = S.omega;
+                S.check = 0;
+                S.res2 = q[1].x;
+                if (!par_finite(S.res2)) S.status = SEG_BREAKDOWN;
+                else if (S.res2 <= S.tol2) S.status = SEG_CONVERGED;
+                else if (!dgood(om) || !dgood(rho)) S.status = SEG_BREAKDOWN;
+                else {
+                    const double2 beta = cmul(dcdiv(rho, om), S.iq);
+                    S.rho = rho;
+                    S.cbeta = cmk<C>(beta.x, beta.y);
+                }
+            });
+        }
     }
     // x of a half step (x += alpha p) or of the last full step (no p update followed it)
     const C ac = S.calpha, oc = S.comega;
