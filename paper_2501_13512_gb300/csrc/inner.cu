@@ -379,6 +379,7 @@ __device__ __forceinline__ void solve_block(const InnerGroup<C>& g, int b, doubl
         S.half = 0;
         S.status = SEG_ACTIVE;
         if (!(bn2 > 0.0) || !isfinite(bn2)) S.status = bn2 == 0.0 ? SEG_CONVERGED : SEG_BREAKDOWN;
+        else if (bn2 <= S.tol2) S.status = SEG_CONVERGED;   // x = 0 meets a tolerance of 1 or more
         else next_beta(S);
     });
     for (int it = 0; it < maxit && S.status == SEG_ACTIVE; ++it) {

@@ -745,6 +745,7 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
         S.check = 0;
         S.status = SEG_ACTIVE;
         if (!(bn2 > 0.0) || !isfinite(bn2)) S.status = bn2 == 0.0 ? SEG_CONVERGED : SEG_BREAKDOWN;
+        else if (bn2 <= S.tol2) S.status = SEG_CONVERGED;   // x = 0 meets a tolerance of 1 or more
         else S.cbeta = cmk<C>(bn2, 0.0);        // (rho / 1) (1 / 1); p = v = 0
     });
     for (int it = 0; it < maxit && S.status == SEG_ACTIVE; ++it) {

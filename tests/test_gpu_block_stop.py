@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2501_13512_gb300 import vie
+from paper_2501_13512_gb300 import inputs, vie
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +39,21 @@ def test_block_stops_on_the_residual_itself(precision, contrast, tau):
         _, st = grid.precond(grid.spectrum(K0), b, inner_tol=tau, inner_maxit=50)
         assert st["not_converged"] == 0 and st["breakdowns"] == 0
         assert st["mean_iters"] == 1.5, inner
+
+
+@pytest.mark.parametrize("inner", [vie.INNER_AUTO, vie.INNER_BATCHED, vie.INNER_PERSISTENT])
+@pytest.mark.parametrize("ext", [(6, 5, 4), (18, 17, 4)])
+@pytest.mark.parametrize("precision", [vie.C64, vie.C128])
+def test_start_that_meets_the_tolerance_is_kept(precision, ext, inner):
+    # x = 0 leaves ||b||, within a tolerance of 1 or more: no iteration, whichever solver takes the block
+    nx, ny, nz = ext
+    eps_r, _, b = inputs.random_case((nx + 1, ny, nz), seed=3)
+    bid = np.full((nz, ny, nx + 1), -1, np.int32)
+    bid[:, :, :nx] = 0
+    b = torch.from_numpy(b).to(device="cuda", dtype=DT[precision])
+    grid = vie.Grid(eps_r, H, bid, inner=inner)
+    sp = grid.spectrum(K0)
+    for tau in (1.0, 1.5):
+        y, st = grid.precond(sp, b, inner_tol=tau)
+        assert st["max_iters"] == 0 and st["not_converged"] == 0 and st["breakdowns"] == 0
+        assert not y[..., :nx].any() and torch.equal(y[..., nx], b[..., nx])
