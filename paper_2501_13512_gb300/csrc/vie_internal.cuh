@@ -133,15 +133,15 @@ template <> __device__ __forceinline__ float2 from_c128<float2>(double2 a) { ret
 
 // ---------------------------------------------------------------- dependent launches
 // The kernels of a product and of a BiCGSTAB step follow one another on a stream and take a few microseconds
-// each on small grids. They are launched with programmatic stream serialization: a kernel's CTAs may be placed
-// while the last CTAs of its predecessor run, and wait in pdl_wait, before their first access to memory, until
-// the predecessor has finished and its writes are visible. Each kernel lets its successor be placed once its own
-// wait is over. (Plain launches -> these: 16^3 complex64 product 17.8 -> 14.6 us, preconditioner with 16 coarse
-// blocks 6.15 -> 5.46 ms, 8 particles of 24^3 15.7 -> 12.8 ms.)
+// each on small grids. They are launched with programmatic stream serialization: a kernel's launch is prepared
+// while its predecessor drains, and its CTAs wait in pdl_wait, before their first access to memory, until the
+// predecessor has finished and its writes are visible. No kernel lets its successor start before its own CTAs
+// end (griddepcontrol.launch_dependents): CTAs placed beside running ones crowd a few SMs, which cost up to
+// half of the rate where they are too few to fill the GPU several times (complex128 8x300x8 product 287 us with
+// that instruction, 160 without; 128x128x4 283 and 211; complex64 300x8x8 25.5 and 20.9, 16^3 14.6 and 13.5).
 __device__ __forceinline__ void pdl_wait() {
 #ifdef __CUDA_ARCH__
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
 }
 // Opt-in of a kernel to dynamic shared memory of up to bytes on the current device. The limit is shared by all
