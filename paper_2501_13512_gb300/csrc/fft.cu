@@ -372,6 +372,28 @@ __global__ void __launch_bounds__(kZRegThreads) k_zgreen_reg(ZArgs<float2> a) {
         if (j < bz) dst[(int64_t)j * P] = u[j] + twc<false>(v[j], j * (kLmax / LZ));
 }
 
+// Pass Z of a single plane (Mz = 1): no transform, one thread multiplies a column's three components. Bound by
+// its loads; in k_zgreen, through tiles in shared memory, the whole complex64 product of 512 x 512 x 1 voxels took
+// 98 us (50 so), complex128 859 (758).
+template <class C, bool OCT>
+__global__ void __launch_bounds__(kThreads) k_z_one(ZArgs<C> a) {
+    pdl_wait();
+    const int b = blockIdx.y;
+    if (!box_active(a.st, b)) return;
+    if (a.units != nullptr && threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(a.units, 1);
+    const int col = blockIdx.x * kThreads + threadIdx.x;
+    if (col >= a.ncols) return;
+    C* W = a.w + (int64_t)b * a.box_stride + col;
+    const ZColumn<C, OCT> zc(a, b, col);
+    C e[6];
+    zc.load(e, 0, a.gcomp);
+    C X = W[0], Y = W[a.comp_stride], Z = W[2 * a.comp_stride];
+    green3<2, false>(X, Y, Z, e);
+    W[0] = X;
+    W[a.comp_stride] = Y;
+    W[2 * a.comp_stride] = Z;
+}
+
 // exp(-2 pi i m / 1024) at a compile-time m, times or conjugated times v.
 template <bool FWD> __device__ __forceinline__ float2 ztw(float2 v, int m, const float2*) { return twc<FWD>(v, m); }
 template <bool FWD> __device__ __forceinline__ double2 ztw(double2 v, int m, const double2* tw) { return twmul<FWD>(v, m, tw); }
@@ -1007,6 +1029,16 @@ static int launch_z_four(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
 }
 
 template <class C, bool OCT>
+static int launch_z_one(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
+    dim3 grid((a.ncols + kThreads - 1) / kThreads, nb);
+    a.units = prof_begin(s, pf.kind, prec_code<C>(), pf.bpu, pf.fixed, true);
+    const cudaError_t e = launch_dependent(k_z_one<C, OCT>, grid, kThreads, 0, s, a);
+    prof_end(s);
+    VIE_CK(e);
+    return VIE_OK;
+}
+
+template <class C, bool OCT>
 static int launch_z_reg(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
     if constexpr (sizeof(C) == 8) {
         switch (a.lL) {
@@ -1035,10 +1067,11 @@ static int launch_z_reg(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
 
 template <class C>
 static int launch_zgreen(ZArgs<C> a, int nb, Prof pf, cudaStream_t s) {
-    // Register transforms for 4 to 512 points of the symmetric operator (the box fills at most half of the
-    // axis); the radix-4 form for the rest: one plane, 1024 points, the nine spectra of the rooftop operator,
+    // One plane: the multiply alone. Register transforms for 4 to 512 points of the symmetric operator (the box
+    // fills at most half of the axis); the radix-4 form for the rest: 1024 points, the nine spectra of the rooftop operator,
     // and complex128 launches of less than two warps' columns per SM, where one thread's serial FP64 work
     // (a column's parity: 84 us at 16^3 against 30 us) sets the time.
+    if (!a.nine && a.lL == 0) return a.oct ? launch_z_one<C, true>(a, nb, pf, s) : launch_z_one<C, false>(a, nb, pf, s);
     const bool few = sizeof(C) == 16 && (int64_t)a.ncols * nb < 152 * 64;
     if (!a.nine && !few && a.lL >= 2 && a.lL <= 9 && 2 * a.nzb <= (1 << a.lL))
         return a.oct ? launch_z_reg<C, true>(a, nb, pf, s) : launch_z_reg<C, false>(a, nb, pf, s);
