@@ -974,8 +974,10 @@ static int launch_cols(ColArgs<C> a, int nb1, int nb2, Prof pf, cudaStream_t s) 
             return launch_cols4<32, FWD>(a, nb1, nb2, pf, s);
         }
     }
-    // two-step register transforms: columns of 64 to 512 points, pruned to half the length
-    if (a.lL >= 6 && a.lL <= 9 &&
+    // two-step register transforms: columns of 64 to 512 points, pruned to half the length; complex128 with a full
+    // tile of columns only (one column of 64 voxels: 17 us here, 10 in the radix-4 form, whose stages spread it
+    // over all threads)
+    if (a.lL >= 6 && a.lL <= 9 && (sizeof(C) == 8 || a.ncols >= LineCols<C>::n) &&
         (FWD ? (2 * a.n_in <= (1 << a.lL) && a.n_out == (1 << a.lL)) : (2 * a.n_out <= (1 << a.lL) && a.n_in == (1 << a.lL))))
         VIE_LONG_LINE_SWITCH(a.lL, return (launch_line_cols<C, AA, BB, FWD>(a, nb1, nb2, pf, s)));
     a.ltc = pick_ltile(a.lL, sizeof(C), 1, 0);
