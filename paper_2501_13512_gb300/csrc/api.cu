@@ -84,8 +84,9 @@ int get_twiddles(Twiddles* out) {
     VIE_CK(cudaMalloc(&t.d64, kLmax * sizeof(float2)));
     VIE_CK(cudaMemcpy(t.d128, h128.data(), kLmax * sizeof(double2), cudaMemcpyHostToDevice));
     VIE_CK(cudaMemcpy(t.d64, h64.data(), kLmax * sizeof(float2), cudaMemcpyHostToDevice));
-    // copies from pageable memory may return before their DMA lands, and later kernels may run on a
-    // non-blocking stream that does not wait for the legacy stream: wait for the tables here
+    VIE_TRY(reg_twiddles_upload(t));
+    // copies from pageable memory and between device addresses may return before they land, and later kernels
+    // may run on a non-blocking stream that does not wait for the legacy stream: wait for the tables here
     VIE_CK(cudaDeviceSynchronize());
     g_tw[dev] = t;
     *out = t;

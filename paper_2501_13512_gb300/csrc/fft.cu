@@ -1122,7 +1122,6 @@ int mvm_boxes(const BoxSet& bs, const C* G, const C* x, C* y, const SegState* st
     if (twp) tw = *twp;
     else VIE_TRY(get_twiddles(&tw));
     const C* T = tw_ptr<C>(tw);
-    if (sizeof(C) == sizeof(float2)) VIE_TRY(reg_twiddles_ready(tw));   // constant table of the register passes
     C* w1 = reinterpret_cast<C*>(bs.w1);
     C* w2 = reinterpret_cast<C*>(bs.w2);
     const int64_t planeXY = (int64_t)bs.Mx * bs.My;

@@ -1,12 +1,6 @@
-// Register-resident radix-2 FFTs of the complex64 passes (fft.cu). The
-// translation unit that includes this header has its own constant-memory
-// twiddle table and calls reg_twiddles_ready() on the host before its first
-// launch that uses them.
+// Register-resident radix-2 FFTs of the complex64 passes (fft.cu), with the
+// constant-memory twiddle table that get_twiddles fills.
 #pragma once
-
-#include <algorithm>
-#include <mutex>
-#include <vector>
 
 #include "vie_internal.cuh"
 
@@ -75,7 +69,7 @@ typedef float2 F;
 
 // Twiddles W_Lmax^m of the complex64 register path in constant memory: the
 // register FFTs index them with compile-time offsets, so they become constant
-// operands instead of loads. Copied once per device before the first launch.
+// operands instead of loads.
 static __constant__ F c_tw64[kLmax];
 
 template <bool FWD>
@@ -99,17 +93,10 @@ template <> struct TwSel<float2> {
     }
 };
 
-// Copies the complex64 twiddles into this translation unit's constant table, once per device.
-static int reg_twiddles_ready(const Twiddles& tw) {
-    static std::mutex mu;
-    static std::vector<int> devs;
-    int dev = 0;
-    VIE_CK(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lock(mu);
-    if (std::find(devs.begin(), devs.end(), dev) == devs.end()) {
-        VIE_CK(cudaMemcpyToSymbol(c_tw64, tw.d64, kLmax * sizeof(float2), 0, cudaMemcpyDeviceToDevice));
-        devs.push_back(dev);
-    }
+// Copies the complex64 twiddles into the constant table of the current device (called by get_twiddles, which
+// waits for the copy).
+int reg_twiddles_upload(const Twiddles& tw) {
+    VIE_CK(cudaMemcpyToSymbol(c_tw64, tw.d64, kLmax * sizeof(float2), 0, cudaMemcpyDeviceToDevice));
     return VIE_OK;
 }
 

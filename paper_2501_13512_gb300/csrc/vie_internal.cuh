@@ -173,6 +173,7 @@ struct Twiddles {              // W_Lmax^m = exp(-2 pi i m / Lmax), m in [0, Lma
     float2* d64 = nullptr;
 };
 int get_twiddles(Twiddles* out);   // per device, created on first use
+int reg_twiddles_upload(const Twiddles& tw);   // the constant table of the register passes (fft_reg.cuh)
 
 // Counted device allocations of the library's handles (grids, spectra, batches).
 // dmalloc refuses with VIE_EBUSY, allocating nothing, when the bytes held would
