@@ -88,9 +88,11 @@ typedef struct {
 
 /* How the inner block solves of the preconditioner run (vie_grid_desc.flags).
  * AUTO: a persistent kernel in which a thread-block cluster solves whole blocks
- * on its own, for every group whose boxes are at most 16 voxels per axis
- * (parity-split MVM, on chip) and for every group whose padded (x, y) plane fits
- * in shared memory when the persistent groups hold at least 32 blocks together;
+ * on its own, for every group whose boxes are at most 16 voxels per axis (parity-
+ * split MVM, on chip; many very small boxes one CTA each) unless complex128
+ * blocks are so few or so flat that the batched launches are faster, and for every
+ * group whose padded (x, y) plane fits in shared memory when the persistent
+ * groups hold at least 32 blocks together;
  * batched multi-CTA launches per BiCGSTAB step otherwise. The two
  * paths compute the same iterations; the flags force one of them. */
 enum vie_grid_flags {
@@ -106,7 +108,8 @@ typedef struct {
     int64_t device_bytes;    /* device memory held by the grid handle              */
     int32_t inner_cluster[2];/* CTAs per block of the persistent block solver for
                                 complex128 [0] and complex64 [1]: 4 for boxes of at
-                                most 16 voxels per axis; for larger ones chosen by the
+                                most 16 voxels per axis (1 for many very small ones);
+                                for larger ones chosen by the
                                 tuner: 2 or 4 for every block, -1 for the split launch
                                 (the slowest blocks on 4 CTAs and the rest on 2);
                                 0 = not yet used or tuned                           */

@@ -306,6 +306,20 @@ extern "C" int vie_last_error(char* buf, size_t len) {
     return (int)g_last_error.size();
 }
 
+// The classes of a group whose blocks run in the parity-split MVM (else none).
+static const std::vector<ParClass>& par_classes(const Group& gr, int prec) {
+    static const std::vector<ParClass> none;
+    return gr.path[prec] == PATH_PAR ? gr.par : none;
+}
+static bool single_cta(const Group& gr, int prec) { return !gr.par.empty() && gr.path[prec] == PATH_PASSES; }
+
+// Moves the work items of single-CTA jobs to the end of the list, both kinds in their order; their number.
+static int single_items_last(const vie_grid* g, int prec, std::vector<int2>& w) {
+    auto first = std::stable_partition(w.begin(), w.end(),
+                                       [&](const int2& i) { return !single_cta(g->groups[g->job_group[prec][i.x]], prec); });
+    return (int)(w.end() - first);
+}
+
 extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
     if (!d || !out) return fail(VIE_EINVAL, "vie_grid_create: null argument");
     *out = nullptr;
@@ -532,23 +546,24 @@ extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
         for (auto& gr : g->groups)
             if (inner_persistent_ok(gr.bs, es, true)) fit_blocks += gr.bs.nb;
         const bool force = d->flags == VIE_GRID_INNER_PERSISTENT || fit_blocks >= kInnerMinBlocks;
+        choose_block_paths(g->groups, prec, d->flags == VIE_GRID_INNER_AUTO);
         for (auto& gr : g->groups) {
+            const bool may = d->flags != VIE_GRID_INNER_BATCHED && (gr.par.empty() || gr.path[prec] != PATH_BATCHED);
             // merged launches across grids take the blocks of grids with kInnerMinBlocks fitting blocks or
             // more, and complex64 blocks of the parity-split MVM (larger boxes stay batched)
-            gr.fit[prec] = d->flags != VIE_GRID_INNER_BATCHED && inner_persistent_ok(gr.bs, es, true) &&
-                           (force || (prec == 1 && !gr.par.empty()));
+            gr.fit[prec] = may && inner_persistent_ok(gr.bs, es, true) && (force || (prec == 1 && !gr.par.empty()));
             gr.last_iters[prec].assign(gr.bs.nb, 0.f);
-            bool ok = d->flags != VIE_GRID_INNER_BATCHED && inner_persistent_ok(gr.bs, es, force);
+            bool ok = may && inner_persistent_ok(gr.bs, es, force);
             (prec == 0 ? gr.persistent128 : gr.persistent64) = ok;
             if (!ok) continue;
             // one job per class of the parity-split MVM, else one for the group
             const int gidx = (int)(&gr - g->groups.data());
-            for (const ParClass& c : gr.par) {
+            for (const ParClass& c : par_classes(gr, prec)) {
                 for (int b : c.boxes) items.push_back({(int64_t)c.hx * c.hy * c.hz * 8, make_int2(job, b)});
                 g->job_group[prec].push_back(gidx);
                 ++job;
             }
-            if (gr.par.empty()) {
+            if (par_classes(gr, prec).empty()) {
                 for (int b = 0; b < gr.bs.nb; ++b) items.push_back({gr.bs.spec_elems(), make_int2(job, b)});
                 g->job_group[prec].push_back(gidx);
                 ++job;
@@ -558,6 +573,7 @@ extern "C" int vie_grid_create(const vie_grid_desc* d, vie_grid** out) {
                          [](const std::pair<int64_t, int2>& a, const std::pair<int64_t, int2>& b) { return a.first > b.first; });
         std::vector<int2> w;
         for (auto& it : items) w.push_back(it.second);
+        g->nsingle[prec] = single_items_last(g, prec, w);
         g->work_host[prec] = w;
         int2** dst = prec == 0 ? &g->work128 : &g->work64;
         (prec == 0 ? g->nwork128 : g->nwork64) = (int)w.size();
@@ -841,8 +857,9 @@ static int merged_launch(MergeCtx* mc, const std::vector<MergeReq*>& reqs) {
     });
     std::vector<int2> w(items.size());
     for (size_t k = 0; k < items.size(); ++k) w[k] = items[k].second;
+    auto single = std::stable_partition(w.begin(), w.end(), [&](const int2& i) { return !jobs[i.x].single; });
     VIE_CK(cudaMemcpyAsync(mc->d_work, w.data(), w.size() * sizeof(int2), cudaMemcpyHostToDevice, mc->ms));
-    return inner_persistent<C>(jobs, mc->d_work, (int)w.size(), mc->d_groups, mc->d_next, reqs[0]->tol,
+    return inner_persistent<C>(jobs, mc->d_work, (int)w.size(), (int)(w.end() - single), mc->d_groups, mc->d_next, reqs[0]->tol,
                                reqs[0]->maxit, mc->ms, 2, nullptr);
 }
 
@@ -948,8 +965,11 @@ static void group_jobs(vie_grid* g, const vie_spectrum* sp, int i, std::vector<I
     j.chi = chi_of<C>(gr.bs);
     j.G = spec_of<C>(sp, 1 + i);
     j.st = gr.st;
-    if (gr.par.empty()) jobs.push_back(j);
-    for (const ParClass& c : gr.par) {
+    const std::vector<ParClass>& par = par_classes(gr, prec_of<C>() == VIE_C128 ? 0 : 1);
+    j.single = single_cta(gr, prec_of<C>() == VIE_C128 ? 0 : 1);
+    if (par.empty()) jobs.push_back(j);
+    j.single = false;
+    for (const ParClass& c : par) {
         const ParSpec* p = &sp->par[i][0];
         for (const ParSpec& q : sp->par[i])
             if (q.hx == c.hx && q.hy == c.hy && q.hz == c.hz) p = &q;
@@ -962,8 +982,8 @@ static void group_jobs(vie_grid* g, const vie_spectrum* sp, int i, std::vector<I
 }
 
 // Padded points of a block's MVM, the weight of its iterations in the work order.
-static double block_weight(const Group& gr, int box) {
-    for (const ParClass& c : gr.par)
+static double block_weight(const Group& gr, int prec, int box) {
+    for (const ParClass& c : par_classes(gr, prec))
         if (std::binary_search(c.boxes.begin(), c.boxes.end(), box)) return 8.0 * c.hx * c.hy * c.hz;
     return (double)gr.bs.spec_elems();
 }
@@ -982,13 +1002,13 @@ static void grid_merge_jobs(vie_grid* g, const vie_spectrum* sp, MergeReq* r) {
         int job = (int)jobs.size();
         group_jobs<C>(g, sp, (int)i, jobs);
         auto add = [&](int b) {
-            r->items.push_back({(gr.last_iters[pi][b] + 1.0) * block_weight(gr, b), make_int2(job, b)});
+            r->items.push_back({(gr.last_iters[pi][b] + 1.0) * block_weight(gr, pi, b), make_int2(job, b)});
         };
-        for (const ParClass& c : gr.par) {
+        for (const ParClass& c : par_classes(gr, pi)) {
             for (int b : c.boxes) add(b);
             ++job;
         }
-        if (gr.par.empty())
+        if (par_classes(gr, pi).empty())
             for (int b = 0; b < gr.bs.nb; ++b) add(b);
     }
 }
@@ -1038,19 +1058,23 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
         merge_arrive(mm, &req);
         guard.armed = true;
     }
-    // Launch shape: the parity-split MVM runs on clusters of 4 CTAs. Without such jobs it is tuned on the
-    // first applies: 2 and 4 CTAs per block, then the split launch (the slowest blocks of the previous
+    // Launch shape: the parity-split MVM runs on clusters of 4 CTAs, and boxes over 16 voxels with it (64 boxes of
+    // 24 x 24 x 6 in complex128 with one of 8 x 8 x 8: 126 ms so, 211 in a launch of their own). Without such jobs it is
+    // tuned on the first applies: 2 and 4 CTAs per block, then the split launch (the slowest blocks of the previous
     // apply on 4 CTAs, the rest on 2), then the best.
-    bool par = false;
-    for (const InnerJob<C>& j : jobs) par = par || j.hx > 0;
+    bool par = false, passes = false;
+    for (const InnerJob<C>& j : jobs) {
+        par = par || j.hx > 0;
+        passes = passes || (j.hx == 0 && !j.single);
+    }
     static const int kCand[3] = {2, 4, -1};
     const int ncand = 3;
     const int pi = c128 ? 0 : 1;
-    if (par) g->tune_best[pi] = 4;
+    if (!jobs.empty() && (par || !passes)) g->tune_best[pi] = par ? 4 : 1;
     // the first apply only warms up (first launches of the kernel pay one-time costs that would bias
     // the candidate tried first); the candidates follow, one per apply
     const int tried = g->tune_count[pi] - 1;
-    const bool tuning = !jobs.empty() && !par && tried < ncand && !inner_cluster_forced();
+    const bool tuning = passes && !par && tried < ncand && !inner_cluster_forced();
     const int choice = tuning ? kCand[std::max(tried, 0)] : (g->tune_best[pi] ? g->tune_best[pi] : 2);
     // with batched groups as well, the persistent launch runs on the grid's second stream beside
     // the batched steps (no split launch then)
@@ -1068,7 +1092,7 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
         sp_stream = g->s2;
     }
     if (tuning) VIE_CK(cudaEventRecord(g->tev[0], sp_stream));
-    VIE_TRY(inner_persistent<C>(jobs, c128 ? g->work128 : g->work64, c128 ? g->nwork128 : g->nwork64,
+    VIE_TRY(inner_persistent<C>(jobs, c128 ? g->work128 : g->work64, c128 ? g->nwork128 : g->nwork64, g->nsingle[pi],
                                 g->inner_groups, g->inner_next, tol, maxit, sp_stream,
                                 choice == -1 ? 2 : choice, &split));
     if (tuning) VIE_CK(cudaEventRecord(g->tev[1], sp_stream));
@@ -1152,11 +1176,12 @@ static int precond_apply(vie_grid* g, const vie_spectrum* sp, const C* b, C* y, 
             items.reserve(wh.size());
             for (const int2& w : wh) {
                 const Group& gr = g->groups[jg[w.x]];
-                items.push_back({(hs[jg[w.x]][w.y].iters + 1.0) * block_weight(gr, w.y), w});
+                items.push_back({(hs[jg[w.x]][w.y].iters + 1.0) * block_weight(gr, pi, w.y), w});
             }
             std::stable_sort(items.begin(), items.end(), [](const std::pair<double, int2>& a,
                                                             const std::pair<double, int2>& b) { return a.first > b.first; });
             for (size_t k = 0; k < items.size(); ++k) wh[k] = items[k].second;
+            single_items_last(g, pi, wh);
             // heavy part of a split launch: blocks that took at least 0.6 of the largest iteration
             // count, at most an eighth of the blocks (measured on the metasurface: 0.5 / 4, 0.75 / 16
             // and 0.9 / 32 were slower)

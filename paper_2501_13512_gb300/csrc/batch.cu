@@ -430,7 +430,7 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
                 merge_arrive(mm, &req);
                 VIE_TRY(merge_wait(mm, &req, s));
             } else {
-                VIE_TRY(inner_persistent<float2>(jobs, b->work, nb, b->inner_groups, b->inner_next, 0.5,
+                VIE_TRY(inner_persistent<float2>(jobs, b->work, nb, 0, b->inner_groups, b->inner_next, 0.5,
                                                  o->outer_maxit, s));
             }
         } else {

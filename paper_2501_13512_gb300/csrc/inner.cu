@@ -584,14 +584,80 @@ bool inner_persistent_ok(const BoxSet& bs, size_t es, bool force) {
     return par_path_ok(bs) || ((force || bs.nb >= kInnerMinBlocks) && inner_tiles(bs, es, &a, &b, &s));
 }
 
+// FP64 instructions per thread of an H-point transform (dft_small.cuh)
+static double dft_ops(int h) {
+    return h == 2 ? 4 : h == 4 ? 16 : h == 6 ? 44 : h == 8 ? 56 : h == 10 || h == 12 ? 112 : 168;
+}
+static int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+// Microseconds of a complex128 iteration of one block in the parity-split solver: the FP64 instructions of the
+// fullest SM quarter (rows of a warp pair, y columns, z columns with the vector updates) over two products, at 64
+// clocks each. Within 10 % of the measured time from 4 x 16 x 4 (89 us) to 16 x 16 x 16 voxels (900 us).
+static double par_iter_us(const ParClass& c) {
+    const double row = ceil_div(ceil_div(c.hz * c.hy, 32), 2) * (6 * dft_ops(c.hx) + 60.0 * c.hx);
+    const double y = ceil_div(3 * c.hz * c.ex, 128) * (2 * dft_ops(c.hy) + 8.0 * c.hy);
+    const double z = ceil_div(3 * c.ex * c.ey, 512) * (4 * dft_ops(c.hz) + 50.0 * c.hz);
+    return std::max(40.0, 0.07 * (row + y + z));
+}
+
+// Groups of boxes of at most 16 voxels per axis, by the time of an iteration of all their blocks.
+// complex64: the parity-split solver is the fastest way at every number of blocks from 3 x 3 x 3 voxels up (1 to 512
+// blocks of 28 shapes). Boxes of up to 128 padded points (2 x 2 x 2, 16 x 1 x 1) use little of a cluster: once
+// they outnumber the 152 clusters in flight, one CTA each in the shared-memory passes is faster (4096 blocks of one
+// voxel 0.43 against 1.16 ms, 1024 of 2 x 2 x 2 0.34 against 0.69).
+// complex128 is bound by the FP64 units, so what counts is how many SMs work:
+//   parity-split  38 blocks at a time, each on 4 SMs, no padding: par_iter_us, longer from 48 blocks on;
+//   batched       every SM, on padded boxes, a group after the other: 75 us, at least 120, plus per
+//                 block 0.1 us and 0.51 (rows of more than 12 voxels) or 0.66 us per 1000 padded points;
+//   passes        one CTA per block on padded boxes, 150 at a time: 40 us + 0.13 per padded point.
+// The factors are fitted to 28 shapes at 1 to 512 blocks, with equal iterations and converged: the chosen way takes
+// 3 % more than the fastest of the three on average, and more than 4 % longer than both the parity-split solver and
+// the solver that came before it in none of them. (One 12 x 12 x 16 block 15.3 -> 4.3 ms, 1024 of 4 x 4 x 4
+// 12.3 -> 3.1, 256 of 16 x 16 x 2 16.6 -> 7.2.)
+void choose_block_paths(std::vector<Group>& groups, int prec, bool batched) {
+    const double per_wave = 38.0;
+    int nsmall = 0;
+    const int64_t small_points = prec == 1 ? 128 : 2048;
+    auto small = [&](const Group& g) { return !g.par.empty() && g.bs.spec_elems() <= small_points; };
+    for (const Group& g : groups)
+        if (small(g)) nsmall += g.bs.nb;
+    double t_par_block = 0.0, t_par_sum = 0.0, t_batched = 0.0;
+    for (Group& g : groups) {
+        if (g.par.empty()) continue;
+        g.path[prec] = PATH_PAR;
+        if (prec == 1) {
+            if (small(g) && nsmall > 152) g.path[prec] = PATH_PASSES;
+            continue;
+        }
+        const double points = (double)g.bs.spec_elems();
+        const double tb = std::max(120.0, 75.0 + g.bs.nb * (0.1 + (g.bs.bx > 12 ? 5.1e-4 : 6.6e-4) * points));
+        double tp = 0.0, sum = 0.0;
+        for (const ParClass& c : g.par) {
+            tp = std::max(tp, par_iter_us(c));
+            sum += par_iter_us(c) * (double)c.boxes.size();
+        }
+        const double ts = (40.0 + 0.13 * points) * std::max(1.0, nsmall / 150.0);
+        if (small(g) && ts < 1.2 * std::min(tp * std::ceil(nsmall / per_wave), batched ? 1.1 * tb : 1e30)) {
+            g.path[prec] = PATH_PASSES;
+            continue;
+        }
+        t_par_block = std::max(t_par_block, tp);
+        t_par_sum += sum;
+        t_batched += tb;
+    }
+    if (batched && 1.1 * t_batched < std::max(t_par_block, 0.85 * t_par_sum / per_wave))
+        for (Group& g : groups)
+            if (!g.par.empty() && g.path[prec] == PATH_PAR) g.path[prec] = PATH_BATCHED;
+}
+
 template <class C>
-int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, int nwork, void* d_groups,
+int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, int nwork, int nsingle, void* d_groups,
                      int* d_next, double tol, int maxit, cudaStream_t s, int cluster, const InnerSplit* split) {
     if (jobs.empty() || nwork == 0) return VIE_OK;
     Twiddles tw;
     VIE_TRY(get_twiddles(&tw));
     std::vector<InnerGroup<C>> hg(jobs.size());
-    size_t smem = 0;
+    size_t smem = 0, single_smem = 0;
     bool any_par = false;
     size_t chip_smem = 0;
     for (size_t i = 0; i < jobs.size(); ++i) {
@@ -639,15 +705,17 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
                                   : 4 * w2b + 6LL * bs.spec_elems() * es + box * (es + 1) + 4 * 3 * box * es;
         g.kb_mvm = (int)((mvm + 1023) / 1024);
         g.kb_upd = (int)((6 * 3 * box * es + 1023) / 1024);
-        smem = std::max(smem, sm);
+        (j.single ? single_smem : smem) = std::max(j.single ? single_smem : smem, sm);
     }
+    const int nmain = nwork - nsingle;
     if (any_par) VIE_TRY(par_twiddles_ready());
     VIE_CK(cudaMemcpyAsync(d_groups, hg.data(), hg.size() * sizeof(InnerGroup<C>), cudaMemcpyHostToDevice, s));
-    const bool two = !any_par && split != nullptr && split->nheavy > 0 && split->nheavy < nwork && !inner_cluster_forced();
-    VIE_CK(cudaMemsetAsync(d_next, 0, (two ? 2 : 1) * sizeof(int), s));
+    const bool two = !any_par && nsingle == 0 && split != nullptr && split->nheavy > 0 && split->nheavy < nwork &&
+                     !inner_cluster_forced();
+    VIE_CK(cudaMemsetAsync(d_next, 0, (two || (nsingle > 0 && nmain > 0) ? 2 : 1) * sizeof(int), s));
     // The on-chip shape while the queue is at most three times the 38 clusters of four SMs: a block's own
     // iterations then set the time of the launch more than the rate does.
-    bool chip = any_par && sizeof(C) == 8 && chip_smem <= kParSmemLimit && nwork <= 3 * 38;
+    bool chip = any_par && sizeof(C) == 8 && chip_smem <= kParSmemLimit && nmain <= 3 * 38;
     if (chip) smem = std::max(smem, chip_smem);
     auto kern = k_inner<C, PAR_NONE>;
     int threads = kInnerThreads;
@@ -660,7 +728,6 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
     }
     // one block per cluster of R CTAs; as many clusters as fit at once, pulling blocks from the queue
     auto launch = [&](const int2* work, int n, int* next, int R, cudaStream_t st, int* units) -> int {
-        if (any_par) R = kParRanks;
         // whatever the size: the default 48 KB limit also counts the static shared memory
         VIE_TRY(raise_dynamic_smem(reinterpret_cast<const void*>(kern), smem));
         cudaLaunchAttribute attr[1];
@@ -684,13 +751,20 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
         if (le != cudaSuccess) return cuda_fail(le, "cudaLaunchKernelEx(k_inner)", __FILE__, __LINE__);
         return VIE_OK;
     };
-    const int R = inner_cluster_forced() ? inner_cluster_forced() : (cluster > 0 ? cluster : 2);
+    const int R = any_par ? kParRanks : inner_cluster_forced() ? inner_cluster_forced() : (cluster > 0 ? cluster : 2);
     // the kernels add the KB they move (per MVM) to one profiling counter; the profiled interval
     // covers both parts of a split launch
     int* units = prof_begin(s, PK_INNER, sizeof(C) == 16 ? VIE_C128 : VIE_C64, 1024, 0, true);
     int rc = VIE_OK;
     if (!two) {
-        rc = launch(d_work, nwork, d_next, R, s, units);
+        if (nmain > 0) rc = launch(d_work, nmain, d_next, R, s, units);
+        if (!rc && nsingle > 0) {
+            kern = k_inner<C, PAR_NONE>;
+            threads = kInnerThreads;
+            smem = single_smem;
+            rc = launch(d_work + nmain, nsingle, d_next + (nmain > 0 ? 1 : 0),
+                        inner_cluster_forced() ? inner_cluster_forced() : 1, s, units);
+        }
     } else {
         // the heavy part first, so its clusters are resident before the light part fills the GPU
         cudaError_t e = cudaEventRecord(split->fork, s);
@@ -708,9 +782,9 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
     return VIE_OK;
 }
 
-template int inner_persistent<double2>(const std::vector<InnerJob<double2>>&, const int2*, int, void*, int*, double,
+template int inner_persistent<double2>(const std::vector<InnerJob<double2>>&, const int2*, int, int, void*, int*, double,
                                        int, cudaStream_t, int, const InnerSplit*);
-template int inner_persistent<float2>(const std::vector<InnerJob<float2>>&, const int2*, int, void*, int*, double, int,
+template int inner_persistent<float2>(const std::vector<InnerJob<float2>>&, const int2*, int, int, void*, int*, double, int,
                                       cudaStream_t, int, const InnerSplit*);
 
 // ---------------------------------------------------------------- spectra of the parity-split MVM

@@ -287,8 +287,16 @@ struct ParSpec {
     float2* g64 = nullptr;
 };
 
+// How a grid solves the blocks of a group (choose_block_paths).
+enum BlockPath {
+    PATH_PAR,          // persistent solver, parity-split MVM
+    PATH_PASSES,       // persistent solver, shared-memory passes of one CTA per block
+    PATH_BATCHED       // batched launches
+};
+
 struct Group {
     std::vector<ParClass> par;         // empty: the boxes are too large for the parity-split MVM
+    BlockPath path[2] = {PATH_PAR, PATH_PAR};   // of boxes that the parity-split MVM takes (0: complex128, 1: complex64)
     bool persistent128 = false;        // solved by the persistent block solver
     bool persistent64 = false;
     bool fit[2] = {false, false};      // may join a merged persistent launch (0: complex128, 1: complex64)
@@ -346,10 +354,11 @@ struct vie_grid {
     double* dscal = nullptr;              // device scalars: [0] ||b||^2, [1] ||r||^2
     char* h_ring = nullptr;               // pinned host: active counts, state, scalar
     cudaEvent_t ev[2] = {nullptr, nullptr};
-    // persistent block solver: work lists (job, box), largest boxes first
+    // persistent block solver: work lists (job, box), longest first, those of single-CTA jobs last
     int2* work128 = nullptr;
     int2* work64 = nullptr;
     int nwork128 = 0, nwork64 = 0;
+    int nsingle[2] = {0, 0};              // items of single-CTA jobs, at the end of each list
     // host copies of the work lists and the group of each job, per precision (0: c128, 1: c64);
     // after every apply the list is re-sorted by the blocks' measured cost (longest first)
     std::vector<int2> work_host[2];
@@ -473,8 +482,11 @@ template <class C> struct InnerJob {
     // parity-split MVM (hx > 0): transform lengths, extents and the spectrum (null with Gb)
     int hx = 0, hy = 0, hz = 0, ex = 0, ey = 0, ez = 0;
     const C* Gq = nullptr;
+    bool single = false;            // one CTA per block (PATH_PASSES)
 };
 bool inner_persistent_ok(const BoxSet& bs, size_t es, bool force);
+// Sets path[prec] of every group; batched: whether the batched launches may be chosen.
+void choose_block_paths(std::vector<Group>& groups, int prec, bool batched);
 // Parity-split MVM (inner_parity.cuh): smallest transform length holding b voxels (0: none), whether a
 // box set takes it, and its spectra from the lattice samples K of green_octant.
 int par_len(int b);
@@ -485,9 +497,11 @@ int par_spectra(const BoxSet& bs, const double2* K, const std::vector<ParSpec>& 
 size_t inner_group_desc_bytes();
 // cluster: CTAs per block (1, 2, 4, 8; 0 = 2) of launches without parity-split jobs (those take 4),
 // unless VIE_INNER_CLUSTER forces one.
-// Split launch (split != null, 0 < split->nheavy < nwork, no parity-split jobs): the first nheavy work
-// items run with split->cluster CTAs per block on s while the rest run with `cluster` CTAs per block on
-// split->s2, concurrently; d_next must hold two counters; s waits for both.
+// The last nsingle work items are those of the single-CTA jobs, a launch of its own after the others' (d_next must
+// hold two counters).
+// Split launch (split != null, 0 < split->nheavy < nwork, neither parity-split nor single-CTA jobs): the first
+// nheavy work items run with split->cluster CTAs per block on s while the rest run with `cluster` CTAs per block
+// on split->s2, concurrently; s waits for both.
 struct InnerSplit {
     int nheavy = 0;
     int cluster = 4;
@@ -495,7 +509,7 @@ struct InnerSplit {
     cudaEvent_t fork = nullptr, join = nullptr;
 };
 template <class C>
-int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, int nwork, void* d_groups,
+int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, int nwork, int nsingle, void* d_groups,
                      int* d_next, double tol, int maxit, cudaStream_t s, int cluster = 0,
                      const InnerSplit* split = nullptr);
 int inner_cluster_forced();
