@@ -356,11 +356,10 @@ template <class C2, class T> __device__ __forceinline__ void par_put(C2& z, int 
 
 // Scalars of the iteration, written by warp 0 inside par_sum.
 template <class C> struct ParState {
-    double2 rho, iq, omega;                     // iq = 1 / <rhat, v>
+    double2 rho, iq;                            // iq = 1 / <rhat, v>
     double tol2, bn2, res2;
     int halves;                                 // half steps done
     int status, half, pend;                     // pend: the last full step's x update is pending
-    int check;                                  // the recurrence's ||r||^2 does not decide, r's own is due
     C cbeta, comega, calpha;                    // coefficients of the vector updates
 };
 
@@ -651,43 +650,12 @@ __device__ __noinline__ void par_output_cols(const InnerGroup<C>& g, const ParVe
     for (int i = 0; i < (T ? 4 : 1); ++i) out[i] = acc[i];
 }
 
-// ||r||^2 and <rhat, r> summed over r = s - omega t itself: converged, or the scalars of the next iteration.
-template <int NW, bool CHIP, class C>
-__device__ __forceinline__ void par_residual(const InnerGroup<C>& g, const ParVecs<C, CHIP>& V, ParState<C>& S, ParSums<C>& xs,
-                                             int& slot) {
-    const ParMap map(g);
-    const C oc = S.comega;
-    C q4[4] = {czero<C>(), czero<C>(), czero<C>(), czero<C>()};
-    for (int i = threadIdx.x; i < V.n; i += blockDim.x) {
-        constexpr bool COLS = par_by_column<C>();
-        const int e0 = COLS ? par_col(g, V.n0 + i).e : CHIP ? i : map(V.n0 + i).e;
-        for (int z = 0; z < (COLS ? g.ez : 1); ++z) {
-            const int e = e0 + z * g.by * g.bx;
-            const C r = V.s[e] - cmul(oc, V.t[e]);
-            acc_dot(q4[0], V.rhat[e], r);
-            q4[1].x += r.x * r.x + r.y * r.y;
-        }
-    }
-    par_sum<NW>(q4, xs, slot, [&](const double2* q, int) {
-        const double2 rho = q[0], om = S.omega;
-        S.check = 0;
-        S.res2 = q[1].x;
-        if (!par_finite(S.res2)) S.status = SEG_BREAKDOWN;
-        else if (S.res2 <= S.tol2) S.status = SEG_CONVERGED;
-        else if (!dgood(om) || !dgood(rho)) S.status = SEG_BREAKDOWN;
-        else {
-            const double2 beta = cmul(dcdiv(rho, om), S.iq);
-            S.rho = rho;
-            S.cbeta = cmk<C>(beta.x, beta.y);
-        }
-    });
-}
-
 // One block's BiCGSTAB from x = 0 to ||r|| <= tol ||b|| on a cluster of kParRanks CTAs, in the merged form:
 // r = s - omega t and x += alpha p + omega s are applied in the next p update, and <rhat, r> = <rhat, s> -
 // omega <rhat, t> and ||r||^2 = ||s||^2 - |<t, s>|^2 / ||t||^2 come from the sums of the t pass. That difference
-// carries the rounding of the sums (in complex64 it can be negative where r is 2e-4 of s): a block stops on it when it
-// meets the tolerance by more than that, and where it does not decide, on ||r||^2 summed over r = s - omega t.
+// carries the rounding of the sums (in complex64 it can be negative where r is 2e-4 of s), so a block stops on it only
+// when ||s|| is near enough to the tolerance; where it does not decide, the next half step does, on ||s||^2 itself.
+// (Summing ||r||^2 over r = s - omega t instead, rare as it is, cost 2 to 10 % of every solve in registers.)
 template <bool CHIP, class C>
 __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double tol, int maxit, C* sm, int* units) {
     typedef typename real_of<C>::type R;
@@ -774,7 +742,6 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
         S.res2 = bn2;
         S.half = 0;
         S.pend = 0;
-        S.check = 0;
         S.status = SEG_ACTIVE;
         if (!(bn2 > 0.0) || !isfinite(bn2)) S.status = bn2 == 0.0 ? SEG_CONVERGED : SEG_BREAKDOWN;
         else if (bn2 <= S.tol2) S.status = SEG_CONVERGED;   // x = 0 meets a tolerance of 1 or more
@@ -858,10 +825,7 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             const double rhox = par_lane(v, 0), rhoy = par_lane(v, 1);
             const double res2 = par_lane(v, 4);
             const R coef = (R)(g == 0 ? m : beta);
-            // rounding of res2: at most 24 elements a thread, 5 shuffles and the products, in each of the four sums
-            constexpr double kRound = sizeof(C) == 8 ? 1.0 / (1 << 16) : 1.0 / (1ll << 45);
-            const unsigned le = __ballot_sync(0xffffffffu, (l == 0 ? sn2 : l == 1 ? res2 : l == 3 ? fma(kRound, sn2, res2) : tt) <=
-                                                               (l < 2 || l == 3 ? tol2 : 0.0));
+            const unsigned le = __ballot_sync(0xffffffffu, (l == 0 ? sn2 : l == 1 ? res2 : tt) <= (l < 2 ? tol2 : 0.0));
             if (le & 1u) {
                 S.half = 1;
                 S.res2 = sn2;
@@ -875,7 +839,6 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             }
             if (g == 0) {
                 par_put(S.comega, c, coef);
-                par_put(S.omega, c, m);
                 par_put(S.rho, c, v);
             } else if (g == 1) {
                 par_put(S.cbeta, c, coef);
@@ -884,12 +847,15 @@ __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double 
             S.res2 = res2;
             if (l == 0) S.halves += 2;
             if (!par_finite(res2)) S.status = SEG_BREAKDOWN;
-            else if (le & 8u) S.status = SEG_CONVERGED;
-            else if (le & 2u) S.check = 1;
+            // The sums round by 1.3e-5 of ||s||^2 at most in complex64 (24 elements a thread, 5 shuffles, the products;
+            // 1e-7 as a rule) and 2.5e-14 in complex128: res2 decides while ||s||^2 is below 2^12 (2^36) times the square
+            // of the tolerance. (By the exponents: one FP64 instruction more here cost 1 % of an iteration.)
+            else if ((le & 2u) && (__double2hiint(sn2) < __double2hiint(tol2) + ((sizeof(C) == 8 ? 12 : 36) << 20) ||
+                                   (par_zero(rhox) && par_zero(rhoy))))
+                S.status = SEG_CONVERGED;
             else if ((par_zero(ox) && par_zero(oy)) || !par_finite(rhox) || !par_finite(rhoy) || (par_zero(rhox) && par_zero(rhoy)))
                 S.status = SEG_BREAKDOWN;
         });
-        if (S.check) par_residual<NW>(g, V, S, xs, slot);
     }
     // x of a half step (x += alpha p) or of the last full step (no p update followed it)
     const C ac = S.calpha, oc = S.comega;
