@@ -467,26 +467,25 @@ __device__ __forceinline__ void solve_block(const InnerGroup<C>& g, int b, doubl
     __syncthreads();
 }
 
-enum { PAR_NONE = 0, PAR_L2 = 1, PAR_CHIP = 2 };
 template <int PAR, class C>
 __device__ __forceinline__ void solve_dispatch(const InnerGroup<C>& g, int b, double tol, int maxit, C* sm, const C* tw,
                                                double2* red, int* units) {
     if constexpr (PAR) {
-        if (g.par) {
-            par_solve<PAR == PAR_CHIP>(g, b, tol, maxit, sm, units);
+        if (PAR == PAR_SMALL || g.par) {           // (the small shape takes no other jobs)
+            par_solve<PAR>(g, b, tol, maxit, sm, units);
             return;
         }
     }
-    solve_block<C, SmemMvm<C>>(g, b, tol, maxit, sm, tw, red, units);
+    if constexpr (PAR != PAR_SMALL) solve_block<C, SmemMvm<C>>(g, b, tol, maxit, sm, tw, red, units);
 }
 
 // PAR: the kernel of launches with groups that use the parity-split MVM, in one of its shapes (clusters of
 // kParRanks CTAs); otherwise 256 threads and two CTAs per SM.
 template <class C, int PAR> __host__ __device__ constexpr int inner_threads() {
-    return PAR == PAR_NONE ? kInnerThreads : par_threads<C, PAR == PAR_CHIP>();
+    return PAR == PAR_NONE ? kInnerThreads : par_threads<C, PAR>();
 }
 template <class C, int PAR>
-__global__ void __launch_bounds__((inner_threads<C, PAR>()), (PAR == PAR_NONE ? 2 : par_ctas<C, PAR == PAR_CHIP>()))
+__global__ void __launch_bounds__((inner_threads<C, PAR>()), (PAR == PAR_NONE ? 2 : par_ctas<C, PAR>()))
     k_inner(const InnerGroup<C>* groups, const int2* work, int nwork, int* next, double tol, int maxit, const C* tw,
             int* units) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -658,7 +657,8 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
     VIE_TRY(get_twiddles(&tw));
     std::vector<InnerGroup<C>> hg(jobs.size());
     size_t smem = 0, single_smem = 0;
-    bool any_par = false;
+    bool any_par = false, any_pass = false;         // among the jobs that are not single-CTA ones
+    int par_points = 0;                             // of the largest parity-split box
     size_t chip_smem = 0;
     for (size_t i = 0; i < jobs.size(); ++i) {
         const InnerJob<C>& j = jobs[i];
@@ -687,6 +687,7 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
             make_fastdiv((unsigned)g.ex, g.fd_ex);
             make_fastdiv((unsigned)(g.ex * g.ey), g.fd_exy);
             make_fastdiv((unsigned)g.hy, g.fd_hy);
+            par_points = std::max(par_points, g.hx * g.hy * g.hz);
             sm = (size_t)par_data_elems(g) * sizeof(C) + (sizeof(C) == 8 ? (size_t)par_rank_spec(g) * sizeof(C) : 0);
             chip_smem = std::max(chip_smem, (size_t)(par_data_elems(g) + par_rank_spec(g)) * sizeof(C) +
                                                 (size_t)((3 * g.ez * g.ey * g.ex + kParRanks - 1) / kParRanks) *
@@ -705,6 +706,7 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
                                   : 4 * w2b + 6LL * bs.spec_elems() * es + box * (es + 1) + 4 * 3 * box * es;
         g.kb_mvm = (int)((mvm + 1023) / 1024);
         g.kb_upd = (int)((6 * 3 * box * es + 1023) / 1024);
+        any_pass = any_pass || (!g.par && !j.single);
         (j.single ? single_smem : smem) = std::max(j.single ? single_smem : smem, sm);
     }
     const int nmain = nwork - nsingle;
@@ -713,18 +715,26 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
     const bool two = !any_par && nsingle == 0 && split != nullptr && split->nheavy > 0 && split->nheavy < nwork &&
                      !inner_cluster_forced();
     VIE_CK(cudaMemsetAsync(d_next, 0, (two || (nsingle > 0 && nmain > 0) ? 2 : 1) * sizeof(int), s));
-    // The on-chip shape while the queue is at most three times the 38 clusters of four SMs: a block's own
-    // iterations then set the time of the launch more than the rate does.
-    bool chip = any_par && sizeof(C) == 8 && chip_smem <= kParSmemLimit && nmain <= 3 * 38;
+    // Shape of a launch with parity-split jobs (complex64). On chip while few blocks queue: a block's own iterations
+    // then set the time more than the rate does. How many waves of its 38 clusters may queue depends on the points of
+    // a box (one up to 256, two up to 1024, 2.75 above: 96 blocks of 12 x 12 x 16 1.25 ms on chip, 1.47 in the L2 shape;
+    // 114 blocks 1.51 and 1.44; 48 blocks of 4 x 4 x 4 0.16 and 0.11). Then the small shape up to 1024 points, L2 above.
+    // With boxes over 16 voxels among them three waves on chip, then L2.
+    const double waves = any_pass ? 3.0 : par_points <= 256 ? 1.0 : par_points <= 1024 ? 2.0 : 2.75;
+    const bool chip = any_par && sizeof(C) == 8 && chip_smem <= kParSmemLimit && nmain <= waves * 38;
+    const bool small = any_par && sizeof(C) == 8 && !chip && !any_pass && par_points <= 1024;
     if (chip) smem = std::max(smem, chip_smem);
     auto kern = k_inner<C, PAR_NONE>;
     int threads = kInnerThreads;
     if (chip) {
         if constexpr (sizeof(C) == 8) kern = k_inner<C, PAR_CHIP>;
-        threads = par_threads<C, true>();
+        threads = par_threads<C, PAR_CHIP>();
+    } else if (small) {
+        if constexpr (sizeof(C) == 8) kern = k_inner<C, PAR_SMALL>;
+        threads = par_threads<C, PAR_SMALL>();
     } else if (any_par) {
         kern = k_inner<C, PAR_L2>;
-        threads = par_threads<C, false>();
+        threads = par_threads<C, PAR_L2>();
     }
     // one block per cluster of R CTAs; as many clusters as fit at once, pulling blocks from the queue
     auto launch = [&](const int2* work, int n, int* next, int R, cudaStream_t st, int* units) -> int {

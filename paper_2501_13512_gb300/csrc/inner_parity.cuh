@@ -35,15 +35,20 @@
 namespace vie {
 
 constexpr int kParRanks = 4;
-// Two shapes in complex64. On chip: one CTA of 12 warps per SM, the Krylov vectors and the rank's spectrum in
-// shared memory: the shortest iteration of a block (26.4 us for a 12 x 12 x 16 box, 33 us in the other
-// shape). L2: two CTAs of 6 warps per SM, which hide each other's barriers, vectors in L2: the higher rate
-// when many blocks queue (0.52 us per block iteration of the 256 metasurface pillars against 0.65).
+// Three shapes in complex64. On chip: one CTA of 12 warps per SM, the Krylov vectors and the rank's spectrum in
+// shared memory: the shortest iteration of a block (26.4 us for a 12 x 12 x 16 box, 33 us with the vectors in L2).
+// L2: two CTAs of 6 warps per SM, which hide each other's barriers: the higher rate when many blocks queue (0.52 us
+// per block iteration of the 256 metasurface pillars against 0.65). Small: four CTAs of 4 warps per SM, for boxes
+// that leave most threads of more warps idle (256 blocks of 4 x 4 x 4: 38 us an iteration, 55 in the L2 shape; 256 of
+// 8 x 8 x 16 88 and 124; 256 of 12 x 12 x 16 212 and 180).
 // complex128 (FP64-bound): one CTA of 8 warps of 255 registers. The row stage pairs warps: a multiple of 64.
-template <class C, bool CHIP> __host__ __device__ constexpr int par_threads() {
-    return sizeof(C) == 16 ? 256 : CHIP ? 384 : 192;
+enum { PAR_NONE = 0, PAR_L2 = 1, PAR_CHIP = 2, PAR_SMALL = 3 };
+template <class C, int PAR> __host__ __device__ constexpr int par_threads() {
+    return sizeof(C) == 16 ? 256 : PAR == PAR_CHIP ? 384 : PAR == PAR_SMALL ? 128 : 192;
 }
-template <class C, bool CHIP> __host__ __device__ constexpr int par_ctas() { return sizeof(C) == 16 || CHIP ? 1 : 2; }
+template <class C, int PAR> __host__ __device__ constexpr int par_ctas() {
+    return sizeof(C) == 16 || PAR == PAR_CHIP ? 1 : PAR == PAR_SMALL ? 4 : 2;
+}
 // elements per thread whose loads are issued together (vectors in L2: 1, 2, 3 elements 41, 37, 36 us)
 template <class C, bool CHIP> __host__ __device__ constexpr int par_batch() { return CHIP ? 1 : 3; }
 
@@ -656,13 +661,13 @@ __device__ __noinline__ void par_output_cols(const InnerGroup<C>& g, const ParVe
 // carries the rounding of the sums (in complex64 it can be negative where r is 2e-4 of s), so a block stops on it only
 // when ||s|| is near enough to the tolerance; where it does not decide, the next half step does, on ||s||^2 itself.
 // (Summing ||r||^2 over r = s - omega t instead, rare as it is, cost 2 to 10 % of every solve in registers.)
-template <bool CHIP, class C>
+template <int PAR, class C>
 __device__ __forceinline__ void par_solve(const InnerGroup<C>& g, int b, double tol, int maxit, C* sm, int* units) {
     typedef typename real_of<C>::type R;
-    constexpr bool STG = sizeof(C) == 8, COLS = par_by_column<C>();
-    constexpr int NW = par_threads<C, CHIP>() / 32;
+    constexpr bool STG = sizeof(C) == 8, COLS = par_by_column<C>(), CHIP = PAR == PAR_CHIP;
+    constexpr int NW = par_threads<C, PAR>() / 32;
     // a lone warp would wait in pair_sync for ever; par_sum has a slot for each warp, and four of them add
-    static_assert(par_threads<C, CHIP>() % 64 == 0 && NW >= 4 && NW <= kParWarpsMax, "par_solve: threads per CTA");
+    static_assert(par_threads<C, PAR>() % 64 == 0 && NW >= 4 && NW <= kParWarpsMax, "par_solve: threads per CTA");
     __shared__ ParState<C> S;
     __shared__ ParSums<C> xs;
     __shared__ ParVecs<C, CHIP> V;
