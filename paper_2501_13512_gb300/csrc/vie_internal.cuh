@@ -144,6 +144,12 @@ __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 #endif
 }
+// The exception: a kernel of several waves of CTAs, all its successors' too, may let them fill its last one.
+__device__ __forceinline__ void pdl_trigger() {
+#ifdef __CUDA_ARCH__
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
 // Opt-in of a kernel to dynamic shared memory of up to bytes on the current device. The limit is shared by all
 // threads of the process, which launch the same kernel with different sizes, so it is only ever raised: set to
 // the size of each launch, one thread could lower it between another's call and launch.
