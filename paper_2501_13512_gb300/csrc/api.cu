@@ -257,7 +257,8 @@ static bool is_device_pointer(const void* p) {
 // the bound protects callers from a device that stopped answering). Polls for
 // the first 2 ms, the length of a preconditioner apply or a product on the
 // served grids (a sleep of 20 us costs the timer's slack of 50 us on top, twice
-// or four times per outer iteration), then sleeps between polls.
+// or four times per outer iteration), offering the core to other threads between
+// polls, then sleeps between them.
 static int wait_event(cudaEvent_t ev, double timeout_ms) {
     if (timeout_ms <= 0) timeout_ms = 60000.0;
     auto t0 = std::chrono::steady_clock::now();
@@ -268,6 +269,7 @@ static int wait_event(cudaEvent_t ev, double timeout_ms) {
         double el = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         if (el > timeout_ms) return fail(VIE_ETIMEOUT, "device did not finish within the wait bound");
         if (el > 2.0) std::this_thread::sleep_for(std::chrono::microseconds(20));
+        else std::this_thread::yield();
     }
 }
 
