@@ -46,7 +46,8 @@ struct vie_batch {
     struct Spec {
         double2* g128 = nullptr;          // octant
         float2* g64 = nullptr;            // parity-split layout (boxes up to 16 voxels) or octant
-        float2* full64 = nullptr;         // full layout, boxes over 16 voxels that fit the persistent solver
+        float2* full64 = nullptr;         // full layout, once a merged launch of boxes over 16 voxels reads it
+        int64_t bytes = 0;
     };
     std::map<double, Spec> spectra;       // cached per wavenumber
     std::vector<void*> allocations;
@@ -284,34 +285,41 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
     std::vector<double2*> gb128(nb);
     std::vector<float2*> gb64(nb), gb64full(nb);
     // complex128: octant layout (batched MVMs); complex64: the layout of the parity-split MVM for boxes it
-    // takes, else octant for the batched launches and full for the persistent solver
-    const int64_t so = 6 * bs.oct_elems();
+    // takes, else octant for the batched launches, and full for the persistent solver of merged launches (only those
+    // read it, so it is built on the first of them)
+    const int64_t so = 6 * bs.oct_elems(), sf = 6 * bs.spec_elems();
     const int hx = par_len(bs.bx), hy = par_len(bs.by), hz = par_len(bs.bz);
-    const bool par = b->persistent && par_path_ok(bs);
+    const bool par = b->persistent && par_path_ok(bs), full = b->persistent && !par && mm != nullptr;
     for (int i = 0; i < nb; ++i) {
         auto it = b->spectra.find(k0s[i]);
-        if (it == b->spectra.end()) {
+        if (it == b->spectra.end() || (full && !it->second.full64)) {
             vie_batch::Spec g;
-            const int64_t n64 = par ? par_spectrum_elems(hx, hy, hz) : so;
-            int arc = dmalloc((void**)&g.g128, so * sizeof(double2), "vie_batch_solve");
-            if (!arc) arc = dmalloc((void**)&g.g64, n64 * sizeof(float2), "vie_batch_solve");
-            if (!arc && b->persistent && !par)
-                arc = dmalloc((void**)&g.full64, 6 * bs.spec_elems() * sizeof(float2), "vie_batch_solve");
-            if (!arc) {
-                BoxSet one = bs;
-                one.nb = 1;
-                SpecOut so;
-                std::vector<ParSpec> ps(par ? 1 : 0);
-                so.oct128 = g.g128;
-                so.full64 = g.full64;
+            SpecOut out;
+            std::vector<ParSpec> ps(par ? 1 : 0);
+            int arc = VIE_OK;
+            if (it == b->spectra.end()) {
+                const int64_t n64 = par ? par_spectrum_elems(hx, hy, hz) : so;
+                arc = dmalloc((void**)&g.g128, so * sizeof(double2), "vie_batch_solve");
+                if (!arc) arc = dmalloc((void**)&g.g64, n64 * sizeof(float2), "vie_batch_solve");
+                out.oct128 = g.g128;
                 if (par) {
                     ps[0].hx = hx; ps[0].hy = hy; ps[0].hz = hz;
                     ps[0].g64 = g.g64;
-                    so.par = &ps;
+                    out.par = &ps;
                 } else {
-                    so.oct64 = g.g64;
+                    out.oct64 = g.g64;
                 }
-                arc = spectrum_build(one, k0s[i], b->h, so, s);
+                g.bytes = so * (int64_t)sizeof(double2) + n64 * (int64_t)sizeof(float2);
+            }
+            if (!arc && full) {
+                arc = dmalloc((void**)&g.full64, sf * sizeof(float2), "vie_batch_solve");
+                out.full64 = g.full64;
+                g.bytes += sf * (int64_t)sizeof(float2);
+            }
+            if (!arc) {
+                BoxSet one = bs;
+                one.nb = 1;
+                arc = spectrum_build(one, k0s[i], b->h, out, s);
                 if (arc) cudaStreamSynchronize(s);
             }
             if (arc) {
@@ -320,7 +328,12 @@ static int batch_solve_impl(vie_batch* b, const double* k0s, const void* einc_de
                 dfree(g.full64);
                 return arc;
             }
-            it = b->spectra.emplace(k0s[i], g).first;
+            if (it == b->spectra.end()) {
+                it = b->spectra.emplace(k0s[i], g).first;
+            } else {
+                it->second.full64 = g.full64;
+                it->second.bytes += g.bytes;
+            }
         }
         gb128[i] = it->second.g128;
         gb64[i] = it->second.g64;
@@ -571,7 +584,7 @@ extern "C" int vie_batch_get_info(const vie_batch* b, int64_t* device_bytes, int
     if (!b) return fail(VIE_EINVAL, "vie_batch_get_info: null batch");
     if (device_bytes) {
         int64_t sp = 0;
-        for (auto& kv : b->spectra) sp += 6 * b->bs.spec_elems() * (16 + 8);
+        for (auto& kv : b->spectra) sp += kv.second.bytes;
         *device_bytes = b->device_bytes + sp;
     }
     if (persistent) *persistent = b->persistent ? 1 : 0;
