@@ -9,8 +9,7 @@ w = chi E in the continuum), Eq. 4 with Eq. 1 reads
 
 the three pieces of L^c_ii (contrast term and vector potential, Eq. 8) and L^q_ij (scalar potential,
 Eq. 9, read as acting on w_j), with the sign of Eq. 4 (E_tot = E_inc + E_s, Eq. 3). Discretisation
-on the uniform grid of cells of edge h (the readings the paper leaves open are listed here and in
-DESIGN.md):
+on the uniform grid of cells of edge h (with the readings the paper leaves open):
 
 * Basis (Eq. 5): component a of w is expanded in rooftops T_(a,c): the hat of half-width h along
   axis a centred on the face between cell c and cell c + e_a, times the pulse of the cell section

@@ -934,12 +934,12 @@ static int launch_rows(RowArgs<C> a, Prof pf, cudaStream_t s) {
     // complex128 rows of 256 and 512 points, given two waves of CTAs (below that the radix-4 form spreads a row
     // over more threads: 28 against 42 us for 540 rows); complex64 rows are faster in the radix-2 form above
     // (32 and 50 us forward and inverse against 37 and 62 at 256x256x16)
-    if (sizeof(C) == 16 && (a.lL == 8 || a.lL == 9) && a.nrows * (1 << a.lL) >= 2 * 152 * 4096) {
+    if constexpr (sizeof(C) == 16) {
         const int L = 1 << a.lL;
-        if (MODE == ROW_FWD_CHI && 2 * a.n_in <= L && a.n_out == L)
-            VIE_LONG_LINE_SWITCH(a.lL, return (launch_line_rows<C, AA, BB, true>(a, pf, s)));
-        if (MODE == ROW_INV_UPDATE && 2 * a.n_out <= L && a.n_in == L)
-            VIE_LONG_LINE_SWITCH(a.lL, return (launch_line_rows<C, AA, BB, false>(a, pf, s)));
+        constexpr bool FWD = MODE == ROW_FWD_CHI;
+        if ((a.lL == 8 || a.lL == 9) && a.nrows * L >= 2 * 152 * 4096 &&
+            (FWD ? 2 * a.n_in <= L && a.n_out == L : MODE == ROW_INV_UPDATE && 2 * a.n_out <= L && a.n_in == L))
+            return a.lL == 8 ? launch_line_rows<C, 16, 16, FWD>(a, pf, s) : launch_line_rows<C, 32, 16, FWD>(a, pf, s);
     }
     a.ltr = pick_ltile(a.lL, sizeof(C), 1, 1);
     const int TR = 1 << a.ltr;

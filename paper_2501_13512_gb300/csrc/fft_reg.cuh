@@ -80,12 +80,6 @@ __device__ __forceinline__ F twc(F v, int m) {
     return FWD ? cmul(v, w) : cmulc(v, w);
 }
 
-template <> struct TwSel<double2> {
-    template <bool FWD>
-    static __device__ __forceinline__ double2 apply(double2 v, int m, const double2* __restrict__ tw) {
-        return twmul<FWD>(v, m, tw);
-    }
-};
 template <> struct TwSel<float2> {
     template <bool FWD>
     static __device__ __forceinline__ float2 apply(float2 v, int m, const float2* __restrict__) {

@@ -35,7 +35,6 @@ namespace vie {
 
 template <class C> struct InnerGroup {
     C *b, *x, *r, *rhat, *p, *v, *s, *t;   // [nb][3][bz][by][bx]
-    C* w1;                                  // [nb][3][bz][by][Mx] (register path)
     C* w2;                                  // [nb][3][bz][My][Mx]
     const C* chi;                           // [nb][bz][by][bx]
     const uint8_t* mask;                    // [nb][bz][by][bx]
@@ -47,14 +46,14 @@ template <class C> struct InnerGroup {
     int lpt;                                // log2 planes per XY tile
     int ltc;                                // log2 columns per Z tile
     int kb_mvm;                             // profiling: KB moved by one MVM and its fused updates
-    int kb_upd;                             // profiling: KB moved by the x/r update pass
+    int kb_upd;                             // profiling: KB moved by the x/r update pass (shared-memory passes)
     // parity-split MVM (inner_parity.cuh)
     int par;                                // 1: the block uses it
     int ex, ey, ez;                         // the blocks' own extents within the box
     int hx, hy, hz;                         // transform lengths per axis (>= extent)
     int yp;                                 // row pitch in shared memory (ex made odd: no bank conflicts)
     unsigned fd_ex[3], fd_exy[3], fd_hy[3]; // FastDiv constants for ex, ex*ey and hy
-    const C* Gq;                            // spectrum [4][hx+1][6][hz/2+1][hy/2+1] (par_spectrum)
+    const C* Gq;                            // spectrum [4][hx+1][6][hz/2+1][hy/2+1] (par_spectra)
 };
 
 constexpr int kInnerThreads = 256;
@@ -299,28 +298,6 @@ __device__ __forceinline__ FastDiv fd_of(const unsigned (&v)[3]) { return FastDi
 
 namespace vie {
 
-// MVM through shared-memory passes and the block scratch in global memory, for boxes of any size whose
-// padded (x, y) plane fits (ParMvm of inner_parity.cuh is the other implementation solve_block uses).
-template <class C> struct SmemMvm {
-    template <int IN>
-    static __device__ C fwd(const InnerGroup<C>& g, int64_t voff, C* W1, C* W2, const C* chi, C* sm, const C* tw,
-                            C c1, C c2) {
-        C r = phase_xy<C, IN>(g, voff, W2, chi, sm, tw, c1, c2);
-        team_sync();
-        return r;                                 // this thread's part of ||s||^2 (IN_S)
-    }
-    static __device__ void mid(const InnerGroup<C>& g, C* W2, C* sm, const C* tw) {
-        phase_z<C>(g, W2, sm, tw);
-        team_sync();
-    }
-    // this thread's partials of the iteration's inner products
-    template <int OUT>
-    static __device__ void inv(const InnerGroup<C>& g, int64_t voff, C* W1, C* W2, const uint8_t* mask, C* sm,
-                               const C* tw, C& a1, C& a2) {
-        phase_xy_inv<C, OUT>(g, voff, W2, mask, sm, tw, a1, a2);
-    }
-};
-
 // BiCGSTAB state of the block being solved, in shared memory: written by thread 0
 // inside team_sum (the FP64 scalar work of an iteration runs in that one thread)
 // and read by every thread after the sum's closing barrier.
@@ -342,14 +319,15 @@ template <class C> __device__ __forceinline__ void next_beta(BiState<C>& S) {
     S.comega = cmk<C>(S.omega.x, S.omega.y);
 }
 
-template <class C, class Mvm>
+// One block's BiCGSTAB with the MVM through the shared-memory passes above and the block scratch in global memory, for
+// boxes of any size whose padded (x, y) plane fits (par_solve of inner_parity.cuh takes the others).
+template <class C>
 __device__ __forceinline__ void solve_block(const InnerGroup<C>& g, int b, double tol, int maxit, C* sm, const C* tw,
                             double2* red, int* units) {
     const int64_t box = (int64_t)g.bx * g.by * g.bz;
     const int64_t voff = (int64_t)b * 3 * box;
     const int n = 3 * (int)box;                 // elements of the block's vectors, at voff
     C* W = g.w2 + (int64_t)b * 3 * g.bz * g.My * g.Mx;
-    C* W1 = g.w1 + (int64_t)b * 3 * g.bz * g.by * g.Mx;
     const C* chi = g.chi + (int64_t)b * box;
     const uint8_t* mask = g.mask + (int64_t)b * box;
     __shared__ BiState<C> S;
@@ -384,11 +362,13 @@ __device__ __forceinline__ void solve_block(const InnerGroup<C>& g, int b, doubl
     });
     for (int it = 0; it < maxit && S.status == SEG_ACTIVE; ++it) {
         // v = A p, p = r + beta (p - omega v)
-        Mvm::template fwd<IN_P>(g, voff, W1, W, chi, sm, tw, S.cbeta, S.comega);
-        Mvm::mid(g, W, sm, tw);
+        phase_xy<C, IN_P>(g, voff, W, chi, sm, tw, S.cbeta, S.comega);
+        team_sync();
+        phase_z<C>(g, W, sm, tw);
+        team_sync();
         if (units != nullptr && rk == 0 && threadIdx.x == 0) atomicAdd(units, g.kb_mvm);
         C p1 = czero<C>(), p2 = czero<C>();
-        Mvm::template inv<OUT_V>(g, voff, W1, W, mask, sm, tw, p1, p2);
+        phase_xy_inv<C, OUT_V>(g, voff, W, mask, sm, tw, p1, p2);
         team_sum(p1, p2, red, [&](double2 sigma, double2) {
             if (!dgood(sigma)) {
                 S.status = SEG_BREAKDOWN;
@@ -400,12 +380,14 @@ __device__ __forceinline__ void solve_block(const InnerGroup<C>& g, int b, doubl
         if (S.status != SEG_ACTIVE) break;
         // s = r - alpha v and t = A s; ||s||^2 is summed together with <t,s> and <t,t>, so the
         // half-step test (same value, same decision) costs no reduction of its own
-        const C snp = Mvm::template fwd<IN_S>(g, voff, W1, W, chi, sm, tw, S.calpha, czero<C>());
-        Mvm::mid(g, W, sm, tw);
+        const C snp = phase_xy<C, IN_S>(g, voff, W, chi, sm, tw, S.calpha, czero<C>());
+        team_sync();
+        phase_z<C>(g, W, sm, tw);
+        team_sync();
         if (units != nullptr && rk == 0 && threadIdx.x == 0) atomicAdd(units, g.kb_mvm + g.kb_upd);
         p1 = czero<C>();
         p2 = czero<C>();
-        Mvm::template inv<OUT_T>(g, voff, W1, W, mask, sm, tw, p1, p2);
+        phase_xy_inv<C, OUT_T>(g, voff, W, mask, sm, tw, p1, p2);
         p2.y = snp.x;                           // the deferred ||s||^2 rides in the unused slot
         team_sum(p1, p2, red, [&](double2 ts, double2 tt) {
             const double sn2 = tt.y;
@@ -476,7 +458,7 @@ __device__ __forceinline__ void solve_dispatch(const InnerGroup<C>& g, int b, do
             return;
         }
     }
-    if constexpr (PAR != PAR_SMALL) solve_block<C, SmemMvm<C>>(g, b, tol, maxit, sm, tw, red, units);
+    if constexpr (PAR != PAR_SMALL) solve_block<C>(g, b, tol, maxit, sm, tw, red, units);
 }
 
 // PAR: the kernel of launches with groups that use the parity-split MVM, in one of its shapes (clusters of
@@ -665,7 +647,6 @@ int inner_persistent(const std::vector<InnerJob<C>>& jobs, const int2* d_work, i
         const BoxSet& bs = *j.bs;
         InnerGroup<C>& g = hg[i];
         g.b = j.v.b; g.x = j.v.x; g.r = j.v.r; g.rhat = j.v.rhat; g.p = j.v.p; g.v = j.v.v; g.s = j.v.s; g.t = j.v.t;
-        g.w1 = reinterpret_cast<C*>(bs.w1);
         g.w2 = reinterpret_cast<C*>(bs.w2);
         g.chi = j.chi;
         g.mask = bs.mask;

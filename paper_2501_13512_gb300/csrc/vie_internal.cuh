@@ -58,7 +58,7 @@ __host__ __device__ __forceinline__ double radd(double a, double b) {
 
 // Complex64 sums as one packed instruction on the register pair (add / sub / fma.rn.f32x2: two FP32 results of
 // the same rounding). The units take no more of them a clock than of plain ones, but half the instructions
-// leave the issue slots and the instruction cache to the rest: 256 pillar blocks to 1e-6 17.1 -> 15.6 ms,
+// leave the issue slots and the instruction cache to the rest: 256 pillar blocks to 1e-6 17.1 -> 15.3 ms,
 // 256x256x16 product 224 -> 205 us.
 __device__ __forceinline__ unsigned long long f2_bits(float2 a) {
     unsigned long long r;
@@ -286,7 +286,7 @@ struct ParClass {
     int ex = 0, ey = 0, ez = 0;        // largest extents of its blocks
     std::vector<int> boxes;            // indices within the group
 };
-// Spectrum of one set of transform lengths (par_spectrum).
+// Spectrum of one set of transform lengths (par_spectra).
 struct ParSpec {
     int hx = 0, hy = 0, hz = 0;
     double2* g128 = nullptr;
