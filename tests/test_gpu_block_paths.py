@@ -94,3 +94,22 @@ def test_spectrum_serves_a_grid_of_another_path(precision):
     ga, gb = vie.Grid(eps_r, H, few), vie.Grid(eps_r, H, bid)
     check(gb, ga.spectrum(K0), eps_r, bid, b, precision)
     check(ga, gb.spectrum(K0), eps_r, few, b, precision)
+
+
+@pytest.mark.parametrize("mode", [vie.MODE_MIXED, vie.MODE_PLAIN_C128])
+def test_merged_solves_with_every_kind_of_block(mode):
+    # two grids in one session, their very small blocks in one launch and the others in another; the solutions are those
+    # of the grids alone (both within 1e-8 of the right-hand side in residual, ||A^-1|| <= 10 for |chi| <= 0.7)
+    problems, alone = [], []
+    for seed in (21, 22):
+        eps_r, bid, b = lattice([(2, 2, 2)] * 170 + [(6, 7, 5)] * (2 + seed % 2) + [(9, 9, 10)], 20, seed=seed)
+        b = torch.from_numpy(b).cuda()
+        grids = [vie.Grid(eps_r, H, bid) for _ in range(2)]
+        specs = [g.spectrum(K0) for g in grids]
+        alone.append(grids[0].solve(specs[0], b, outer_tol=1e-8, mode=mode))
+        problems.append({"grid": grids[1], "spec": specs[1], "einc": b, "outer_tol": 1e-8, "mode": mode})
+    res, ms = vie.solve_many(problems)
+    assert ms["launches"] >= 1 and ms["max_solves"] == 2
+    for (e, st), (e1, st1) in zip(res, alone):
+        assert st["status"] == vie.VIE_OK and st1["status"] == vie.VIE_OK
+        assert float((e - e1).norm() / e1.norm()) <= 2e-7
